@@ -44,8 +44,8 @@ constexpr int kBatchMaxThreads = 512;
 
 // Block-wide sum of NV values, then cluster-wide through DSMEM; every thread
 // of every CTA returns the same totals.
-template <int NV>
-__device__ __forceinline__ void team_sum(double (&v)[NV], double (&tot)[NV], cg::cluster_group& cl,
+template <int NV, typename V>
+__device__ __forceinline__ void team_sum(const V (&v)[NV], double (&tot)[NV], cg::cluster_group& cl,
                                          double (*spart)[kMaxPartials], double (*swarp)[32], int& parity) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
 #pragma unroll
@@ -64,9 +64,9 @@ __device__ __forceinline__ void team_sum(double (&v)[NV], double (&tot)[NV], cg:
   }
   cl.sync();
   // lane r reads CTA r's partials (all T remote loads in flight at once), then
-  // an xor butterfly over the warp: every step adds the same two operands in
-  // both lanes of a pair (addition commutes exactly), so every thread of every
-  // CTA ends with the same bits
+  // the warp's integer sum (rp_reduce.cuh): the same bits in every thread of
+  // every CTA. All sums stay off the FP64 pipe: as xor trees of FP64 adds the
+  // three sums of an iteration took 10 us of a team's SMs
   const unsigned T = cl.num_blocks();
 #pragma unroll
   for (int i = 0; i < NV; ++i)
@@ -629,7 +629,8 @@ __global__ void __launch_bounds__(kBatchMaxThreads, 2) k_batch(BatchArgs a) {
           };
           if (sl) spmv_slices<float, U4>(a, a.sl_vals32, s0, p, p, i0, i1, n, stage, qrow);
           else spmv_rows<float>(rp, col, vals32, p, p, i0, i1, n, qrow);
-          double v1[1] = {(double)acc}, t1[1];
+          const float v1[1] = {acc};
+          double t1[1];
           team_sum<1>(v1, t1, cl, spart, swarp, parity);
           if (!(t1[0] > 0.0) || !isfinite(t1[0])) { status = RP_BREAKDOWN; broke = true; break; }
           const float alpha = (float)(rz / t1[0]);
@@ -661,9 +662,16 @@ __global__ void __launch_bounds__(kBatchMaxThreads, 2) k_batch(BatchArgs a) {
                 rstep(rv.w, qv.w, dv.w);
                 reinterpret_cast<float4*>(a.r32)[v] = rv;
               });
-          if (SCALED) a0 = a1;  // z = r: (r, z) = (r, r)
-          double v2[2] = {(double)a0, (double)a1}, t2[2];
-          team_sum<2>(v2, t2, cl, spart, swarp, parity);
+          double t2[2];
+          if constexpr (SCALED) {  // z = r: (r, z) = (r, r)
+            const float v2[1] = {a1};
+            double t[1];
+            team_sum<1>(v2, t, cl, spart, swarp, parity);
+            t2[0] = t2[1] = t[0];
+          } else {
+            const float v2[2] = {a0, a1};
+            team_sum<2>(v2, t2, cl, spart, swarp, parity);
+          }
           ++it;
           ++iters;
           bool stop = false;

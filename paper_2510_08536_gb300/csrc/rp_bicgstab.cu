@@ -295,7 +295,8 @@ struct BsEpiV {
     c->stop = 1;
   }
   __device__ __forceinline__ void finish() {
-    double v[1] = {(double)acc}, tot[1];
+    const T v[1] = {acc};
+    double tot[1];
     if (reduce_last_block<1>(v, partials, &c->ticket, tot) && threadIdx.x == 0) {
       if (c->status == RP_DEVICE_TIMEOUT) {
         c->stop = 1;
@@ -325,7 +326,8 @@ struct BsEpiT {
     c->stop = 1;
   }
   __device__ __forceinline__ void finish() {
-    double v[2] = {(double)ts, (double)tt}, tot[2];
+    const T v[2] = {ts, tt};
+    double tot[2];
     if (reduce_last_block<2>(v, partials, &c->ticket, tot) && threadIdx.x == 0) {
       const double omega = tot[0] / tot[1];
       if (c->status == RP_DEVICE_TIMEOUT) {
@@ -418,7 +420,8 @@ __global__ void __launch_bounds__(kThreads) k_bs_s(BsArgs a) {
     V.shat[i] = V.dinv[i] * si;
     ss = fma(si, si, ss);
   }
-  double v[1] = {(double)ss}, tot[1];
+  const T v[1] = {ss};
+  double tot[1];
   if (reduce_last_block<1>(v, a.partials, &c->ticket, tot) && threadIdx.x == 0) {
     c->ss = tot[0];
     c->half = tot[0] <= c->ithresh ? 1 : 0;
@@ -511,7 +514,8 @@ __global__ void __launch_bounds__(kThreads) k_bs_xr(BsArgs a) {
       rhr = fma(V.rhat[i], ri, rhr);
     }
   }
-  double v[2] = {(double)rr, (double)rhr}, tot[2];
+  const T v[2] = {rr, rhr};
+  double tot[2];
   if (reduce_last_block<2>(v, a.partials, &c->ticket, tot) && threadIdx.x == 0) {
     c->iter += 1;
     if (half) {

@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "../../include/repart.h"
+#include "rp_reduce.cuh"
 
 namespace rp {
 
@@ -434,55 +435,60 @@ void free_batch(rp_handle* h);
 
 namespace rp {
 
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
 // Block-wide partial sums of NV values, written to partials[blockIdx.x*NV+i];
 // returns true in every thread of the one block that arrives last, with the
-// grid totals in tot[] (summed in block order: deterministic for a fixed
-// grid). The ticket is reset by that block.
-template <int NV>
-__device__ __forceinline__ bool reduce_last_block(double (&v)[NV], double* partials,
-                                                  unsigned int* ticket, double (&tot)[NV]) {
+// grid totals in tot[] of its first warp (the block partials are summed in an
+// order fixed by the grid: deterministic). The ticket is reset by that block.
+// The sums run on the integer pipe (rp_reduce.cuh): with FP64 trees the
+// iteration's residual kernel ended in 6 us of FP64 adds, whatever its size.
+template <int NV, typename T>
+__device__ __forceinline__ bool reduce_last_block(const T (&v)[NV], double* partials, unsigned int* ticket,
+                                                  double (&tot)[NV]) {
   __shared__ double sm[NV][32];
   __shared__ int last;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
 #pragma unroll
   for (int i = 0; i < NV; ++i) {
-    double s = warp_sum(v[i]);
+    const double s = warp_sum(v[i]);
     if (lane == 0) sm[i][wid] = s;
   }
   __syncthreads();
   if (wid == 0) {
 #pragma unroll
     for (int i = 0; i < NV; ++i) {
-      double s = lane < nw ? sm[i][lane] : 0.0;
-      s = warp_sum(s);
-      if (lane == 0) partials[(size_t)blockIdx.x * NV + i] = s;
+      const double s = warp_sum(lane < nw ? sm[i][lane] : 0.0);
+      if (lane == 0) __stcg(partials + (size_t)blockIdx.x * NV + i, s);
     }
-  }
-  if (threadIdx.x == 0) {
-    __threadfence();
-    unsigned int t = atomicAdd(ticket, 1u);
-    last = (t == gridDim.x - 1);
+    if (lane == 0) {
+      __threadfence();
+      last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    }
   }
   __syncthreads();
   if (!last) return false;
   __threadfence();
+  // up to kPer partials a thread in flight at once; grids have at most
+  // kBlocksPerSm blocks an SM, so more than one trip is not expected
+  constexpr int kPer = 5;
 #pragma unroll
   for (int i = 0; i < NV; ++i) {
     double s = 0.0;
-    for (unsigned int b = threadIdx.x; b < gridDim.x; b += blockDim.x)
-      s += __ldcg(partials + (size_t)b * NV + i);
-    s = warp_sum(s);
-    __syncthreads();
+    for (unsigned int b0 = 0; b0 < gridDim.x; b0 += kPer * blockDim.x) {
+      double x[kPer];
+#pragma unroll
+      for (int j = 0; j < kPer; ++j) {
+        const unsigned int b = b0 + j * blockDim.x + threadIdx.x;
+        x[j] = b < gridDim.x ? __ldcg(partials + (size_t)b * NV + i) : 0.0;
+      }
+      const double t = warp_sum_n(x);
+      s = b0 ? s + t : t;
+    }
     if (lane == 0) sm[i][wid] = s;
-    __syncthreads();
-    double t = lane < nw ? sm[i][lane] : 0.0;
-    tot[i] = warp_sum(t);  // every warp computes the same total
+  }
+  __syncthreads();
+  if (wid == 0) {
+#pragma unroll
+    for (int i = 0; i < NV; ++i) tot[i] = warp_sum(lane < nw ? sm[i][lane] : 0.0);
   }
   if (threadIdx.x == 0) *ticket = 0u;
   return true;

@@ -137,7 +137,8 @@ __global__ void __launch_bounds__(kThreads)
 // than FP32); one conversion per thread feeds the FP64 block reduction.
 template <typename T>
 __device__ __forceinline__ void pcg_k1_finish(Ctl* c, double* partials, T acc) {
-  double v[1] = {(double)acc}, tot[1];
+  const T v[1] = {acc};
+  double tot[1];
   if (reduce_last_block<1>(v, partials, &c->ticket, tot) && threadIdx.x == 0) {
     const double pq = tot[0];
     c->pq = pq;
@@ -481,7 +482,6 @@ __global__ void __launch_bounds__(kThreads) k_it_resid(IterArgs<T> a) {
       a.r[i] = ri;
       rr = fma(ri, ri, rr);
     }
-    rz = rr;
   }
   if constexpr (!LINE && !SCALED) {
     // two vectors of each stream in flight per thread
@@ -508,8 +508,14 @@ __global__ void __launch_bounds__(kThreads) k_it_resid(IterArgs<T> a) {
       rr = fma(ri, ri, rr);
     }
   }
-  double v[2] = {(double)rz, (double)rr}, tot[2];
-  if (reduce_last_block<2>(v, a.partials, &c->ticket, tot) && threadIdx.x == 0) {
+  // SCALED: (r, z) = (r, r), one sum
+  constexpr int NV = SCALED ? 1 : 2;
+  T v[NV];
+  v[NV - 1] = rr;
+  if constexpr (!SCALED) v[0] = rz;
+  double sums[NV];
+  if (reduce_last_block<NV>(v, a.partials, &c->ticket, sums) && threadIdx.x == 0) {
+    const double tot[2] = {sums[0], sums[NV - 1]};
     c->iter += 1;
     c->iter_total += 1;
     c->rr = tot[1];

@@ -1,0 +1,128 @@
+// Sums across a warp, a block and a grid without the FP64 pipe.
+//
+// GB300 adds two FP64 lanes a clock and SM: one warp-wide FP64 add keeps a
+// quarter of an SM's FP64 pipe busy for 64 clocks (76 with all four quarters
+// adding), however many lanes are active. The usual xor tree of FP64 adds
+// (five a warp and value) therefore costs 380 clocks of that pipe a warp, and
+// with 64 resident warps an SM and two values it was the largest fixed cost of
+// every kernel that ends in a dot product: 6 us a launch.
+//
+// A warp's values are instead summed as integers: the largest exponent of the
+// warp (redux.sync) fixes a common unit, every value becomes a 64-bit integer
+// multiple of it (rounded to nearest), and the integers are added exactly, as
+// three limbs of 26, 26 and 12 bits by redux.sync. The unit lies 2^-62 (FP64)
+// or 2^-61 (FP32) below the largest exponent, so the sum of 32 values is within
+// 32 half units of the true sum before its one rounding to FP64 -- an error
+// bound of 2^-57 of the largest value, where the tree rounds five times at
+// 2^-53. The integer sum does not depend on the order of the lanes.
+// Infinities and NaN fall back to the FP64 tree.
+#pragma once
+
+#include <cstdint>
+
+#include <cuda_runtime.h>
+
+namespace rp {
+
+// the tree of FP64 adds (fallback for infinities and NaN)
+__device__ __forceinline__ double warp_sum_tree(double v) {
+#pragma unroll 1
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// Biased exponent (0: zero or subnormal, all ones: infinity or NaN), and the
+// value as a signed integer multiple of 2^(exponent of emax) 2^-S (emax at
+// least the value's own exponent and 1).
+template <typename T>
+struct FixOf;
+template <>
+struct FixOf<double> {
+  static constexpr int kMant = 52, kBias = 1023, kSpecial = 2047;
+  static __device__ __forceinline__ int expo(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
+  static __device__ __forceinline__ uint64_t mant(double v, int e) {
+    const uint32_t hi = ((uint32_t)__double2hiint(v) & 0xfffffu) | (e ? 0x100000u : 0u);
+    return (uint64_t)hi << 32 | (uint32_t)__double2loint(v);
+  }
+  static __device__ __forceinline__ bool neg(double v) { return __double2hiint(v) < 0; }
+};
+template <>
+struct FixOf<float> {
+  static constexpr int kMant = 23, kBias = 127, kSpecial = 255;
+  static __device__ __forceinline__ int expo(float v) { return (__float_as_int(v) >> 23) & 0xff; }
+  static __device__ __forceinline__ uint64_t mant(float v, int e) {
+    return ((uint32_t)__float_as_int(v) & 0x7fffffu) | (e ? 0x800000u : 0u);
+  }
+  static __device__ __forceinline__ bool neg(float v) { return __float_as_int(v) < 0; }
+};
+
+template <typename T, int S>
+__device__ __forceinline__ long long fix_term(T v, int emax) {
+  using F = FixOf<T>;
+  const int e = F::expo(v);
+  uint64_t m = F::mant(v, e) << S;
+  const int d = emax - (e > 1 ? e : 1);
+  if (d > 0) m = d < 64 ? (m + (1ull << (d - 1))) >> d : 0ull;
+  return F::neg(v) ? -(long long)m : (long long)m;
+}
+
+// h 2^26 + l (0 <= l < 2^26, |h| < 2^44) times 2^q, rounded to nearest even
+__device__ __forceinline__ double fix_value(long long h, uint32_t l, int q) {
+  long long t;
+  if (h < (1ll << 36) && h >= -(1ll << 36)) {
+    t = (long long)((uint64_t)h << 26 | l);
+  } else {  // eight bits lower, the dropped ones kept as a sticky bit
+    t = (long long)((uint64_t)h << 18 | (l >> 8) | ((l & 255u) ? 1u : 0u));
+    q += 8;
+  }
+  if (t == 0) return 0.0;
+  const bool neg = t < 0;
+  uint64_t m = neg ? 0ull - (uint64_t)t : (uint64_t)t;
+  const int lz = __clzll((long long)m);
+  const int e = q + 63 - lz + 1023;  // biased exponent of the leading bit
+  if (e < 1 || e > 2046) {           // subnormal or overflowing: rounded by the library
+    const double r = ldexp((double)m, q);
+    return neg ? -r : r;
+  }
+  m <<= lz;
+  uint64_t r = m >> 11;
+  const uint32_t rem = (uint32_t)m & 0x7ffu;
+  r += (rem > 0x400u || (rem == 0x400u && (r & 1u))) ? 1u : 0u;
+  r += (uint64_t)(e - 1) << 52;  // the leading bit carries into the exponent
+  return __longlong_as_double((long long)(r | (neg ? 1ull << 63 : 0ull)));
+}
+
+// Sum of N values of every lane of a warp; all lanes call it and get the sum.
+template <typename T, int N>
+__device__ __forceinline__ double warp_sum_n(const T (&v)[N]) {
+  using F = FixOf<T>;
+  static_assert(N >= 1 && N <= 8, "at most 8 values a lane");
+  constexpr int kLane = N > 4 ? 3 : N > 2 ? 2 : N > 1 ? 1 : 0;  // headroom of the lane's own sum
+  constexpr int S = 62 - F::kMant - kLane;                      // |term| < 2^(63 - kLane)
+  int em = 1;
+#pragma unroll
+  for (int i = 0; i < N; ++i) em = max(em, F::expo(v[i]));
+  const int emax = (int)__reduce_max_sync(0xffffffffu, (unsigned)em);
+  if (emax == F::kSpecial) {
+    double s = (double)v[0];
+#pragma unroll
+    for (int i = 1; i < N; ++i) s += (double)v[i];
+    return warp_sum_tree(s);
+  }
+  long long m = 0;
+#pragma unroll
+  for (int i = 0; i < N; ++i) m += fix_term<T, S>(v[i], emax);
+  const uint32_t r0 = __reduce_add_sync(0xffffffffu, (uint32_t)m & 0x3ffffffu);
+  const uint32_t r1 = __reduce_add_sync(0xffffffffu, (uint32_t)(m >> 26) & 0x3ffffffu);
+  const int32_t r2 = __reduce_add_sync(0xffffffffu, (int32_t)(m >> 52));
+  const long long h = (long long)r2 * (1ll << 26) + (long long)r1 + (long long)(r0 >> 26);
+  return fix_value(h, r0 & 0x3ffffffu, emax - F::kBias - F::kMant - S);
+}
+
+template <typename T>
+__device__ __forceinline__ double warp_sum(T v) {
+  const T a[1] = {v};
+  return warp_sum_n<T, 1>(a);
+}
+
+}  // namespace rp
