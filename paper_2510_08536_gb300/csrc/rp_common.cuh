@@ -167,6 +167,7 @@ struct Parts {
   const int32_t* nl_col;     // compressed column of each non-local entry
   const int32_t* nl_cols;    // global row behind each compressed column
   const T* nl_vals;
+  const int32_t* nl_gcol;    // global row behind each non-local entry (nl_cols[nl_col]: one gather less)
 };
 
 // Sliced layout of the merged matrix (one part): rows in slices of 32, one
@@ -310,6 +311,7 @@ struct rp_handle {
   int32_t* nl_col_idx = nullptr;
   int32_t* nl_src_of = nullptr;
   int32_t* nl_cols = nullptr;
+  int32_t* nl_gcol = nullptr;     // nl_cols[nl_col_idx], global rows (n_parts > 1)
   // rank tables on the device (k + 1 entries)
   int64_t* d_row_off = nullptr;
   int64_t* d_slot_off = nullptr;
@@ -374,6 +376,7 @@ struct rp_handle {
   rp::Ctl* ctl_spmv = nullptr;     // device, rp_iter_spmv's own
   rp::SolveIO* io = nullptr;       // device
   unsigned int* ticket = nullptr;  // spare ticket for rp_spmv
+  unsigned int* rsync = nullptr;   // grid barrier of the resident iteration
   int grid = 0;                    // blocks of every streaming kernel
   rp::IterGrid igrid64, igrid32;   // blocks of the PCG iteration kernels
   rp::Graphs graphs;

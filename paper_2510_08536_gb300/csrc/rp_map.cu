@@ -326,6 +326,18 @@ __global__ void k_renumber(int64_t r0, int64_t r1, const int32_t* __restrict__ p
     out[q] = idx[gcol[q]];
 }
 
+// the global row behind every non-local entry (part p's entries at nl_off[p],
+// its compressed columns at nlcol_off[p])
+__global__ void k_nl_gcol(int64_t nl_nnz, int n_parts, const int64_t* __restrict__ nl_off,
+                          const int64_t* __restrict__ nlcol_off, const int32_t* __restrict__ nl_col,
+                          const int32_t* __restrict__ nl_cols, int32_t* __restrict__ gcol) {
+  for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < nl_nnz; q += (int64_t)gridDim.x * blockDim.x) {
+    const int p = find_rank(nl_off, n_parts, q);
+    const int64_t c = nlcol_off[p] + nl_col[q];
+    gcol[q] = RP_IN(c, nlcol_off[p], nlcol_off[p + 1], kChkNonlocal) ? nl_cols[c] : 0;
+  }
+}
+
 // ------------------------------------------------------------------ host side
 
 namespace {
@@ -541,7 +553,7 @@ extern "C" const char* rp_status_str(rp_status s) {
 
 static void free_handle_memory(rp_handle* h) {
   void* ptrs[] = {h->row_ptr, h->col_idx, h->src_of, h->diag_pos, h->tpos, h->nl_row_ptr, h->nl_col_idx,
-                  h->nl_src_of, h->nl_cols, h->d_row_off, h->d_slot_off, h->d_face_off, h->d_iface_off,
+                  h->nl_src_of, h->nl_cols, h->nl_gcol, h->d_row_off, h->d_slot_off, h->d_face_off, h->d_iface_off,
                   h->d_lower, h->d_upper, h->d_iface_row, h->d_iface_gcol, h->d_out_off, h->staging, h->vals,
                   h->vals32, h->nl_vals, h->valsT, h->dinv, h->dinv32, h->dinvT, h->nl_vals32,
                   h->d_part_row_off, h->d_part_nnz_off, h->d_part_nl_off, h->d_part_nlcol_off};
@@ -860,6 +872,13 @@ extern "C" rp_status rp_build_repartition(const rp_ldu_desc* ranks, int32_t k, c
     CU(cudaMemcpyAsync(H->d_part_nnz_off, H->part_nnz_off.data(), 8 * np1, cudaMemcpyHostToDevice, st));
     CU(cudaMemcpyAsync(H->d_part_nl_off, H->part_nl_off.data(), 8 * np1, cudaMemcpyHostToDevice, st));
     CU(cudaMemcpyAsync(H->d_part_nlcol_off, nlcol.data(), 8 * np1, cudaMemcpyHostToDevice, st));
+    ALLOC(H->nl_gcol, H->nl_nnz + pad);
+    if (H->nl_nnz > 0) {
+      k_nl_gcol<<<grid_for(H, H->nl_nnz), kThreads, 0, st>>>(H->nl_nnz, o.n_parts, H->d_part_nl_off,
+                                                             H->d_part_nlcol_off, H->nl_col_idx, H->nl_cols,
+                                                             H->nl_gcol);
+      CU(cudaGetLastError());
+    }
   }
   CU(cudaStreamSynchronize(st));
   H->grid = grid_for(H, n);
@@ -914,6 +933,7 @@ namespace rp {
 rp_status check_read_update(CheckWord*, int);
 rp_status check_read_sliced(CheckWord*, int);
 rp_status check_read_pcg(CheckWord*, int);
+rp_status check_read_resident(CheckWord*, int);
 rp_status check_read_batch(CheckWord*, int);
 rp_status check_read_bicgstab(CheckWord*, int);
 rp_status check_read_adjoint(CheckWord*, int);
@@ -930,7 +950,7 @@ extern "C" rp_status rp_check_violations(uint64_t* count, int32_t* first_site, i
 #ifdef RP_CHECK
   using Reader = rp_status (*)(CheckWord*, int);
   const Reader readers[] = {check_read_map,   check_read_update,   check_read_sliced, check_read_pcg,
-                            check_read_batch, check_read_bicgstab, check_read_adjoint, check_read_noalloc};
+                            check_read_resident, check_read_batch, check_read_bicgstab, check_read_adjoint, check_read_noalloc};
   RP_TRY_CUDA(cudaDeviceSynchronize());
   for (Reader r : readers) {
     CheckWord w{};

@@ -19,30 +19,10 @@
 #include <type_traits>
 
 #include "rp_common.cuh"
+#include "rp_pcg.cuh"
 #include "rp_spmv.cuh"
 
 namespace rp {
-
-template <typename T>
-struct IterArgs {
-  int64_t n;
-  const int32_t* row_ptr;
-  const int32_t* col;
-  const T* vals;
-  const T* dinv;
-  T* r;
-  T* p;
-  T* q;
-  T* xd;  // iterate updated by K3: the correction d (mixed); nullptr = io->x
-  Ctl* ctl;
-  SolveIO* io;
-  double* partials;
-  cudaGraphConditionalHandle inner;
-  int in_graph;  // 0: launched on a stream (kernel timing), no condition to set
-  Parts<T> parts;
-  Sliced<T> sl;  // K1 runs k_it_spmv_sl when built (n_slices > 0)
-  Line<T> line;  // line preconditioner (K2 writes z, K3 reads it); l == nullptr: Jacobi
-};
 
 struct ResArgs {
   int64_t n;
@@ -61,7 +41,7 @@ struct ResArgs {
   double* partials;
   cudaGraphConditionalHandle inner;
   cudaGraphConditionalHandle outer;
-  int in_graph;
+  int in_graph;  // 1: in a graph without the inner while node (resident iteration), 2: with it
   int ru;  // mixed: continued (not restarted) inner PCG across refinements
   Parts<double> parts;
   Line<double> line;   // FP64 path, line preconditioner
@@ -658,7 +638,7 @@ __global__ void __launch_bounds__(kThreads) k_res64(ResArgs a) {
     c->stop = go ? 0 : 1;
     c->skip_x = 0;
     if (a.in_graph) {
-      cudaGraphSetConditional(a.inner, go ? 1u : 0u);
+      if (a.in_graph > 1) cudaGraphSetConditional(a.inner, go ? 1u : 0u);
       cudaGraphSetConditional(a.outer, go ? 1u : 0u);
     }
   }
@@ -759,7 +739,7 @@ __global__ void __launch_bounds__(kThreads) k_res_mixed(ResArgs a) {
     c->skip_x = 0;
     c->skip_correct = go ? 0 : 1;
     if (a.in_graph) {
-      cudaGraphSetConditional(a.inner, go ? 1u : 0u);
+      if (a.in_graph > 1) cudaGraphSetConditional(a.inner, go ? 1u : 0u);
       cudaGraphSetConditional(a.outer, go ? 1u : 0u);
     }
   }
@@ -802,7 +782,7 @@ __global__ void __launch_bounds__(kThreads) k_correct(CorrectArgs a) {
 }
 
 __global__ void k_setup(Ctl* c, SolveIO* io, const double* b, double* x, double tol, double inner_tol, int x_zero,
-                        int max_iter, int max_restarts, int max_outer, double ru_delta = 0.0) {
+                        int max_iter, int max_restarts, int max_outer, double ru_delta, unsigned int* sync) {
   io->b = b;
   io->x = x;
   c->tol = tol;
@@ -823,6 +803,7 @@ __global__ void k_setup(Ctl* c, SolveIO* io, const double* b, double* x, double 
   c->skip_correct = 1;
   c->alpha = c->beta = 0.0;
   c->ticket = 0u;
+  sync[0] = sync[32] = 0u;
 }
 
 // y = A x and, optionally, x.y
@@ -891,6 +872,9 @@ struct SolveSet {
   CorrectArgs ca;
   void *res, *rup, *k2_64, *k3_64, *k2_32, *k3_32;
   int g2_64, g3_64, g2_32, g3_32;
+  ResidentPlan resident;  // of the inner iteration in the set's precision; fn = nullptr: K1-K3
+  ResidentArgs<double> rs64;
+  ResidentArgs<float> rs32;
 };
 
 SolveSet solve_set(rp_handle* h, int mode, const double* vals, const double* dinv, cudaGraphConditionalHandle hin,
@@ -965,6 +949,9 @@ SolveSet solve_set(rp_handle* h, int mode, const double* vals, const double* din
     k.g2_32 = h->igrid32.k2;
     k.g3_32 = h->igrid32.k3;
   }
+  k.resident = mixed ? resident_plan<float>(h, k.a32, k.scaled) : resident_plan<double>(h, k.a64, false);
+  k.rs64 = ResidentArgs<double>{k.a64, h->rsync, h->opts.spin_limit, k.resident.rows, INT32_MAX};
+  k.rs32 = ResidentArgs<float>{k.a32, h->rsync, h->opts.spin_limit, k.resident.rows, INT32_MAX};
   return k;
 }
 
@@ -974,9 +961,11 @@ rp_status launch1(void* fn, int grid, int threads, int smem, void* argp, cudaStr
   return RP_OK;
 }
 
-// while (outer) { residual pass; [p = z + beta p]; while (inner) { K1; K2; K3 }; [x += d] }
+// while (outer) { residual pass; [p = z + beta p]; while (inner) { K1; K2; K3 }; [x += d] },
+// the inner while replaced by the resident kernel where it takes the system (and
+// may be used: a cooperative node is refused under MPS).
 // mode: 0 FP64, 1 mixed (restarted inner PCG), 2 mixed with continued inner PCG
-rp_status build_solve_graph(rp_handle* h, int mode, const double* vals, const double* dinv,
+rp_status build_solve_graph(rp_handle* h, int mode, const double* vals, const double* dinv, bool may_reside,
                             cudaGraphExec_t* exec) {
   const bool mixed = mode != 0;
   GraphGuard top;
@@ -986,14 +975,28 @@ rp_status build_solve_graph(rp_handle* h, int mode, const double* vals, const do
   cudaGraphNode_t wout, nres, win, n1, n2, n3, ncor;
   cudaGraph_t obody = nullptr, ibody = nullptr;
   RP_TRY(add_while(top.g, &wout, nullptr, hout, &obody));
-  RP_TRY_CUDA(cudaGraphConditionalHandleCreate(&hin, obody, 0, 0));
-
-  SolveSet k = solve_set(h, mode, vals, dinv, hin, hout, 1);
+  SolveSet k = solve_set(h, mode, vals, dinv, 0, hout, 1);
+  const bool resident = may_reside && k.resident.fn != nullptr;
+  if (!resident) {
+    RP_TRY_CUDA(cudaGraphConditionalHandleCreate(&hin, obody, 0, 0));
+    k.ra.inner = k.a64.inner = k.a32.inner = hin;
+    k.ra.in_graph = 2;
+  }
   RP_TRY(add_kernel(obody, &nres, nullptr, k.res, h->grid, &k.ra));
   cudaGraphNode_t before_inner = nres, nru;
   if (mode == 2) {
     RP_TRY(add_kernel(obody, &nru, &nres, k.rup, h->grid, &k.ru));
     before_inner = nru;
+  }
+  if (resident) {
+    RP_TRY(add_kernel(obody, &win, &before_inner, k.resident.fn, k.resident.grid,
+                      mixed ? (void*)&k.rs32 : (void*)&k.rs64, k.resident.smem, k.resident.threads));
+    cudaLaunchAttributeValue coop{};
+    coop.cooperative = 1;
+    RP_TRY_CUDA(cudaGraphKernelNodeSetAttribute(win, cudaLaunchAttributeCooperative, &coop));
+    if (mixed) RP_TRY(add_kernel(obody, &ncor, &win, (void*)k_correct, h->grid, &k.ca));
+    RP_TRY_CUDA(cudaGraphInstantiate(exec, top.g, 0));
+    return RP_OK;
   }
   RP_TRY(add_while(obody, &win, &before_inner, hin, &ibody));
   if (mixed) {
@@ -1116,6 +1119,7 @@ rp_status ensure_solver_buffers(rp_handle* h) {
   RP_TRY(dalloc(&h->ctl, 1));
   RP_TRY(dalloc(&h->io, 1));
   RP_TRY(dalloc(&h->ticket, 4));
+  RP_TRY(dalloc(&h->rsync, 64));
   RP_TRY_CUDA(cudaMemset(h->ctl, 0, sizeof(Ctl)));
   RP_TRY_CUDA(cudaMemset(h->ticket, 0, 4 * sizeof(unsigned int)));
   return RP_OK;
@@ -1123,7 +1127,7 @@ rp_status ensure_solver_buffers(rp_handle* h) {
 
 void free_solver(rp_handle* h) {
   void* ptrs[] = {h->r, h->p, h->q, h->r32, h->p32, h->q32, h->d32, h->b_host_stage, h->x_host_stage,
-                  h->partials, h->ctl, h->io, h->ticket, h->ctl_spmv};
+                  h->partials, h->ctl, h->io, h->ticket, h->rsync, h->ctl_spmv};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   h->r = h->p = h->q = nullptr;
@@ -1133,6 +1137,7 @@ void free_solver(rp_handle* h) {
   h->ctl = nullptr;
   h->io = nullptr;
   h->ticket = nullptr;
+  h->rsync = nullptr;
   h->ctl_spmv = nullptr;
   if (h->graphs.fp64) cudaGraphExecDestroy(h->graphs.fp64);
   if (h->graphs.mixed) cudaGraphExecDestroy(h->graphs.mixed);
@@ -1144,7 +1149,7 @@ void free_solver(rp_handle* h) {
 rp_status launch_solve(rp_handle* h, cudaGraphExec_t exec, const double* b, double* x, double tol, bool x_zero,
                        int max_iter, rp_solve_info* info, cudaStream_t s) {
   k_setup<<<1, 1, 0, s>>>(h->ctl, h->io, b, x, tol, h->opts.inner_tol, x_zero ? 1 : 0, max_iter,
-                          h->opts.max_restarts, h->opts.max_outer, h->opts.ru_delta);
+                          h->opts.max_restarts, h->opts.max_outer, h->opts.ru_delta, h->rsync);
   RP_TRY_CUDA(cudaGetLastError());
   RP_TRY_CUDA(cudaGraphLaunch(exec, s));
   (void)info;
@@ -1182,7 +1187,12 @@ rp_status host_loop_solve(rp_handle* h, int mode, const double* vals, const doub
     RP_TRY(read());
     const bool go = !c.stop;
     while (!c.stop) {
-      if (mixed) {
+      if (k.resident.fn) {  // one iteration a launch
+        k.rs64.cap = k.rs32.cap = 1;
+        void* args[1] = {mixed ? (void*)&k.rs32 : (void*)&k.rs64};
+        RP_TRY_CUDA(cudaLaunchCooperativeKernel(k.resident.fn, dim3((unsigned)k.resident.grid),
+                                                dim3((unsigned)k.resident.threads), args, (size_t)k.resident.smem, s));
+      } else if (mixed) {
         launch_k1(k.a32, k1_grid(k.a32, h->igrid32), s);
         RP_TRY(launch1(k.k2_32, k.g2_32, kThreads, 0, &k.a32, s));
         RP_TRY(launch1(k.k3_32, k.g3_32, kThreads, 0, &k.a32, s));
@@ -1204,7 +1214,11 @@ rp_status host_loop_solve(rp_handle* h, int mode, const double* vals, const doub
 rp_status solve_common(rp_handle* h, int mode, const double* vals, const double* dinv, cudaGraphExec_t* slot,
                        const double* b, double* x, double tol, int32_t x_is_guess, int32_t where,
                        rp_solve_info* info, cudaStream_t s) {
-  if (!*slot && !h->opts.host_loop) RP_TRY(build_solve_graph(h, mode, vals, dinv, slot));
+  if (!*slot && !h->opts.host_loop && build_solve_graph(h, mode, vals, dinv, true, slot) != RP_OK) {
+    cudaGetLastError();
+    *slot = nullptr;
+    RP_TRY(build_solve_graph(h, mode, vals, dinv, false, slot));
+  }
   const double* bd = b;
   double* xd = x;
   if (where == RP_MEM_HOST) {
@@ -1217,7 +1231,7 @@ rp_status solve_common(rp_handle* h, int mode, const double* vals, const double*
   }
   if (h->opts.host_loop) {
     k_setup<<<1, 1, 0, s>>>(h->ctl, h->io, bd, xd, tol, h->opts.inner_tol, x_is_guess ? 0 : 1, h->opts.max_iter,
-                            h->opts.max_restarts, h->opts.max_outer, h->opts.ru_delta);
+                            h->opts.max_restarts, h->opts.max_outer, h->opts.ru_delta, h->rsync);
     RP_TRY(host_loop_solve(h, mode, vals, dinv, s));
   } else {
     RP_TRY(launch_solve(h, *slot, bd, xd, tol, !x_is_guess, h->opts.max_iter, info, s));
@@ -1367,7 +1381,7 @@ extern "C" rp_status rp_profile_iteration(rp_handle* h, const double* b, int32_t
   }
   RP_TRY(dalloc(&h->x_host_stage, h->n + 64));
   // a fresh CG run from x = 0 that never meets its tolerance (tol = 0)
-  k_setup<<<1, 1, 0, s>>>(h->ctl, h->io, b, h->x_host_stage, 0.0, 0.0, 1, iters + 2, 0, 1);
+  k_setup<<<1, 1, 0, s>>>(h->ctl, h->io, b, h->x_host_stage, 0.0, 0.0, 1, iters + 2, 0, 1, 0.0, h->rsync);
   SolveSet k = solve_set(h, mixed ? 1 : 0, h->vals, h->dinv, 0, 0, 0);
   RP_TRY(launch1(k.res, h->grid, kThreads, 0, &k.ra, s));
   std::vector<cudaEvent_t> ev(3 * iters + 1, nullptr);

@@ -10,16 +10,24 @@
 
 namespace rp {
 
+// A gather from x: read-only path, or (COH) a plain load for a vector that the
+// same kernel writes.
+template <bool COH, typename T>
+__device__ __forceinline__ T xload(const T* p) {
+  if (COH) return *p;
+  return __ldg(p);
+}
+
 // Row i of a CSR matrix with ncols columns (ncols bounds the gathers in the
 // bounds-checked build).
-template <typename T>
+template <typename T, bool COH = false>
 __device__ __forceinline__ T row_dot(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
-                                     const T* __restrict__ vals, const T* __restrict__ x, int64_t i, int64_t ncols) {
+                                     const T* __restrict__ vals, const T* x, int64_t i, int64_t ncols) {
   const int s = __ldg(row_ptr + i), e = __ldg(row_ptr + i + 1);
   T sum = T(0);
   for (int j = s; j < e; ++j) {
     const int c = __ldg(col + j);
-    if (RP_IN(c, 0, ncols, kChkGather)) sum = fma(__ldg(vals + j), __ldg(x + c), sum);
+    if (RP_IN(c, 0, ncols, kChkGather)) sum = fma(__ldg(vals + j), xload<COH>(x + c), sum);
   }
   return sum;
 }
@@ -29,23 +37,28 @@ __device__ __forceinline__ T row_dot(const int32_t* __restrict__ row_ptr, const 
 // when the compressed column or its row is out of range.
 template <typename T>
 __device__ __forceinline__ int nl_row_of(const Parts<T>& P, int p, int64_t nlo, int64_t nco, int j) {
+#ifdef RP_CHECK
   const int cc = __ldg(P.nl_col + nlo + j);
   if (!RP_IN(cc, 0, __ldg(P.nlcol_off + p + 1) - nco, kChkNonlocal)) return -1;
   const int g = __ldg(P.nl_cols + nco + cc);
   return RP_IN(g, 0, __ldg(P.row_off + P.n), kChkNonlocal) ? g : -1;
+#else
+  (void)p, (void)nco;
+  return __ldg(P.nl_gcol + nlo + j);
+#endif
 }
 
 // The non-local entries of row i (part p) added to sum in their CSR order:
 // the part's non-local CSR, whose compressed columns name the halo rows -- on
 // one GPU the halo exchange is this gather from x (global vector).
-template <typename T>
-__device__ __forceinline__ T nonlocal_add(const Parts<T>& P, int p, int64_t i, const T* __restrict__ x, T sum) {
+template <typename T, bool COH = false>
+__device__ __forceinline__ T nonlocal_add(const Parts<T>& P, int p, int64_t i, const T* x, T sum) {
   const int64_t r0 = __ldg(P.row_off + p), li = i - r0;
   const int32_t* nrp = P.nl_row_ptr + r0 + p;
   const int64_t nlo = __ldg(P.nl_off + p), nco = __ldg(P.nlcol_off + p);
   for (int j = __ldg(nrp + li); j < __ldg(nrp + li + 1); ++j) {
     const int g = nl_row_of<T>(P, p, nlo, nco, j);
-    if (RP_IDX_OK(g)) sum = fma(__ldg(P.nl_vals + nlo + j), __ldg(x + g), sum);
+    if (RP_IDX_OK(g)) sum = fma(__ldg(P.nl_vals + nlo + j), xload<COH>(x + g), sum);
   }
   return sum;
 }
@@ -58,28 +71,26 @@ struct NlRange {
 };
 template <typename T>
 __device__ __forceinline__ NlRange nonlocal_range(const Parts<T>& P, int p, int64_t i) {
-  const int64_t r0 = __ldg(P.row_off + p), li = i - r0;
-  const int32_t* nrp = P.nl_row_ptr + r0 + p;
-  return NlRange{__ldg(nrp + li), __ldg(nrp + li + 1)};
+  const int32_t* nrp = P.nl_row_ptr + i + p;  // part p's segment starts at row_off[p] + p
+  return NlRange{__ldg(nrp), __ldg(nrp + 1)};
 }
-template <typename T>
-__device__ __forceinline__ T nonlocal_sum(const Parts<T>& P, int p, const NlRange& r, const T* __restrict__ x,
-                                          T sum) {
+template <typename T, bool COH = false>
+__device__ __forceinline__ T nonlocal_sum(const Parts<T>& P, int p, const NlRange& r, const T* x, T sum) {
   if (r.j0 == r.j1) return sum;
   const int64_t nlo = __ldg(P.nl_off + p), nco = __ldg(P.nlcol_off + p);
   for (int j = r.j0; j < r.j1; ++j) {
     const int g = nl_row_of<T>(P, p, nlo, nco, j);
-    if (RP_IDX_OK(g)) sum = fma(__ldg(P.nl_vals + nlo + j), __ldg(x + g), sum);
+    if (RP_IDX_OK(g)) sum = fma(__ldg(P.nl_vals + nlo + j), xload<COH>(x + g), sum);
   }
   return sum;
 }
 
 // Row i of the matrix split into parts (Sec. 3): the part's local CSR (part-
 // local columns), then its non-local entries.
-template <typename T>
+template <typename T, bool COH = false>
 __device__ __forceinline__ T row_dot_parts(const Parts<T>& P, const int32_t* __restrict__ row_ptr,
                                            const int32_t* __restrict__ col, const T* __restrict__ vals,
-                                           const T* __restrict__ x, int64_t i) {
+                                           const T* x, int64_t i) {
   const int p = find_rank(P.row_off, P.n, i);
   const int64_t r0 = __ldg(P.row_off + p), li = i - r0;
   const int32_t* rp = row_ptr + r0 + p;
@@ -87,26 +98,27 @@ __device__ __forceinline__ T row_dot_parts(const Parts<T>& P, const int32_t* __r
   T sum = T(0);
   for (int j = __ldg(rp + li); j < __ldg(rp + li + 1); ++j) {
     const int c = __ldg(col + no + j);
-    if (RP_IN(c, 0, __ldg(P.row_off + p + 1) - r0, kChkGather)) sum = fma(__ldg(vals + no + j), __ldg(x + r0 + c), sum);
+    if (RP_IN(c, 0, __ldg(P.row_off + p + 1) - r0, kChkGather)) sum = fma(__ldg(vals + no + j), xload<COH>(x + r0 + c), sum);
   }
-  return nonlocal_add<T>(P, p, i, x, sum);
+  return nonlocal_add<T, COH>(P, p, i, x, sum);
 }
 
 inline Parts<double> parts64(const rp_handle* h) {
   return Parts<double>{h->n_parts, h->d_part_row_off, h->d_part_nnz_off, h->d_part_nl_off, h->d_part_nlcol_off,
-                       h->nl_row_ptr, h->nl_col_idx, h->nl_cols, h->nl_vals};
+                       h->nl_row_ptr, h->nl_col_idx, h->nl_cols, h->nl_vals, h->nl_gcol};
 }
 inline Parts<float> parts32(const rp_handle* h) {
   return Parts<float>{h->n_parts, h->d_part_row_off, h->d_part_nnz_off, h->d_part_nl_off, h->d_part_nlcol_off,
-                      h->nl_row_ptr, h->nl_col_idx, h->nl_cols, h->nl_vals32};
+                      h->nl_row_ptr, h->nl_col_idx, h->nl_cols, h->nl_vals32, h->nl_gcol};
 }
 
 // Row i of the merged matrix (n rows), one part or several.
-template <typename T>
+template <typename T, bool COH = false>
 __device__ __forceinline__ T row_dot_any(const Parts<T>& P, const int32_t* __restrict__ row_ptr,
                                          const int32_t* __restrict__ col, const T* __restrict__ vals,
-                                         const T* __restrict__ x, int64_t i, int64_t n) {
-  return P.n > 1 ? row_dot_parts<T>(P, row_ptr, col, vals, x, i) : row_dot<T>(row_ptr, col, vals, x, i, n);
+                                         const T* x, int64_t i, int64_t n) {
+  return P.n > 1 ? row_dot_parts<T, COH>(P, row_ptr, col, vals, x, i)
+                 : row_dot<T, COH>(row_ptr, col, vals, x, i, n);
 }
 
 // The sliced layout of the iteration (with per-slice row records when the
@@ -300,14 +312,6 @@ __device__ __forceinline__ bool slice_ok(uint32_t wd, int e, int off, int D, con
   (void)wd, (void)e, (void)off, (void)D, (void)ck;
   return true;
 #endif
-}
-
-// A gather from x: read-only path, or (COH) a plain load for a vector that the
-// same kernel writes.
-template <bool COH, typename T>
-__device__ __forceinline__ T xload(const T* p) {
-  if (COH) return *p;
-  return __ldg(p);
 }
 
 // Sum of one row of a slice, L entries: values at v[32 k] (lane applied),
