@@ -365,6 +365,7 @@ struct rp_handle {
   // the first such solve, refilled by every value update afterwards
   float* sl_vals32s = nullptr;
   double* s64 = nullptr;  // n: s_i = 1/sqrt(a_ii)
+  float2* s2 = nullptr;   // n: s_i as FP32 pairs (rp_values.cuh)
 
   // solver work space
   double *r = nullptr, *p = nullptr, *q = nullptr;
@@ -417,7 +418,7 @@ inline int grid_for(const rp_handle* h, int64_t n) {
 rp_status ensure_solver_buffers(rp_handle* h);
 rp_status build_sliced(rp_handle* h, cudaStream_t s);  // after the CSR map
 rp_status fill_sliced_transposed(rp_handle* h, cudaStream_t s);  // sl_valsT from valsT
-rp_status fill_sliced(rp_handle* h, cudaStream_t s);   // after every value update
+rp_status fill_sliced(rp_handle* h, const double* buf, cudaStream_t s);  // the value update of a sliced handle
 // the scaled inner system of the mixed PCG solves: allocated and filled from the
 // current values on first use (then refilled by fill_sliced); false when the
 // handle does not take it (several parts, CSR layout, no FP32 copy)
@@ -505,6 +506,24 @@ __device__ __forceinline__ int find_rank(const int64_t* __restrict__ off, int k,
     if (__ldg(off + mid) <= t) lo = mid; else hi = mid;
   }
   return lo;
+}
+
+// Elements t of a table off[0..k] (off[r] <= t < off[r + 1]: rank r), a run of
+// 128 a warp, four a lane: f(r, t) for every t. One search serves the run
+// where it lies in one rank (a search an element took 7 dependent loads).
+template <typename F>
+__device__ __forceinline__ void for_ranked(const int64_t* __restrict__ off, int k, F&& f) {
+  const int lane = threadIdx.x & 31;
+  const int64_t total = __ldg(off + k), step = ((int64_t)gridDim.x * blockDim.x) * 4;
+  for (int64_t t0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 128; t0 < total; t0 += step) {
+    const int r0 = find_rank(off, k, t0);
+    const bool one = __ldg(off + r0 + 1) >= t0 + 128;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int64_t t = t0 + 32 * u + lane;
+      if (t < total) f(one ? r0 : find_rank(off, k, t), t);
+    }
+  }
 }
 
 }  // namespace rp

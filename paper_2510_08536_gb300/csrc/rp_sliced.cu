@@ -32,6 +32,7 @@
 #include <vector>
 
 #include "rp_common.cuh"
+#include "rp_values.cuh"
 
 namespace rp {
 namespace {
@@ -203,10 +204,9 @@ __global__ void __launch_bounds__(kThreads)
 }
 
 // sliced values from the CSR values: v[q] = vals[pos[q]], 0 for padding
-template <bool FP32>
 __global__ void __launch_bounds__(kThreads)
     k_slice_vals(int64_t nq4, const int4* __restrict__ pos, const double* __restrict__ vals,
-                 double2* __restrict__ out, float4* __restrict__ out32, int64_t nnz) {
+                 double2* __restrict__ out, int64_t nnz) {
   // a CSR position, or -1 for padding (bounds-checked build: anything else reads 0)
   auto at = [&](int32_t q) { return q >= 0 && RP_IN(q, 0, nnz, kChkSliceValues) ? __ldg(vals + q) : 0.0; };
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nq4; i += (int64_t)gridDim.x * blockDim.x) {
@@ -214,7 +214,157 @@ __global__ void __launch_bounds__(kThreads)
     const double a = at(p.x), b = at(p.y), c = at(p.z), d = at(p.w);
     __stcs(out + 2 * i, make_double2(a, b));
     __stcs(out + 2 * i + 1, make_double2(c, d));
-    if (FP32) __stcs(out32 + i, make_float4((float)a, (float)b, (float)c, (float)d));
+  }
+}
+
+// The value update of the sliced layout: CSR values, FP32 copies and sliced
+// values of both precisions (SCALED: and the FP32 values of S A S) from the
+// buffer in one pass.
+struct FillArgs {
+  int64_t S, n;
+  const double* buf;
+  const int64_t* slot_off;  // buffer of part p: slots slot_off[p alpha] .. slot_off[(p + 1) alpha]
+  int32_t alpha;
+  const int64_t* nnz_off;
+  const int2* srow;  // several parts
+  const int32_t* row_ptr;
+  const int32_t* src_of;
+  const uint2* desc;
+  const uint32_t* tinfo;
+  const int32_t* tabs;
+  const uint32_t* ibuf;
+  const double* s64;
+  const float2* s2;
+  double* vals;
+  float* vals32;
+  double* out;
+  float* out32;
+  float* out32s;
+};
+
+// One warp a slice. Its rows are one run of CSR entries: the warp reads the
+// run's slots and gathers the buffer coalesced (eight of each in flight),
+// writes the CSR values, keeps the run in shared memory and writes the slice
+// from there, a row a lane. (A permutation to CSR, a gather from CSR to the slices
+// and a third pass for S A S moved 60 bytes an entry where this moves 40: 2.30 ms
+// an update at 256^3 with S A S, 1.27 ms now; 120 us of it here at 128^3, 60% of
+// HBM, bound by the chain row pointer, slot, buffer.) Runs of more than kRun entries (rows longer than 8 on
+// average) gather the slice's entries from the buffer again, rows of more than 8
+// entries and 8-bit indices take the general loop.
+constexpr int kRun = 8 * kSliceRows;
+template <bool FP32, bool SCALED>
+__global__ void __launch_bounds__(kThreads, 4) k_fill_slices(const FillArgs A) {
+  __shared__ double sval[kWarpsPerBlock][kRun];
+  __shared__ float sval32[FP32 ? kWarpsPerBlock : 1][kRun];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  double* sv = sval[w];
+  float* sf = sval32[FP32 ? w : 0];
+  const int S = (int)A.S, step = gridDim.x * kWarpsPerBlock;
+  for (int s = blockIdx.x * kWarpsPerBlock + w; s < S; s += step) {
+    int row0 = s * kSliceRows, rows = min(kSliceRows, (int)A.n - s * kSliceRows), part = 0;
+    if (A.srow) {
+      const int2 r = __ldg(A.srow + s);
+      row0 = r.x;
+      rows = r.y & 63;
+      part = r.y >> 6;
+    }
+    const bool valid = lane < rows;
+    const int i = row0 + lane;
+    const int32_t* rp = A.row_ptr + i + part;
+    const int beg = valid ? __ldg(rp) : 0, len = valid ? __ldg(rp + 1) - beg : 0;
+    const uint2 d0 = __ldg(A.desc + s), d1 = __ldg(A.desc + s + 1);
+    const uint32_t info = SCALED ? __ldg(A.tinfo + s) : kSliceW4;
+    const int32_t* tab = A.tabs + (info & ~kSliceW4);
+    const int L = (int)((d1.x - d0.x) >> 5);
+    const int beg0 = __shfl_sync(0xffffffffu, beg, 0), m = (int)__reduce_add_sync(0xffffffffu, (unsigned)len);
+    const int at = beg - beg0;
+    const int64_t q0 = __ldg(A.nnz_off + part) + beg0;
+    const int64_t b0 = __ldg(A.slot_off + (int64_t)part * A.alpha);
+    const int64_t blen = __ldg(A.slot_off + (int64_t)(part + 1) * A.alpha) - b0;
+    const double* buf = A.buf + b0;
+    float2 si = make_float2(0.f, 0.f);
+    if (SCALED && valid) si = __ldg(A.s2 + i);
+    // entry v with the column's scale sj, offset id of the slice's table
+    auto scaled = [&](double v, float2 sj, uint32_t id) {
+      bool ok;
+      float f = scaled_value(v, si, sj, ok);
+      if (!ok) {
+        const int j = i + __ldg(tab + id);
+        f = RP_IN(j, 0, A.n, kChkGather) ? (float)(v * (__ldg(A.s64 + i) * __ldg(A.s64 + j))) : 0.f;
+      }
+      return f;
+    };
+    const int32_t* src = A.src_of + q0 + lane;
+    double* cv = A.vals + q0 + lane;
+    double* out = A.out + d0.x + lane;
+    float* out32 = FP32 ? A.out32 + d0.x + lane : nullptr;
+    float* out32s = SCALED ? A.out32s + d0.x + lane : nullptr;
+    __syncwarp();  // the previous slice's readers of sv are done
+    for (int c = 0; c < m; c += kRun, src += kRun, cv += kRun) {
+      const int rest = m - c - lane;
+      int32_t t[8];
+      double v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (32 * u < rest) t[u] = __ldcs(src + 32 * u);
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (32 * u < rest) v[u] = slot_value(buf, t[u], blen);
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (32 * u < rest) {
+          __stcs(cv + 32 * u, v[u]);
+          sv[32 * u + lane] = v[u];
+          if (FP32) {
+            const float f = f32_rn(v[u]);
+            __stcs(A.vals32 + (cv - A.vals) + 32 * u, f);
+            sf[32 * u + lane] = f;
+          }
+        }
+    }
+    __syncwarp();
+    if (m <= kRun && L <= 8 && (info & kSliceW4)) {
+      const uint32_t wd = SCALED ? __ldg(A.ibuf + d0.y + lane) : 0u;
+      const int32_t tv = SCALED ? __ldg(tab + (lane & 15)) : 0;
+#pragma unroll
+      for (int u0 = 0; u0 < 8; u0 += 4) {  // in halves: the gathered scales of all eight spill
+        float2 sj[4];
+        if (SCALED) {
+#pragma unroll
+          for (int u = u0; u < u0 + 4; ++u)
+            if (u < L) {
+              const int off = __shfl_sync(0xffffffffu, tv, (int)(wd >> (4 * u)), 16);
+              sj[u - u0] = u < len && RP_IN(i + off, 0, A.n, kChkGather) ? __ldg(A.s2 + i + off) : make_float2(0.f, 0.f);
+            }
+        }
+#pragma unroll
+        for (int u = u0; u < u0 + 4; ++u)
+          if (u < L) {
+            const bool has = u < len;
+            const double v = has ? sv[at + u] : 0.0;
+            __stcs(out + kSliceRows * u, v);
+            if (FP32) __stcs(out32 + kSliceRows * u, has ? sf[at + u] : 0.f);
+            if (SCALED) __stcs(out32s + kSliceRows * u, has ? scaled(v, sj[u - u0], (wd >> (4 * u)) & 15u) : 0.f);
+          }
+      }
+    } else {
+      const int per = (info & kSliceW4) ? 8 : 4, bits = (info & kSliceW4) ? 4 : 8;
+      for (int k = 0; k < L; ++k) {
+        const bool has = k < len;
+        double v = 0.0;
+        if (has) v = m <= kRun ? sv[at + k] : slot_value(buf, A.src_of[q0 + at + k], blen);
+        __stcs(out + kSliceRows * k, v);
+        if (FP32) __stcs(out32 + kSliceRows * k, has ? f32_rn(v) : 0.f);
+        if (SCALED) {
+          float f = 0.f;
+          const uint32_t wd = __ldg(A.ibuf + d0.y + (uint32_t)(kSliceRows * (k / per)) + lane);
+          const uint32_t id = (wd >> (bits * (k % per))) & ((1u << bits) - 1u);
+          const int off = __ldg(tab + id);
+          if (has && RP_IN(i + off, 0, A.n, kChkGather)) f = scaled(v, __ldg(A.s2 + i + off), id);
+          __stcs(out32s + kSliceRows * k, f);
+        }
+      }
+    }
   }
 }
 
@@ -247,11 +397,12 @@ struct Tmp {
 
 void free_sliced(rp_handle* h) {
   void* ptrs[] = {h->sl_part_soff, h->sl_srow, h->sl_desc, h->sl_tinfo, h->sl_tabs, h->sl_ibuf, h->sl_pos,
-                  h->sl_vals, h->sl_vals32, h->sl_valsT, h->sl_vals32s, h->s64};
+                  h->sl_vals, h->sl_vals32, h->sl_valsT, h->sl_vals32s, h->s64, h->s2};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   h->sl_vals32s = nullptr;
   h->s64 = nullptr;
+  h->s2 = nullptr;
   h->sl_part_soff = nullptr;
   h->sl_srow = nullptr;
   h->sl_desc = nullptr;
@@ -401,13 +552,16 @@ rp_status build_sliced(rp_handle* h, cudaStream_t st) {
   return RP_OK;
 }
 
-// s_i = 1 / sqrt(a_ii): FP64 square root and division (both correctly rounded)
+// s_i = 1 / sqrt(a_ii): FP64 square root and division (both correctly rounded), from
+// the current values (the value update computes them itself, k_dinv)
 __global__ void __launch_bounds__(kThreads)
     k_scaling(int64_t n, const int32_t* __restrict__ diag_pos, const double* __restrict__ vals, int64_t nnz,
-              double* __restrict__ s64) {
+              double* __restrict__ s64, float2* __restrict__ s2) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const int32_t d = diag_pos[i];
-    s64[i] = RP_IN(d, 0, nnz, kChkSliceValues) ? 1.0 / sqrt(__ldg(vals + d)) : 0.0;
+    const double s = RP_IN(d, 0, nnz, kChkSliceValues) ? 1.0 / sqrt(__ldg(vals + d)) : 0.0;
+    s64[i] = s;
+    s2[i] = scale_pair(s);
   }
 }
 
@@ -448,8 +602,9 @@ __global__ void __launch_bounds__(kThreads)
   }
 }
 
+// the values of S A S from the current ones, for the first mixed solve
 static rp_status fill_scaled(rp_handle* h, cudaStream_t s) {
-  k_scaling<<<grid_for(h, h->n), kThreads, 0, s>>>(h->n, h->diag_pos, h->vals, h->nnz, h->s64);
+  k_scaling<<<grid_for(h, h->n), kThreads, 0, s>>>(h->n, h->diag_pos, h->vals, h->nnz, h->s64, h->s2);
   k_slice_vals_scaled<<<grid_for(h, h->sl_slices * kSliceRows), kThreads, 0, s>>>(
       h->sl_slices, h->sl_desc, h->sl_tinfo, h->sl_tabs, reinterpret_cast<const uint32_t*>(h->sl_ibuf), h->sl_vals,
       h->s64, h->n, h->sl_vals32s);
@@ -460,31 +615,24 @@ static rp_status fill_scaled(rp_handle* h, cudaStream_t s) {
 rp_status ensure_scaled(rp_handle* h, cudaStream_t s, bool* ok) {
   *ok = h->n_parts == 1 && h->sl_slices > 0 && h->sl_vals32 != nullptr && h->n > 0;
   if (!*ok || h->sl_vals32s) return RP_OK;
-  RP_TRY(salloc(&h->s64, h->n + 64));
-  rp_status st = salloc(&h->sl_vals32s, h->sl_entries);
-  if (st != RP_OK) {
-    cudaFree(h->s64);
-    h->s64 = nullptr;
-    return st;
-  }
+  if (!h->s64) RP_TRY(salloc(&h->s64, h->n + 64));
+  if (!h->s2) RP_TRY(salloc(&h->s2, h->n + 64));
+  RP_TRY(salloc(&h->sl_vals32s, h->sl_entries));
   return fill_scaled(h, s);
 }
 
 RP_CHECK_TU(sliced)
 
-rp_status fill_sliced(rp_handle* h, cudaStream_t s) {
-  if (h->sl_slices == 0) return RP_OK;
-  const int64_t nq4 = h->sl_entries / 4;  // a multiple of 32 entries
-  const int g = grid_for(h, nq4);
-  const int4* pos = reinterpret_cast<const int4*>(h->sl_pos);
-  double2* out = reinterpret_cast<double2*>(h->sl_vals);
-  if (h->sl_vals32)
-    k_slice_vals<true><<<g, kThreads, 0, s>>>(nq4, pos, h->vals, out, reinterpret_cast<float4*>(h->sl_vals32),
-                                              h->nnz);
-  else
-    k_slice_vals<false><<<g, kThreads, 0, s>>>(nq4, pos, h->vals, out, nullptr, h->nnz);
+rp_status fill_sliced(rp_handle* h, const double* buf, cudaStream_t s) {
+  const FillArgs a{h->sl_slices, h->n, buf, h->d_slot_off, h->k / h->n_parts, h->d_part_nnz_off, h->sl_srow,
+                   h->row_ptr, h->src_of, h->sl_desc, h->sl_tinfo, h->sl_tabs,
+                   reinterpret_cast<const uint32_t*>(h->sl_ibuf), h->s64, h->s2, h->vals, h->vals32, h->sl_vals,
+                   h->sl_vals32, h->sl_vals32s};
+  const int g = slice_grid(h, h->sl_slices);
+  if (h->sl_vals32s) k_fill_slices<true, true><<<g, kThreads, 0, s>>>(a);
+  else if (h->sl_vals32) k_fill_slices<true, false><<<g, kThreads, 0, s>>>(a);
+  else k_fill_slices<false, false><<<g, kThreads, 0, s>>>(a);
   RP_TRY_CUDA(cudaGetLastError());
-  if (h->sl_vals32s) RP_TRY(fill_scaled(h, s));
   return RP_OK;
 }
 
@@ -495,8 +643,8 @@ rp_status fill_sliced_transposed(rp_handle* h, cudaStream_t s) {
   if (h->sl_slices == 0 || !h->valsT) return RP_OK;
   if (!h->sl_valsT) RP_TRY(salloc(&h->sl_valsT, h->sl_entries));
   const int64_t nq4 = h->sl_entries / 4;
-  k_slice_vals<false><<<grid_for(h, nq4), kThreads, 0, s>>>(nq4, reinterpret_cast<const int4*>(h->sl_pos), h->valsT,
-                                                            reinterpret_cast<double2*>(h->sl_valsT), nullptr, h->nnz);
+  k_slice_vals<<<grid_for(h, nq4), kThreads, 0, s>>>(nq4, reinterpret_cast<const int4*>(h->sl_pos), h->valsT,
+                                                     reinterpret_cast<double2*>(h->sl_valsT), h->nnz);
   RP_TRY_CUDA(cudaGetLastError());
   return RP_OK;
 }

@@ -1,21 +1,17 @@
 // Value update (Sec. 3, update procedure): the continuous buffer, ordered by
 // rank and LDU order, is reordered into the row-major device matrix by the
-// permutation P (src_of). The sparsity is never rebuilt. When the iteration
-// runs on the sliced layout, a second gather refills its values from the
-// CSR values (k_slice_vals: 4 + 8 bytes read, 8 + 4 written per padded entry).
+// permutation P (src_of). The sparsity is never rebuilt. Where the iteration
+// runs on the sliced layout, the same pass over the buffer writes the CSR
+// values, their FP32 copies, the sliced values in both precisions and, once a
+// mixed solve has asked for them, the FP32 values of S A S.
 //
-// Roofline: HBM bound. Per stored entry one 4-byte index read, one 8-byte
-// gathered read and one 8-byte write (+4 bytes for the FP32 copy); the
-// gather is nearly sequential (a handful of monotone streams per rank), so
-// it moves close to the algorithmic bytes.
+// Bound: HBM, with the FP64 pipe (two lanes a clock and SM, conversions
+// included) close behind: 4 + 8 bytes read and 8 + 4 + 8 + 4 [+ 4] written an
+// entry, and per row one division (with S A S: two and a square root).
 #include "rp_common.cuh"
+#include "rp_values.cuh"
 
 namespace rp {
-
-// buffer value at slot s (bounds-checked build: slots outside [0, len) read 0)
-__device__ __forceinline__ double slot_value(const double* __restrict__ buf, int32_t s, int64_t len) {
-  return RP_IN(s, 0, len, kChkPermute) ? __ldg(buf + s) : 0.0;
-}
 
 template <bool FP32>
 __global__ void __launch_bounds__(kThreads)
@@ -48,54 +44,79 @@ __global__ void __launch_bounds__(kThreads)
   }
 }
 
-// Jacobi diagonal straight from the diagonal block of each rank (contiguous
-// in the buffer): dinv[i] = 1 / a_ii, and 1/(float)a_ii for the FP32 copy.
+// The non-local entries of all parts: entry i belongs to the part whose range
+// of nl_off holds it, its slot counts from the part's first buffer slot
+// (slot_off[part * alpha], alpha ranks a part).
 template <bool FP32>
 __global__ void __launch_bounds__(kThreads)
-    k_dinv(const double* __restrict__ buf, const int64_t* __restrict__ row_off,
-           const int64_t* __restrict__ slot_off, int k, int64_t n, double* __restrict__ dinv,
-           float* __restrict__ dinv32) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    int r = find_rank(row_off, k, i);
-    double d = __ldg(buf + slot_off[r] + (i - row_off[r]));
-    dinv[i] = 1.0 / d;
-    if (FP32) dinv32[i] = 1.0f / (float)d;
+    k_permute_nonlocal(const double* __restrict__ buf, const int64_t* __restrict__ slot_off, int alpha,
+                       const int64_t* __restrict__ nl_off, int n_parts, const int32_t* __restrict__ src_of,
+                       double* __restrict__ vals, float* __restrict__ vals32, int64_t nnz) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nnz; i += (int64_t)gridDim.x * blockDim.x) {
+    const int p = find_rank(nl_off, n_parts, i);
+    const int64_t b0 = __ldg(slot_off + (int64_t)p * alpha);
+    const double v = slot_value(buf + b0, src_of[i], __ldg(slot_off + (int64_t)(p + 1) * alpha) - b0);
+    vals[i] = v;
+    if (FP32) vals32[i] = (float)v;
   }
 }
 
+// Jacobi diagonal straight from the diagonal block of each rank (contiguous
+// in the buffer): dinv[i] = 1 / a_ii, and 1/(float)a_ii for the FP32 copy.
+// s64: also the scaling s_i = 1/sqrt(a_ii) of S A S and its FP32 pair (one
+// part; the same values the merged diagonal holds).
+template <bool FP32>
+__global__ void __launch_bounds__(kThreads)
+    k_dinv(const double* __restrict__ buf, const int64_t* __restrict__ row_off,
+           const int64_t* __restrict__ slot_off, int k, double* __restrict__ dinv,
+           float* __restrict__ dinv32, double* __restrict__ s64, float2* __restrict__ s2) {
+  for_ranked(row_off, k, [&](int r, int64_t i) {
+    const double d = __ldcs(buf + __ldg(slot_off + r) + (i - __ldg(row_off + r)));
+    dinv[i] = recip_rn(d);
+    if (FP32) dinv32[i] = 1.0f / f32_rn(d);
+    if (s64) {
+      const double sc = recip_rn(sqrt_rn(d));
+      s64[i] = sc;
+      s2[i] = scale_pair(sc);
+    }
+  });
+}
+
 static rp_status permute_all(rp_handle* h, const double* buf, cudaStream_t s) {
-  for (int p = 0; p < h->n_parts; ++p) {
-    const double* base = buf + h->part_buf_off[p];
-    const int64_t blen = h->part_buf_off[p + 1] - h->part_buf_off[p];
-    int64_t o = h->part_nnz_off[p], cnt = h->part_nnz_off[p + 1] - o;
-    int g = grid_for(h, (cnt + 3) / 4);
-    if (cnt > 0) {
+  if (h->n > 0) {
+    if (h->want_fp32)
+      k_dinv<true><<<grid_for(h, h->n / 4), kThreads, 0, s>>>(buf, h->d_row_off, h->d_slot_off, h->k, h->dinv, h->dinv32,
+                                                              h->sl_vals32s ? h->s64 : nullptr, h->s2);
+    else
+      k_dinv<false><<<grid_for(h, h->n / 4), kThreads, 0, s>>>(buf, h->d_row_off, h->d_slot_off, h->k, h->dinv, nullptr,
+                                                               nullptr, nullptr);
+  }
+  if (h->sl_slices > 0) {
+    RP_TRY(fill_sliced(h, buf, s));
+  } else {
+    for (int p = 0; p < h->n_parts; ++p) {
+      const double* base = buf + h->part_buf_off[p];
+      const int64_t blen = h->part_buf_off[p + 1] - h->part_buf_off[p];
+      int64_t o = h->part_nnz_off[p], cnt = h->part_nnz_off[p + 1] - o;
+      int g = grid_for(h, (cnt + 3) / 4);
+      if (cnt <= 0) continue;
       if (h->want_fp32)
         k_permute<true><<<g, kThreads, 0, s>>>(base, h->src_of + o, h->vals + o, h->vals32 + o, cnt, blen);
       else
         k_permute<false><<<g, kThreads, 0, s>>>(base, h->src_of + o, h->vals + o, nullptr, cnt, blen);
     }
-    int64_t no = h->part_nl_off[p], ncnt = h->part_nl_off[p + 1] - no;
-    if (ncnt > 0) {
-      if (h->want_fp32)
-        k_permute<true><<<grid_for(h, (ncnt + 3) / 4), kThreads, 0, s>>>(base, h->nl_src_of + no, h->nl_vals + no,
-                                                                         h->nl_vals32 + no, ncnt, blen);
-      else
-        k_permute<false><<<grid_for(h, (ncnt + 3) / 4), kThreads, 0, s>>>(base, h->nl_src_of + no,
-                                                                          h->nl_vals + no, nullptr, ncnt, blen);
-    }
   }
-  if (h->n > 0) {
+  if (h->nl_nnz > 0) {
+    const int g = grid_for(h, h->nl_nnz), alpha = h->k / h->n_parts;
     if (h->want_fp32)
-      k_dinv<true><<<grid_for(h, h->n), kThreads, 0, s>>>(buf, h->d_row_off, h->d_slot_off, h->k, h->n, h->dinv,
-                                                          h->dinv32);
+      k_permute_nonlocal<true><<<g, kThreads, 0, s>>>(buf, h->d_slot_off, alpha, h->d_part_nl_off, h->n_parts,
+                                                      h->nl_src_of, h->nl_vals, h->nl_vals32, h->nl_nnz);
     else
-      k_dinv<false><<<grid_for(h, h->n), kThreads, 0, s>>>(buf, h->d_row_off, h->d_slot_off, h->k, h->n, h->dinv,
-                                                           nullptr);
+      k_permute_nonlocal<false><<<g, kThreads, 0, s>>>(buf, h->d_slot_off, alpha, h->d_part_nl_off, h->n_parts,
+                                                       h->nl_src_of, h->nl_vals, nullptr, h->nl_nnz);
   }
   RP_TRY_CUDA(cudaGetLastError());
-  RP_TRY(line_factors(h, s));
-  return fill_sliced(h, s);
+  return line_factors(h, s);
 }
 
 // Buffers, copy stream and events of RP_MEM_HOST_ASYNC, made on first use.
