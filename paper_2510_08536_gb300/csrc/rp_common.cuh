@@ -321,7 +321,6 @@ struct rp_handle {
   int32_t* d_upper = nullptr;
   int32_t* d_iface_row = nullptr;
   int32_t* d_iface_gcol = nullptr;  // global column of each interface entry
-  int64_t* d_out_off = nullptr;     // per-rank offsets of the face-gradient output
 
   // values
   double* staging = nullptr;  // n_slots

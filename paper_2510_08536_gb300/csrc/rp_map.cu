@@ -554,7 +554,7 @@ extern "C" const char* rp_status_str(rp_status s) {
 static void free_handle_memory(rp_handle* h) {
   void* ptrs[] = {h->row_ptr, h->col_idx, h->src_of, h->diag_pos, h->tpos, h->nl_row_ptr, h->nl_col_idx,
                   h->nl_src_of, h->nl_cols, h->nl_gcol, h->d_row_off, h->d_slot_off, h->d_face_off, h->d_iface_off,
-                  h->d_lower, h->d_upper, h->d_iface_row, h->d_iface_gcol, h->d_out_off, h->staging, h->vals,
+                  h->d_lower, h->d_upper, h->d_iface_row, h->d_iface_gcol, h->staging, h->vals,
                   h->vals32, h->nl_vals, h->valsT, h->dinv, h->dinv32, h->dinvT, h->nl_vals32,
                   h->d_part_row_off, h->d_part_nnz_off, h->d_part_nl_off, h->d_part_nlcol_off};
   for (void* p : ptrs)

@@ -1,10 +1,11 @@
-"""The single passes over the matrix: the fused value update, at the shapes where they branch: rows
+"""The single passes over the matrix: the fused value update and the gradients in
+buffer order, at the shapes where they branch: rows
 longer than a warp's shared run, 8-bit and long offset tables, several parts,
 ranks smaller than a warp's run, symmetric storage, and values outside the
 range of the FP32 product of pairs.
 
 The update is a permutation and conversions: every copy is compared bit for
-bit with FP64 arithmetic on the same values.
+bit with FP64 arithmetic on the same values. Gradients: one product (symmetric storage: two and their sum), bit for bit.
 """
 import types
 
@@ -182,4 +183,28 @@ def test_diagonal_reciprocal_and_root():
             np.testing.assert_array_equal(view["scale"].cpu().numpy(), s)
             pos = view["pos"].cpu().numpy()
             np.testing.assert_array_equal(view["vals32s"].cpu().numpy()[pos >= 0], (v * (s * s)).astype(np.float32))
+    h.close()
+
+
+@pytest.mark.parametrize("shape", ["box", "tiny_ranks", "symmetric", "long_rows"])
+def test_gradients(shape):
+    ranks, kw = SHAPES[shape][0](), SHAPES[shape][1]
+    if shape == "tiny_ranks":  # and a rank without cells between others
+        z = np.zeros(0, np.int32)
+        empty = types.SimpleNamespace(n_cells=0, n_faces=0, n_iface=0, lower_addr=z, upper_addr=z, iface_row=z,
+                                      iface_nbr_rank=z, iface_nbr_col=z)
+        ranks = list(ranks) + [empty]
+    sym = kw.get("symmetric", False)
+    h = repart.build_repartition(ranks, **kw)
+    (m,) = O.repartition_map(ranks, 1, sym)
+    rng = np.random.default_rng(5)
+    lam, x = rng.uniform(-1, 1, h.n), rng.uniform(-1, 1, h.n)
+    g = torch.full((h.n_slots,), 7.0, dtype=torch.float64, device=DEV)
+    f = torch.full((sum(len(r.lower_addr) + len(r.iface_row) for r in ranks),), 7.0, dtype=torch.float64, device=DEV)
+    ld, xd = torch.from_numpy(lam).to(DEV), torch.from_numpy(x).to(DEV)
+    repart.entry_grad(h, ld, xd, g)
+    repart.face_grad(h, ld, xd, f)
+    want = O.slot_grad(m.src_of, O.entry_grad(m.row_ptr, m.col_idx, lam, x), h.n_slots)
+    assert np.array_equal(g.cpu().numpy(), want)
+    assert np.array_equal(f.cpu().numpy(), O.face_grad_ldu(ranks, lam, x))
     h.close()
