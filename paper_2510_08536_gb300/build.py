@@ -22,7 +22,7 @@ BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "librepart.so")
 BUILD_CHECK = os.path.join(HERE, "_build_check")
 LIB_CHECK = os.path.join(HERE, "librepart_check.so")
-SOURCES = ["rp_map.cu", "rp_update.cu", "rp_pcg.cu", "rp_resident.cu", "rp_adjoint.cu", "rp_batch.cu", "rp_noalloc.cu", "rp_sliced.cu", "rp_bicgstab.cu"]
+SOURCES = ["rp_map.cu", "rp_update.cu", "rp_pcg.cu", "rp_resident.cu", "rp_resident_bs.cu", "rp_adjoint.cu", "rp_batch.cu", "rp_noalloc.cu", "rp_sliced.cu", "rp_bicgstab.cu"]
 HEADERS = [os.path.join(CSRC, h) for h in sorted(os.listdir(CSRC)) if h.endswith(".cuh")] + [
     os.path.join(ROOT, "include", "repart.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

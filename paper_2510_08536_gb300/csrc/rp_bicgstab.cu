@@ -25,43 +25,9 @@
 // Roofline: FP64-FMA bound on GB300 (one FMA per stored entry per product,
 // two products per iteration, ~14 FP64 instructions per row in B1/B3/B5); the
 // FP32 inner loop is bound by HBM and the products' gathers instead.
-#include "rp_common.cuh"
-#include "rp_spmv.cuh"
+#include "rp_bicgstab.cuh"
 
 namespace rp {
-
-struct BsCtl {
-  double bb, thresh, tol, rr, ss;
-  double rho, rho_old, alpha, omega;
-  double ithresh, inner_tol;  // the inner loop's target: thresh (FP64); inner_tol^2 (r32, r32) (mixed)
-  int32_t iter, max_iter, stop, status, pass, restarts, max_restarts, half, x_zero;
-  int32_t outer, max_outer;
-  unsigned int ticket;
-};
-
-// the vectors and the matrix of one working precision
-template <typename T>
-struct BsVecs {
-  const T* vals;
-  const T* dinv;
-  Parts<T> parts;
-  Sliced<T> sl;
-  T *r, *rhat, *p, *v, *s, *t, *phat, *shat;
-  T* x;  // FP32: the correction d; FP64: unused (the caller's x, through SolveIO)
-};
-
-struct BsArgs {
-  int64_t n;
-  const int32_t* row_ptr;
-  const int32_t* col;
-  BsVecs<double> d;  // FP64 solve; its matrix also serves the residual passes
-  BsVecs<float> f;   // FP32 inner solve (mixed)
-  BsCtl* c;
-  SolveIO* io;
-  double* partials;
-  cudaGraphConditionalHandle inner, outer;
-  int in_graph;
-};
 
 struct BsState {
   double *rhat = nullptr, *s = nullptr, *t = nullptr, *phat = nullptr, *shat = nullptr;
@@ -86,7 +52,8 @@ __device__ __forceinline__ const BsVecs<float>& vecs<float>(const BsArgs& a) {
 }
 
 __global__ void k_bs_setup(BsCtl* c, SolveIO* io, const double* b, double* x, double tol, int x_zero, int max_iter,
-                           int max_restarts, int max_outer, double inner_tol) {
+                           int max_restarts, int max_outer, double inner_tol, unsigned int* sync) {
+  sync[0] = sync[32] = 0u;
   io->b = b;
   io->x = x;
   c->tol = tol;
@@ -155,7 +122,7 @@ __global__ void __launch_bounds__(kThreads) k_bs_res(BsArgs a) {
     }
     c->stop = go ? 0 : 1;
     if (a.in_graph) {
-      cudaGraphSetConditional(a.inner, go ? 1u : 0u);
+      if (a.in_graph > 1) cudaGraphSetConditional(a.inner, go ? 1u : 0u);
       cudaGraphSetConditional(a.outer, go ? 1u : 0u);
     }
   }
@@ -217,7 +184,7 @@ __global__ void __launch_bounds__(kThreads) k_bs_res_mixed(BsArgs a) {
     }
     c->stop = go ? 0 : 1;
     if (a.in_graph) {
-      cudaGraphSetConditional(a.inner, go ? 1u : 0u);
+      if (a.in_graph > 1) cudaGraphSetConditional(a.inner, go ? 1u : 0u);
       cudaGraphSetConditional(a.outer, go ? 1u : 0u);
     }
   }
@@ -679,28 +646,58 @@ void bs_inner(const rp_handle* h, BsLaunch (&k)[5]) {
   k[4] = {(void*)k_bs_xr<T>, b->grid_vec, kThreads, 0};
 }
 
-// mixed: the FP64 residual pass, the FP32 inner loop, then the correction
-rp_status build_bs_graph(rp_handle* h, bool mixed, cudaGraphExec_t* exec) {
+// the resident form of the inner loop, where it takes the system
+struct BsResident {
+  ResidentPlan plan;
+  ResidentBsArgs<double> a64;
+  ResidentBsArgs<float> a32;
+  void* args(bool mixed) { return mixed ? (void*)&a32 : (void*)&a64; }
+};
+BsResident bs_resident(const rp_handle* h, bool mixed, const BsArgs& a, int cap) {
+  BsResident r;
+  r.plan = mixed ? resident_bs_plan<float>(h, a.f) : resident_bs_plan<double>(h, a.d);
+  r.a64 = ResidentBsArgs<double>{a, h->rsync, h->opts.spin_limit, r.plan.rows, cap};
+  r.a32 = ResidentBsArgs<float>{a, h->rsync, h->opts.spin_limit, r.plan.rows, cap};
+  return r;
+}
+
+// while (outer) { residual pass; while (inner) { B1 .. B5 }; [x += d] }, the inner
+// while replaced by the resident kernel where it takes the system (and may be
+// used: a cooperative node is refused under MPS); mixed: FP32 inner loop
+rp_status build_bs_graph(rp_handle* h, bool mixed, bool may_reside, cudaGraphExec_t* exec) {
   cudaGraph_t top = nullptr;
   RP_TRY_CUDA(cudaGraphCreate(&top, 0));
   struct Guard {
     cudaGraph_t g;
     ~Guard() { cudaGraphDestroy(g); }
   } guard{top};
-  cudaGraphConditionalHandle hout, hin;
+  cudaGraphConditionalHandle hout, hin = 0;
   RP_TRY_CUDA(cudaGraphConditionalHandleCreate(&hout, top, 1, cudaGraphCondAssignDefault));
   cudaGraphNode_t wout, nres, win, nk[5];
   cudaGraph_t obody = nullptr, ibody = nullptr;
   RP_TRY(while_node(top, &wout, nullptr, hout, &obody));
-  RP_TRY_CUDA(cudaGraphConditionalHandleCreate(&hin, obody, 0, 0));
-  BsArgs a = bs_args(h, hin, hout, 1);
+  BsArgs a = bs_args(h, 0, hout, 1);
+  BsResident r = bs_resident(h, mixed, a, INT32_MAX);
+  const bool resident = may_reside && r.plan.fn != nullptr;
+  if (!resident) {
+    RP_TRY_CUDA(cudaGraphConditionalHandleCreate(&hin, obody, 0, 0));
+    a.inner = hin;
+    a.in_graph = 2;
+  }
   RP_TRY(node(obody, &nres, nullptr, mixed ? (void*)k_bs_res_mixed : (void*)k_bs_res, h->grid, kThreads, 0, &a));
-  RP_TRY(while_node(obody, &win, &nres, hin, &ibody));
-  BsLaunch k[5];
-  if (mixed) bs_inner<float>(h, k);
-  else bs_inner<double>(h, k);
-  for (int j = 0; j < 5; ++j)
-    RP_TRY(node(ibody, &nk[j], j ? &nk[j - 1] : nullptr, k[j].fn, k[j].grid, k[j].threads, k[j].smem, &a));
+  if (resident) {
+    RP_TRY(node(obody, &win, &nres, r.plan.fn, r.plan.grid, r.plan.threads, r.plan.smem, r.args(mixed)));
+    cudaLaunchAttributeValue coop{};
+    coop.cooperative = 1;
+    RP_TRY_CUDA(cudaGraphKernelNodeSetAttribute(win, cudaLaunchAttributeCooperative, &coop));
+  } else {
+    RP_TRY(while_node(obody, &win, &nres, hin, &ibody));
+    BsLaunch k[5];
+    if (mixed) bs_inner<float>(h, k);
+    else bs_inner<double>(h, k);
+    for (int j = 0; j < 5; ++j)
+      RP_TRY(node(ibody, &nk[j], j ? &nk[j - 1] : nullptr, k[j].fn, k[j].grid, k[j].threads, k[j].smem, &a));
+  }
   if (mixed) {
     cudaGraphNode_t ncor;
     RP_TRY(node(obody, &ncor, &win, (void*)k_bs_correct, h->bs->grid_vec, kThreads, 0, &a));
@@ -713,6 +710,7 @@ rp_status build_bs_graph(rp_handle* h, bool mixed, cudaGraphExec_t* exec) {
 // inside conditional graphs); the control block is read after every kernel group
 rp_status bs_host_loop(rp_handle* h, bool mixed, cudaStream_t s) {
   BsArgs a = bs_args(h, 0, 0, 0);
+  BsResident r = bs_resident(h, mixed, a, 1);  // one iteration a launch
   BsLaunch k[5];
   if (mixed) bs_inner<float>(h, k);
   else bs_inner<double>(h, k);
@@ -726,9 +724,14 @@ rp_status bs_host_loop(rp_handle* h, bool mixed, cudaStream_t s) {
     if (c.stop) break;
     while (!c.stop) {
       void* args[1] = {&a};
-      for (auto& kk : k)
-        RP_TRY_CUDA(cudaLaunchKernel(kk.fn, dim3((unsigned)kk.grid), dim3((unsigned)kk.threads), args,
-                                     (size_t)kk.smem, s));
+      void* rargs[1] = {r.args(mixed)};
+      if (r.plan.fn)
+        RP_TRY_CUDA(cudaLaunchCooperativeKernel(r.plan.fn, dim3((unsigned)r.plan.grid),
+                                                dim3((unsigned)r.plan.threads), rargs, (size_t)r.plan.smem, s));
+      else
+        for (auto& kk : k)
+          RP_TRY_CUDA(cudaLaunchKernel(kk.fn, dim3((unsigned)kk.grid), dim3((unsigned)kk.threads), args,
+                                       (size_t)kk.smem, s));
       RP_TRY_CUDA(cudaMemcpyAsync(&c, h->bs->ctl, sizeof(BsCtl), cudaMemcpyDeviceToHost, s));
       RP_TRY_CUDA(cudaStreamSynchronize(s));
     }
@@ -785,7 +788,11 @@ rp_status bicgstab_run(rp_handle* h, bool mixed, const double* b, double* x, dou
   RP_TRY(ensure_bs(h));
   BsState* bs = h->bs;
   cudaGraphExec_t& graph = mixed ? bs->graph_mixed : bs->graph;
-  if (!graph && !h->opts.host_loop) RP_TRY(build_bs_graph(h, mixed, &graph));
+  if (!graph && !h->opts.host_loop && build_bs_graph(h, mixed, true, &graph) != RP_OK) {
+    cudaGetLastError();
+    graph = nullptr;
+    RP_TRY(build_bs_graph(h, mixed, false, &graph));
+  }
   const double* bd = b;
   double* xd = x;
   if (where == RP_MEM_HOST) {
@@ -799,7 +806,7 @@ rp_status bicgstab_run(rp_handle* h, bool mixed, const double* b, double* x, dou
     xd = h->x_host_stage;
   }
   k_bs_setup<<<1, 1, 0, s>>>(bs->ctl, bs->io, bd, xd, tol, x_is_guess ? 0 : 1, h->opts.max_iter,
-                             h->opts.max_restarts, h->opts.max_outer, h->opts.inner_tol);
+                             h->opts.max_restarts, h->opts.max_outer, h->opts.inner_tol, h->rsync);
   RP_TRY_CUDA(cudaGetLastError());
   if (h->opts.host_loop) RP_TRY(bs_host_loop(h, mixed, s));
   else RP_TRY_CUDA(cudaGraphLaunch(graph, s));

@@ -934,6 +934,7 @@ rp_status check_read_update(CheckWord*, int);
 rp_status check_read_sliced(CheckWord*, int);
 rp_status check_read_pcg(CheckWord*, int);
 rp_status check_read_resident(CheckWord*, int);
+rp_status check_read_resident_bs(CheckWord*, int);
 rp_status check_read_batch(CheckWord*, int);
 rp_status check_read_bicgstab(CheckWord*, int);
 rp_status check_read_adjoint(CheckWord*, int);
@@ -950,7 +951,7 @@ extern "C" rp_status rp_check_violations(uint64_t* count, int32_t* first_site, i
 #ifdef RP_CHECK
   using Reader = rp_status (*)(CheckWord*, int);
   const Reader readers[] = {check_read_map,   check_read_update,   check_read_sliced, check_read_pcg,
-                            check_read_resident, check_read_batch, check_read_bicgstab, check_read_adjoint, check_read_noalloc};
+                            check_read_resident, check_read_resident_bs, check_read_batch, check_read_bicgstab, check_read_adjoint, check_read_noalloc};
   RP_TRY_CUDA(cudaDeviceSynchronize());
   for (Reader r : readers) {
     CheckWord w{};

@@ -3,6 +3,7 @@
 #pragma once
 
 #include "rp_common.cuh"
+#include "rp_resident.cuh"
 
 namespace rp {
 
@@ -37,10 +38,6 @@ struct ResidentArgs {
   int64_t spin;        // probe limit of a barrier wait
   int32_t rows;        // rows of shared memory a block holds (a multiple of 32)
   int32_t cap;
-};
-struct ResidentPlan {
-  void* fn = nullptr;  // nullptr: the streaming kernels run
-  int grid = 0, threads = 0, smem = 0, rows = 0;
 };
 // The launch of the resident kernel for these arguments, or fn = nullptr where
 // the vectors of the iteration do not fit the chip's shared memory.

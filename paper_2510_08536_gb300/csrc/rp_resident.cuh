@@ -1,0 +1,293 @@
+// Building blocks of the resident solver kernels (rp_resident.cu: PCG,
+// rp_bicgstab.cu: BiCGStab): one block an SM owns a contiguous run of 32-row
+// slices, a warp takes every nw-th of them in every phase (so a row's values
+// never leave its lane's hands between phases), and the grid meets at an arrival
+// counter.
+#pragma once
+
+#include <algorithm>
+#include <initializer_list>
+
+#include "rp_common.cuh"
+#include "rp_spmv.cuh"
+
+namespace rp {
+
+// layouts of the product: CSR, sliced, sliced and uniform (4-bit indices, rows
+// of at most 8 entries), and both with several parts
+enum : int { kRsCsr = 0, kRsSliced = 1, kRsU4 = 2, kRsParts = 3, kRsPartsU4 = 4 };
+
+// FP64: 24 warps of up to 80 registers (32 warps of 64 spill the prefetched
+// slice, and the FP64 pipe is the bound anyway)
+template <typename T>
+constexpr int kRsThreads = sizeof(T) == 8 ? 768 : 1024;
+
+// Partial sums of a block's warps, and the flags every thread reads after a grid sum.
+struct RsFlags {
+  double warp[2][32];
+  int stop;  // leave the loop (each kernel's own codes)
+  int bad;   // a wait ran out
+};
+
+// One block's arrival at the grid barrier and its wait for all others (one
+// thread; the block's earlier writes are released, the others' acquired).
+struct RsBarrier {
+  unsigned int* cnt;
+  unsigned int target;
+  int64_t spin;
+  __device__ __forceinline__ bool meet() {
+    target += gridDim.x;
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(cnt) : "memory");
+    for (int64_t i = 0; i < spin; ++i) {
+      unsigned int v;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(cnt) : "memory");
+      if ((int)(v - target) >= 0) return true;
+    }
+    return false;
+  }
+};
+
+// Grid sum of NV values a thread. Warp 0 of every block receives the totals in
+// tot[] (all lanes) and calls fin(tot, ok); then the block goes on together.
+template <int NV, typename T, typename Fin>
+__device__ __forceinline__ void grid_sum(const T (&v)[NV], RsFlags& sh, RsBarrier& bar, double* partials, int lane,
+                                         int w, int nw, Fin&& fin) {
+#pragma unroll
+  for (int i = 0; i < NV; ++i) {
+    const double s = warp_sum(v[i]);
+    if (lane == 0) sh.warp[i][w] = s;
+  }
+  __syncthreads();
+  if (w == 0) {
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      const double s = warp_sum(lane < nw ? sh.warp[i][lane] : 0.0);
+      if (lane == 0) __stcg(partials + (size_t)blockIdx.x * NV + i, s);
+    }
+    int ok = 1;
+    if (lane == 0) ok = bar.meet() ? 1 : 0;
+    ok = __shfl_sync(0xffffffffu, ok, 0);
+    __syncwarp();
+    constexpr int kPer = 5;  // 160 blocks a trip: one trip on 152 SMs
+    double tot[NV];
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      double s = 0.0;
+      for (unsigned int b0 = 0; b0 < gridDim.x; b0 += 32 * kPer) {
+        double x[kPer];
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) {
+          const unsigned int b = b0 + 32 * j + lane;
+          x[j] = b < gridDim.x ? __ldcg(partials + (size_t)b * NV + i) : 0.0;
+        }
+        const double t = warp_sum_n(x);
+        s = b0 ? s + t : t;
+      }
+      tot[i] = s;
+    }
+    if (lane == 0 && !ok) sh.bad = 1;
+    fin(tot);
+  }
+  __syncthreads();
+}
+
+// read-only data of one pass an iteration: not worth a line of L1
+__device__ __forceinline__ float ldg_stream(const float* p) {
+  float v;
+  asm volatile("ld.global.nc.L1::no_allocate.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ double ldg_stream(const double* p) {
+  double v;
+  asm volatile("ld.global.nc.L1::no_allocate.f64 %0, [%1];" : "=d"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ uint32_t ldg_stream(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.global.nc.L1::no_allocate.u32 %0, [%1];" : "=r"(v) : "l"(p));
+  return v;
+}
+
+// A slice of the uniform layout (4-bit indices, at most 8 entries a row) held
+// in registers: loaded one slice ahead, across the grid barriers too, so that
+// only the gathers of p wait on memory.
+template <typename T>
+struct RsSlice {
+  T v[8];
+  uint32_t wd;
+  int32_t tv;
+  int L;
+  __device__ __forceinline__ void load(const Sliced<T>& sl, uint2 d0, uint2 d1, uint32_t info, int lane) {
+    L = (int)((d1.x - d0.x) >> 5);
+    const T* p = sl.vals + d0.x + lane;
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (k < L) v[k] = ldg_stream(p + 32 * k);
+    wd = L > 0 ? ldg_stream(reinterpret_cast<const uint32_t*>(sl.ibuf) + d0.y + lane) : 0u;
+    tv = __ldg(sl.tabs + (info & ~kSliceW4) + (lane & 15));
+  }
+  // the row's products in entry order; x: the gathered vector at the lane's row
+  __device__ __forceinline__ T sum(const T* x, bool valid) const {
+    T g[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (k < L) {
+        const int off = slice_offset<kIdx4>(wd, k, tv, nullptr, 0);
+        g[k] = valid ? x[off] : T(0);
+      }
+    T s = T(0);
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (k < L) s = fma(v[k], g[k], s);
+    return s;
+  }
+};
+
+// The block's slices and their products with a gathered vector.
+template <typename T, int LAY>
+struct RsMatrix {
+  static constexpr bool MP = LAY == kRsParts || LAY == kRsPartsU4, U4 = LAY == kRsU4 || LAY == kRsPartsU4;
+  const Sliced<T>& sl;
+  const Parts<T>& parts;
+  const int32_t* row_ptr;
+  const int32_t* col;
+  const T* vals;
+  int n, s0, cnt, lane, w, nw;
+  uint2* sdesc;     // [cnt + 1]
+  int2* srow;       // MP
+  uint32_t* sinfo;
+  int32_t* snl;     // MP: first non-local entry of the slice's part
+  RsSlice<T> f;     // U4: the slice fetched ahead
+  NlRange fnl;
+
+  // bytes of the records of `per` slices
+  static __host__ __device__ int64_t tail_bytes(bool csr, bool mp, int64_t per) {
+    return csr ? 0 : (per + 1) * 8 + per * 4 + (mp ? per * 12 : 0);
+  }
+  __device__ __forceinline__ RsMatrix(const Sliced<T>& sl_, const Parts<T>& parts_, const int32_t* rp, const int32_t* c,
+                                      const T* v, int n_, unsigned char* tail, int per)
+      : sl(sl_), parts(parts_), row_ptr(rp), col(c), vals(v), n(n_), fnl{0, 0} {
+    lane = threadIdx.x & 31;
+    w = threadIdx.x >> 5;
+    nw = blockDim.x >> 5;
+    const int S = LAY == kRsCsr ? (n + 31) / 32 : (int)sl.n_slices;
+    s0 = (int)((int64_t)S * blockIdx.x / gridDim.x);
+    cnt = (int)((int64_t)S * (blockIdx.x + 1) / gridDim.x) - s0;
+    sdesc = reinterpret_cast<uint2*>(tail);
+    srow = reinterpret_cast<int2*>(sdesc + per + 1);
+    sinfo = reinterpret_cast<uint32_t*>(srow + (MP ? per : 0));
+    snl = reinterpret_cast<int32_t*>(sinfo + per);
+    if (LAY != kRsCsr) {
+      for (int j = threadIdx.x; j <= cnt; j += blockDim.x) sdesc[j] = sl.desc[s0 + j];
+      for (int j = threadIdx.x; j < cnt; j += blockDim.x) {
+        sinfo[j] = sl.tinfo[s0 + j];
+        if (MP) {
+          const int2 r = sl.srow[s0 + j];
+          srow[j] = r;
+          snl[j] = (int32_t)parts.nl_off[r.y >> 6];
+        }
+      }
+    }
+    __syncthreads();
+    if (U4 && w < cnt) fetch(w);
+  }
+  // row of slice j for this lane, or -1
+  __device__ __forceinline__ int row_of(int j) const {
+    if (MP) {
+      const int2 r = srow[j];
+      return lane < (r.y & 63) ? r.x + lane : -1;
+    }
+    const int i = (s0 + j) * kSliceRows + lane;
+    return i < n ? i : -1;
+  }
+  __device__ __forceinline__ void fetch(int j) {
+    f.load(sl, sdesc[j], sdesc[j + 1], sinfo[j], lane);
+    if (MP) {
+      const int i = row_of(j);
+      fnl = i >= 0 ? nonlocal_range<T>(parts, srow[j].y >> 6, i) : NlRange{0, 0};
+    }
+  }
+  // slice j's product with x (a vector this kernel writes); i: row_of(j)
+  __device__ __forceinline__ T product(int j, int i, const T* x) {
+    const bool valid = i >= 0;
+    T sum = T(0);
+    if constexpr (U4) {
+      const RsSlice<T> cur = f;
+      const NlRange nl = fnl;
+      fetch(j + nw < cnt ? j + nw : w);  // the last one fetches the first of the next product
+      int g = 0;
+      T gv = T(0);
+      const int nlo = MP ? snl[j] : 0;
+      if (MP && nl.j0 < nl.j1) {  // the first non-local entry alongside the gathers
+        g = __ldg(parts.nl_gcol + nlo + nl.j0);
+        gv = __ldg(parts.nl_vals + nlo + nl.j0);
+      }
+      sum = cur.sum(x + (valid ? i : 0), valid);
+      if (MP && nl.j0 < nl.j1) {
+        sum = fma(gv, x[g], sum);
+        for (int e = nl.j0 + 1; e < nl.j1; ++e)
+          sum = fma(__ldg(parts.nl_vals + nlo + e), x[__ldg(parts.nl_gcol + nlo + e)], sum);
+      }
+    } else if constexpr (LAY == kRsCsr) {
+      if (valid) sum = row_dot_any<T, true>(parts, row_ptr, col, vals, x, i, n);
+    } else {
+      const int part_id = MP ? srow[j].y >> 6 : 0;
+      NlRange nl{0, 0};
+      if constexpr (MP)
+        if (valid) nl = nonlocal_range<T>(parts, part_id, i);
+      const SliceCk ck = slice_ck<T, MP>(sl, parts, part_id, i, n);
+      const uint2 d0 = sdesc[j], d1 = sdesc[j + 1];
+      sum = slice_sum<T, true>(d0, d1, sinfo[j], sl.vals + d0.x + lane,
+                               reinterpret_cast<const uint32_t*>(sl.ibuf) + d0.y + lane, sl.tabs, x + (valid ? i : 0),
+                               valid, lane, ck);
+      if constexpr (MP)
+        if (valid) sum = nonlocal_sum<T, true>(parts, part_id, nl, x, sum);
+    }
+    return sum;
+  }
+};
+
+// The launch of a resident kernel: fn(layout, vectors kept) returns the instance,
+// or nullptr where there is none; the first of the `vecs` counts that fits.
+struct ResidentPlan {
+  void* fn = nullptr;  // nullptr: the streaming kernels run
+  int grid = 0, threads = 0, smem = 0, rows = 0;
+};
+template <typename T, typename Fn>
+ResidentPlan plan_resident(const rp_handle* h, const Sliced<T>& sl, int64_t n, std::initializer_list<int> vecs, Fn&& fn_of) {
+  ResidentPlan p;
+  int coop = 0, smem_max = 0;
+  if (n == 0) return p;
+  if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, h->device) != cudaSuccess || !coop ||
+      cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device) != cudaSuccess) {
+    cudaGetLastError();
+    return p;
+  }
+#ifdef RP_CHECK
+  const bool u4 = false;  // the checked build tests every slice
+#else
+  const bool u4 = sl.u4 != 0;
+#endif
+  const int lay = sl.n_slices == 0 ? kRsCsr : sl.srow ? (u4 ? kRsPartsU4 : kRsParts) : u4 ? kRsU4 : kRsSliced;
+  const int64_t S = lay == kRsCsr ? (n + 31) / 32 : sl.n_slices;
+  const int grid = (int)std::min<int64_t>(h->num_sms, S);
+  const int64_t per = (S + grid - 1) / grid;  // slices a block at most
+  const int64_t tail = RsMatrix<T, kRsCsr>::tail_bytes(lay == kRsCsr, sl.srow != nullptr, per);
+  for (int v : vecs) {
+    void* fn = fn_of(lay, v);
+    const int64_t need = per * 32 * v * (int64_t)sizeof(T) + tail;
+    const int threads = 32 * (int)std::min<int64_t>(std::max<int64_t>(per, 4), kRsThreads<T> / 32);
+    cudaFuncAttributes at;
+    int nb = 0;
+    // the kernel's own (static) shared memory comes off the block's limit
+    if (cudaFuncGetAttributes(&at, fn) == cudaSuccess && need <= smem_max - (int)at.sharedSizeBytes &&
+        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max - (int)at.sharedSizeBytes) ==
+            cudaSuccess &&
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, threads, (size_t)need) == cudaSuccess && nb >= 1)
+      return ResidentPlan{fn, grid, threads, (int)need, (int)(per * 32)};
+    cudaGetLastError();
+  }
+  return p;
+}
+
+}  // namespace rp

@@ -1,0 +1,270 @@
+// The resident form of the BiCGStab inner loop: one cooperative launch (one
+// block an SM) runs every iteration, with four vectors in shared memory.
+//
+// The streaming form (B1-B5 of rp_bicgstab.cu in a conditional graph) makes five
+// launches and three block elections an iteration and moves every vector through
+// L2 between them. Here block b owns a contiguous run of 32-row slices and keeps
+// p, v, t and r (s in its place between B3 and B5) of those rows in shared
+// memory; phat and shat, which the products gather across blocks, are also
+// written to global memory, and their own rows recomputed as D^-1 p and D^-1 s;
+// rhat, x, D^-1 and the matrix are read from L2. The grid meets five times an
+// iteration:
+//   B1  p = r + beta (p - omega v), phat           | barrier
+//   B2  v = A phat, (rhat, v)                      | sum -> alpha
+//   B3  s = r - alpha v, shat, (s, s)              | sum -> half step
+//   B4  t = A shat, (t, s), (t, t)                 | sum -> omega
+//   B5  x += alpha phat + omega shat, r = s - omega t, (r, r), (rhat, r) | sum -> beta, stop
+// with the fused multiply-adds of B1-B5 row by row. Barriers and sums are those
+// of rp_resident.cuh; every wait is bounded and ends the solve with
+// RP_DEVICE_TIMEOUT.
+//
+// Bound: the latency of the gathers and the five meetings; in FP64 the FP64 pipe
+// (28 instructions a row and iteration).
+#include "rp_bicgstab.cuh"
+
+namespace rp {
+namespace {
+
+// The run's scalars, the same in every block: thread 0's alone (registers of
+// every thread would spill the slice fetched ahead). al, om, be: what all threads
+// read. stop 2: the cap; 3: half step (leaves after its x update).
+template <typename T>
+struct BsShared : RsFlags {
+  T al, om, be;
+  double rho, rho_old, alpha, omega, rr, ss;
+  int iter, status, done;
+};
+
+template <typename T>
+__device__ __forceinline__ const BsVecs<T>& vecs_of(const BsArgs& a) {
+  if constexpr (sizeof(T) == 8) return a.d;
+  else return a.f;
+}
+
+template <typename T, int LAY>
+__global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident_bs(const ResidentBsArgs<T> A) {
+  const BsArgs& a = A.a;
+  const BsVecs<T>& V = vecs_of<T>(a);
+  BsCtl* c = a.c;
+  // written again only after every block has arrived once (or given up)
+  if (c->stop || c->status == RP_DEVICE_TIMEOUT) return;
+  extern __shared__ __align__(128) unsigned char sbuf[];
+  __shared__ BsShared<T> sh;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, nw = blockDim.x >> 5;
+  T* rs = reinterpret_cast<T*>(sbuf);
+  T* ps = rs + A.rows;
+  T* vs = ps + A.rows;
+  T* ts = vs + A.rows;
+  T* xg = V.x;
+  if constexpr (sizeof(T) == 8) xg = a.io->x;
+
+  RsBarrier bar{A.sync, A.sync[32], A.spin};
+  const double thresh = c->ithresh;
+  const int max_iter = c->max_iter;
+  if (tid == 0) {
+    sh.rho = c->rho;
+    sh.rho_old = c->rho_old;
+    sh.alpha = c->alpha;
+    sh.omega = c->omega;
+    sh.rr = c->rr;
+    sh.ss = c->ss;
+    sh.iter = c->iter;
+    sh.status = c->status;
+    sh.bad = sh.stop = sh.done = 0;
+    sh.om = (T)sh.omega;
+    sh.be = (T)((sh.rho / sh.rho_old) * (sh.alpha / sh.omega));
+  }
+  RsMatrix<T, LAY> M(V.sl, V.parts, a.row_ptr, a.col, V.vals, (int)a.n,
+                     reinterpret_cast<unsigned char*>(ts + A.rows), A.rows / 32);
+  const int cnt = M.cnt;
+  for (int j = w; j < cnt; j += nw) {
+    const int i = M.row_of(j), k = j * 32 + lane;
+    if (i < 0) continue;
+    rs[k] = V.r[i];
+    ps[k] = V.p[i];
+    vs[k] = V.v[i];
+  }
+
+  double* part = a.partials;  // two sets of partial sums in turn
+  double* part2 = a.partials + 2 * (size_t)gridDim.x;
+  for (;;) {
+    // B1
+    {
+      const T be = sh.be, om = sh.om;
+      for (int j = w; j < cnt; j += nw) {
+        const int i = M.row_of(j), k = j * 32 + lane;
+        if (i < 0) continue;
+        const T pi = fma(be, fma(-om, vs[k], ps[k]), rs[k]);
+        ps[k] = pi;
+        V.phat[i] = __ldg(V.dinv + i) * pi;
+      }
+      __syncthreads();
+      if (tid == 0 && !bar.meet()) sh.bad = 1;
+      __syncthreads();
+      if (sh.bad) break;
+    }
+    // B2
+    {
+      T acc = T(0);
+      for (int j = w; j < cnt; j += nw) {
+        const int i = M.row_of(j), k = j * 32 + lane;
+        const T rh = i >= 0 ? __ldg(V.rhat + i) : T(0);
+        const T y = M.product(j, i, V.phat);
+        if (i >= 0) {
+          vs[k] = y;
+          acc = fma(rh, y, acc);
+        }
+      }
+      const T v[1] = {acc};
+      grid_sum<1>(v, sh, bar, part, lane, w, nw, [&](const double (&tot)[1]) {
+        if (lane != 0) return;
+        if (tot[0] == 0.0 || !isfinite(tot[0])) {
+          sh.status = RP_BREAKDOWN;
+          sh.stop = 1;
+        } else {
+          sh.alpha = sh.rho / tot[0];
+          sh.al = (T)sh.alpha;
+        }
+      });
+    }
+    if (sh.bad || sh.stop) break;
+    const T al = sh.al;
+    // B3
+    {
+      T acc = T(0);
+      for (int j = w; j < cnt; j += nw) {
+        const int i = M.row_of(j), k = j * 32 + lane;
+        if (i < 0) continue;
+        const T si = fma(-al, vs[k], rs[k]);
+        rs[k] = si;
+        V.shat[i] = __ldg(V.dinv + i) * si;
+        acc = fma(si, si, acc);
+      }
+      const T v[1] = {acc};
+      grid_sum<1>(v, sh, bar, part2, lane, w, nw, [&](const double (&tot)[1]) {
+        if (lane != 0) return;
+        sh.ss = tot[0];
+        if (tot[0] <= thresh) sh.stop = 3;
+      });
+    }
+    if (sh.bad) break;
+    if (sh.stop == 3) {
+      for (int j = w; j < cnt; j += nw) {
+        const int i = M.row_of(j), k = j * 32 + lane;
+        if (i >= 0) xg[i] = fma(al, __ldg(V.dinv + i) * ps[k], xg[i]);
+      }
+      if (tid == 0) {
+        ++sh.iter;
+        sh.rr = sh.ss;
+      }
+      break;
+    }
+    // B4
+    {
+      T ats = T(0), att = T(0);
+      for (int j = w; j < cnt; j += nw) {
+        const int i = M.row_of(j), k = j * 32 + lane;
+        const T y = M.product(j, i, V.shat);
+        if (i >= 0) {
+          ts[k] = y;
+          ats = fma(y, rs[k], ats);
+          att = fma(y, y, att);
+        }
+      }
+      const T v[2] = {ats, att};
+      grid_sum<2>(v, sh, bar, part, lane, w, nw, [&](const double (&tot)[2]) {
+        if (lane != 0) return;
+        const double om = tot[0] / tot[1];
+        if (!(tot[1] > 0.0) || !isfinite(om)) {
+          sh.status = RP_BREAKDOWN;
+          sh.stop = 1;
+        } else {
+          sh.omega = om;
+          sh.om = (T)om;
+        }
+      });
+    }
+    if (sh.bad || sh.stop) break;
+    // B5
+    {
+      const T om = sh.om;
+      T arr = T(0), arh = T(0);
+      for (int j = w; j < cnt; j += nw) {
+        const int i = M.row_of(j), k = j * 32 + lane;
+        if (i < 0) continue;
+        const T d = __ldg(V.dinv + i), si = rs[k];
+        xg[i] = fma(om, d * si, fma(al, d * ps[k], xg[i]));
+        const T ri = fma(-om, ts[k], si);
+        rs[k] = ri;
+        arr = fma(ri, ri, arr);
+        arh = fma(__ldg(V.rhat + i), ri, arh);
+      }
+      const T v[2] = {arr, arh};
+      grid_sum<2>(v, sh, bar, part2, lane, w, nw, [&](const double (&tot)[2]) {
+        if (lane != 0) return;
+        sh.rr = tot[0];
+        ++sh.iter;
+        int stop = ++sh.done >= A.cap ? 2 : 0;  // at the cap the next launch goes on
+        if (tot[0] <= thresh || sh.iter >= max_iter) {
+          stop = 1;
+        } else if (sh.omega == 0.0 || tot[1] == 0.0 || !isfinite(tot[1])) {
+          sh.status = RP_BREAKDOWN;
+          stop = 1;
+        } else {
+          sh.rho_old = sh.rho;
+          sh.rho = tot[1];
+          sh.be = (T)((sh.rho / sh.rho_old) * (sh.alpha / sh.omega));
+        }
+        sh.stop = stop;
+      });
+    }
+    if (sh.bad || sh.stop) break;
+  }
+  if (sh.stop == 2) {  // the state back to memory for the next launch
+    for (int j = w; j < cnt; j += nw) {
+      const int i = M.row_of(j), k = j * 32 + lane;
+      if (i < 0) continue;
+      V.r[i] = rs[k];
+      V.p[i] = ps[k];
+      V.v[i] = vs[k];
+    }
+  }
+  if (blockIdx.x == 0 && tid == 0) {
+    A.sync[32] = bar.target;
+    c->iter = sh.iter;
+    c->rho = sh.rho;
+    c->rho_old = sh.rho_old;
+    c->alpha = sh.alpha;
+    c->omega = sh.omega;
+    c->rr = sh.rr;
+    c->ss = sh.ss;
+    c->half = sh.stop == 3;
+    atomicMax(&c->status, sh.status);  // a timeout, the largest status, stands whoever writes last
+    c->stop = sh.stop == 2 ? 0 : 1;
+  }
+  if (tid == 0 && sh.bad) {  // any block may have given up
+    atomicMax(&c->status, (int)RP_DEVICE_TIMEOUT);
+    c->stop = 1;
+  }
+}
+
+}  // namespace
+
+RP_CHECK_TU(resident_bs)
+
+template <typename T>
+ResidentPlan resident_bs_plan(const rp_handle* h, const BsVecs<T>& v) {
+  return plan_resident<T>(h, v.sl, h->n, {4}, [](int lay, int) -> void* {
+    switch (lay) {
+      case kRsU4: return (void*)k_resident_bs<T, kRsU4>;
+      case kRsSliced: return (void*)k_resident_bs<T, kRsSliced>;
+      case kRsParts: return (void*)k_resident_bs<T, kRsParts>;
+      case kRsPartsU4: return (void*)k_resident_bs<T, kRsPartsU4>;
+      default: return (void*)k_resident_bs<T, kRsCsr>;
+    }
+  });
+}
+template ResidentPlan resident_bs_plan<double>(const rp_handle*, const BsVecs<double>&);
+template ResidentPlan resident_bs_plan<float>(const rp_handle*, const BsVecs<float>&);
+
+}  // namespace rp

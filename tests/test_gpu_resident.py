@@ -1,4 +1,4 @@
-"""The resident form of the PCG iteration (one cooperative launch an inner run).
+"""The resident forms of the PCG and BiCGStab iterations (one cooperative launch an inner run).
 
 Against the oracle at the shapes where its split over the SMs changes: fewer
 slices than SMs, ragged last slices, fewer warps than a full block, the
@@ -17,7 +17,8 @@ import pytest
 import torch
 
 from oracle import pcg_omp
-from paper_2510_08536_gb300 import build, repart
+from oracle import repart_oracle as O
+from paper_2510_08536_gb300 import build, repart, synth
 from gpu_util import Case
 
 pytestmark = pytest.mark.gpu
@@ -65,6 +66,41 @@ def test_resident_solves(dims, ranks, kw):
             assert np.linalg.norm(xs - ref.x) <= 1e-7 * np.linalg.norm(ref.x)
             assert abs(info["iterations"] - ref.iterations) <= 2
     h.close()
+
+
+@pytest.mark.parametrize("dims,ranks,kw", [
+    ((1, 1, 31), (1, 1, 1), {}),
+    ((3, 11, 1), (1, 1, 1), {}),
+    ((17, 17, 17), (2, 2, 2), {}),
+    ((19, 23, 29), (2, 3, 2), {"n_parts": 3}),
+    ((37, 29, 31), (2, 2, 2), {"layout": repart.RP_LAYOUT_CSR}),
+    ((109, 103, 101), (2, 2, 2), {}),         # FP64: streaming
+])
+def test_resident_bicgstab(dims, ranks, kw):
+    mesh = synth.box_mesh(*dims, *ranks)
+    stg = synth.momentum_staging(mesh, 0.5, 100)
+    (m,) = O.repartition_map(mesh.ranks, 1)
+    vals = O.update_values(m.src_of, stg)
+    A = O.csr_matrix(m.row_ptr, m.col_idx, vals)
+    b = synth.uniform_vector(mesh, 0)
+    ref = O.bicgstab(A, O.jacobi_inverse(m.row_ptr, m.col_idx, vals, m.diag_pos), b, tol=1e-9)
+    hs = [repart.build_repartition(mesh.ranks, host_loop=k, **kw) for k in (0, 1)]
+    for precision in ("fp64", "mixed"):
+        out = []
+        for h in hs:
+            repart.update_values_packed(h, _t(stg))
+            x = torch.zeros(h.n, dtype=torch.float64, device=DEV)
+            info = repart.solve_bicgstab(h, _t(b), x, tol=1e-9, precision=precision)
+            assert info["status"] == 0, (precision, info)
+            out.append((x, info))
+        assert torch.equal(out[0][0], out[1][0]) and out[0][1] == out[1][1]  # one launch or one an iteration
+        xs = out[0][0].cpu().numpy()
+        assert np.linalg.norm(b - A @ xs) <= 1e-9 * np.linalg.norm(b), precision
+        assert np.linalg.norm(xs - ref.x) <= 1e-7 * np.linalg.norm(ref.x)
+        if precision == "fp64":
+            assert abs(out[0][1]["iterations"] - ref.iterations) <= max(3, ref.iterations // 10)
+    for h in hs:
+        h.close()
 
 
 def test_concurrent_solves():
