@@ -53,7 +53,8 @@ __device__ __forceinline__ const BsVecs<float>& vecs<float>(const BsArgs& a) {
 
 __global__ void k_bs_setup(BsCtl* c, SolveIO* io, const double* b, double* x, double tol, int x_zero, int max_iter,
                            int max_restarts, int max_outer, double inner_tol, unsigned int* sync) {
-  sync[0] = sync[32] = 0u;
+  rs_reset(sync);
+  if (threadIdx.x != 0) return;
   io->b = b;
   io->x = x;
   c->tol = tol;
@@ -805,7 +806,7 @@ rp_status bicgstab_run(rp_handle* h, bool mixed, const double* b, double* x, dou
     bd = h->b_host_stage;
     xd = h->x_host_stage;
   }
-  k_bs_setup<<<1, 1, 0, s>>>(bs->ctl, bs->io, bd, xd, tol, x_is_guess ? 0 : 1, h->opts.max_iter,
+  k_bs_setup<<<1, kRsSync, 0, s>>>(bs->ctl, bs->io, bd, xd, tol, x_is_guess ? 0 : 1, h->opts.max_iter,
                              h->opts.max_restarts, h->opts.max_outer, h->opts.inner_tol, h->rsync);
   RP_TRY_CUDA(cudaGetLastError());
   if (h->opts.host_loop) RP_TRY(bs_host_loop(h, mixed, s));

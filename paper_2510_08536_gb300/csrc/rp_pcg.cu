@@ -783,6 +783,8 @@ __global__ void __launch_bounds__(kThreads) k_correct(CorrectArgs a) {
 
 __global__ void k_setup(Ctl* c, SolveIO* io, const double* b, double* x, double tol, double inner_tol, int x_zero,
                         int max_iter, int max_restarts, int max_outer, double ru_delta, unsigned int* sync) {
+  rs_reset(sync);
+  if (threadIdx.x != 0) return;
   io->b = b;
   io->x = x;
   c->tol = tol;
@@ -803,7 +805,6 @@ __global__ void k_setup(Ctl* c, SolveIO* io, const double* b, double* x, double 
   c->skip_correct = 1;
   c->alpha = c->beta = 0.0;
   c->ticket = 0u;
-  sync[0] = sync[32] = 0u;
 }
 
 // y = A x and, optionally, x.y
@@ -1119,7 +1120,7 @@ rp_status ensure_solver_buffers(rp_handle* h) {
   RP_TRY(dalloc(&h->ctl, 1));
   RP_TRY(dalloc(&h->io, 1));
   RP_TRY(dalloc(&h->ticket, 4));
-  RP_TRY(dalloc(&h->rsync, 64));
+  RP_TRY(dalloc(&h->rsync, kRsSync));
   RP_TRY_CUDA(cudaMemset(h->ctl, 0, sizeof(Ctl)));
   RP_TRY_CUDA(cudaMemset(h->ticket, 0, 4 * sizeof(unsigned int)));
   return RP_OK;
@@ -1148,7 +1149,7 @@ void free_solver(rp_handle* h) {
 
 rp_status launch_solve(rp_handle* h, cudaGraphExec_t exec, const double* b, double* x, double tol, bool x_zero,
                        int max_iter, rp_solve_info* info, cudaStream_t s) {
-  k_setup<<<1, 1, 0, s>>>(h->ctl, h->io, b, x, tol, h->opts.inner_tol, x_zero ? 1 : 0, max_iter,
+  k_setup<<<1, kRsSync, 0, s>>>(h->ctl, h->io, b, x, tol, h->opts.inner_tol, x_zero ? 1 : 0, max_iter,
                           h->opts.max_restarts, h->opts.max_outer, h->opts.ru_delta, h->rsync);
   RP_TRY_CUDA(cudaGetLastError());
   RP_TRY_CUDA(cudaGraphLaunch(exec, s));
@@ -1230,7 +1231,7 @@ rp_status solve_common(rp_handle* h, int mode, const double* vals, const double*
     xd = h->x_host_stage;
   }
   if (h->opts.host_loop) {
-    k_setup<<<1, 1, 0, s>>>(h->ctl, h->io, bd, xd, tol, h->opts.inner_tol, x_is_guess ? 0 : 1, h->opts.max_iter,
+    k_setup<<<1, kRsSync, 0, s>>>(h->ctl, h->io, bd, xd, tol, h->opts.inner_tol, x_is_guess ? 0 : 1, h->opts.max_iter,
                             h->opts.max_restarts, h->opts.max_outer, h->opts.ru_delta, h->rsync);
     RP_TRY(host_loop_solve(h, mode, vals, dinv, s));
   } else {
@@ -1381,7 +1382,7 @@ extern "C" rp_status rp_profile_iteration(rp_handle* h, const double* b, int32_t
   }
   RP_TRY(dalloc(&h->x_host_stage, h->n + 64));
   // a fresh CG run from x = 0 that never meets its tolerance (tol = 0)
-  k_setup<<<1, 1, 0, s>>>(h->ctl, h->io, b, h->x_host_stage, 0.0, 0.0, 1, iters + 2, 0, 1, 0.0, h->rsync);
+  k_setup<<<1, kRsSync, 0, s>>>(h->ctl, h->io, b, h->x_host_stage, 0.0, 0.0, 1, iters + 2, 0, 1, 0.0, h->rsync);
   SolveSet k = solve_set(h, mixed ? 1 : 0, h->vals, h->dinv, 0, 0, 0);
   RP_TRY(launch1(k.res, h->grid, kThreads, 0, &k.ra, s));
   std::vector<cudaEvent_t> ev(3 * iters + 1, nullptr);

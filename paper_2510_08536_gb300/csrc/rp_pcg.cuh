@@ -34,7 +34,7 @@ struct IterArgs {
 template <typename T>
 struct ResidentArgs {
   IterArgs<T> it;
-  unsigned int* sync;  // arrivals at the grid barrier, cleared before each solve; [32]: its base of the next launch
+  unsigned int* sync;  // memory of the grid barrier and sums, cleared before each solve
   int64_t spin;        // probe limit of a barrier wait
   int32_t rows;        // rows of shared memory a block holds (a multiple of 32)
   int32_t cap;

@@ -66,18 +66,8 @@ __device__ __forceinline__ long long fix_term(T v, int emax) {
   return F::neg(v) ? -(long long)m : (long long)m;
 }
 
-// h 2^26 + l (0 <= l < 2^26, |h| < 2^44) times 2^q, rounded to nearest even
-__device__ __forceinline__ double fix_value(long long h, uint32_t l, int q) {
-  long long t;
-  if (h < (1ll << 36) && h >= -(1ll << 36)) {
-    t = (long long)((uint64_t)h << 26 | l);
-  } else {  // eight bits lower, the dropped ones kept as a sticky bit
-    t = (long long)((uint64_t)h << 18 | (l >> 8) | ((l & 255u) ? 1u : 0u));
-    q += 8;
-  }
-  if (t == 0) return 0.0;
-  const bool neg = t < 0;
-  uint64_t m = neg ? 0ull - (uint64_t)t : (uint64_t)t;
+// +-m 2^q rounded to nearest even (m: its low bit may be a sticky one)
+__device__ __forceinline__ double fix_round(bool neg, uint64_t m, int q) {
   const int lz = __clzll((long long)m);
   const int e = q + 63 - lz + 1023;  // biased exponent of the leading bit
   if (e < 1 || e > 2046) {           // subnormal or overflowing: rounded by the library
@@ -90,6 +80,36 @@ __device__ __forceinline__ double fix_value(long long h, uint32_t l, int q) {
   r += (rem > 0x400u || (rem == 0x400u && (r & 1u))) ? 1u : 0u;
   r += (uint64_t)(e - 1) << 52;  // the leading bit carries into the exponent
   return __longlong_as_double((long long)(r | (neg ? 1ull << 63 : 0ull)));
+}
+
+// h 2^26 + l (0 <= l < 2^26, |h| < 2^44) times 2^q, rounded to nearest even
+__device__ __forceinline__ double fix_value(long long h, uint32_t l, int q) {
+  long long t;
+  if (h < (1ll << 36) && h >= -(1ll << 36)) {
+    t = (long long)((uint64_t)h << 26 | l);
+  } else {  // eight bits lower, the dropped ones kept as a sticky bit
+    t = (long long)((uint64_t)h << 18 | (l >> 8) | ((l & 255u) ? 1u : 0u));
+    q += 8;
+  }
+  if (t == 0) return 0.0;
+  const bool neg = t < 0;
+  return fix_round(neg, neg ? 0ull - (uint64_t)t : (uint64_t)t, q);
+}
+
+// (h 2^64 + l) 2^q, two's complement, rounded to nearest even
+__device__ __forceinline__ double fix_value128(long long h, uint64_t l, int q) {
+  const bool neg = h < 0;
+  if (neg) {
+    l = 0ull - l;
+    h = ~h + (l == 0ull ? 1 : 0);
+  }
+  if (h != 0) {
+    const int s = 64 - __clzll(h);  // bits to drop, 1 .. 63
+    const uint64_t sticky = (l << (64 - s)) != 0ull ? 1u : 0u;
+    l = (uint64_t)h << (64 - s) | l >> s | sticky;
+    q += s;
+  }
+  return l == 0ull ? 0.0 : fix_round(neg, l, q);
 }
 
 // Sum of N values of every lane of a warp; all lanes call it and get the sum.
@@ -124,5 +144,47 @@ __device__ __forceinline__ double warp_sum(T v) {
   const T a[1] = {v};
   return warp_sum_n<T, 1>(a);
 }
+
+// ---- Sums in a unit known beforehand (the grid sums of the resident kernels).
+//
+// With the unit agreed, values are turned into integers of 100 bits once, and
+// every level above adds integers: five digits of 20 bits a warp by redux.sync
+// (a block of 32 warps keeps them below 2^30), no exponent search, no conversion
+// back between the levels.
+constexpr int kFixDigits = 5;
+
+// v as an integer multiple of 2^qt in five 20-bit digits (two's complement, the
+// top one signed), rounded to nearest. False where |v| reaches 2^89 units, or v is
+// an infinity or NaN.
+template <typename T>
+__device__ __forceinline__ bool fix_digits(T v, int qt, uint32_t (&u)[kFixDigits]) {
+  using F = FixOf<T>;
+  const int e = F::expo(v);
+  const uint64_t m = F::mant(v, e);
+  const int d = (e > 1 ? e : 1) - F::kBias - F::kMant - qt;
+  const bool ok = e != F::kSpecial && (d <= 88 - F::kMant && d < 64);
+  uint64_t lo, hi = 0ull;
+  if (d >= 0) {
+    lo = m << (d & 63);
+    if (d & 63) hi = m >> (64 - (d & 63));
+  } else {
+    lo = d > -64 ? (m + (1ull << (-d - 1))) >> -d : 0ull;
+  }
+  if (F::neg(v)) {
+    lo = 0ull - lo;
+    hi = ~hi + (lo == 0ull ? 1u : 0u);
+  }
+  u[0] = (uint32_t)lo & 0xfffffu;
+  u[1] = (uint32_t)(lo >> 20) & 0xfffffu;
+  u[2] = (uint32_t)(lo >> 40) & 0xfffffu;
+  u[3] = (uint32_t)((lo >> 60) | (hi << 4)) & 0xfffffu;
+  u[4] = (uint32_t)(hi >> 16);
+  if (!ok) u[0] = u[1] = u[2] = u[3] = u[4] = 0u;
+  return ok;
+}
+
+// The unit for a sum that was t last time: t is between 2^79 and 2^80 of it.
+__device__ __forceinline__ int fix_unit(double t) { return ((__double2hiint(t) >> 20) & 0x7ff) - 1023 - 79; }
+constexpr int kFixNoUnit = INT32_MAX;
 
 }  // namespace rp

@@ -40,7 +40,15 @@ struct RsShared : RsFlags {
   T alpha, beta;
   double pq, rz, rr;
   int iter, iter_total, status, done;
+  int unit[3];  // of (p, q), (r, z) and (r, r)
 };
+
+// a / b in T, for the finite a, b > 0 of an iteration that goes on without the FP64 pipe
+template <typename T>
+__device__ __forceinline__ T ratio(double a, double b) {
+  if constexpr (sizeof(T) == 8) return quot_rn(a, b);
+  else return f32_rn(quot_rn(a, b));
+}
 
 // LAY: layout of the product; SCALED: the system S A S (z = r); ALL: r, x, p
 // and q in shared memory, else r and q.
@@ -60,7 +68,8 @@ __global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident(const ResidentArg
   T* xg = a.xd;
   if (xg == nullptr) xg = reinterpret_cast<T*>(a.io->x);
 
-  RsBarrier bar{A.sync, A.sync[32], A.spin};
+  RsBarrier bar{A.sync + kRsCount, A.sync[kRsBase], A.spin};
+  int set = (int)A.sync[kRsSet];  // accumulators of this iteration's sums
   const double thresh = a.xd ? c->inner_thresh : c->thresh;
   const int max_iter = c->max_iter;
   if (tid == 0) {
@@ -70,7 +79,8 @@ __global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident(const ResidentArg
     sh.iter = c->iter;
     sh.iter_total = c->iter_total;
     sh.status = c->status;
-    sh.bad = sh.stop = sh.done = 0;
+    sh.bad = sh.stop = sh.done = sh.over = 0;
+    for (int k = 0; k < 3; ++k) sh.unit[k] = (int)A.sync[kRsUnit + k];
   }
   RsMatrix<T, LAY> M(a.sl, a.parts, a.row_ptr, a.col, a.vals, (int)a.n,
                      reinterpret_cast<unsigned char*>(rs + (ALL ? 4 : 2) * (size_t)A.rows), A.rows / 32);
@@ -99,10 +109,10 @@ __global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident(const ResidentArg
     }
     {
       const T v[1] = {acc};
-      grid_sum<1>(v, sh, bar, part, lane, w, nw, [&](const double (&tot)[1]) {
+      grid_sum_unit<1>(v, sh.unit, rs_words(A.sync, set, 0), sh, bar, part, lane, w, nw, [&](const double (&tot)[1]) {
         if (lane != 0) return;
         sh.pq = tot[0];
-        sh.alpha = (T)(sh.rz / tot[0]);
+        sh.alpha = ratio<T>(sh.rz, tot[0]);
         if (!(tot[0] > 0.0) || !isfinite(tot[0])) {
           sh.status = RP_BREAKDOWN;
           sh.stop = 2;
@@ -110,6 +120,10 @@ __global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident(const ResidentArg
       });
     }
     if (sh.bad || sh.stop) break;
+    // every block has left the sums of the iteration before: their accumulators are
+    // cleared for the one after the next (seen by all behind barrier C)
+    const int free_set = set == 0 ? 2 : set - 1;
+    if (blockIdx.x == 0 && tid < 8) rs_words(A.sync, free_set, 0)[tid] = 0ull;
     // B: r -= alpha q, z = D^-1 r (kept in q's place), x += alpha p, (r, z), (r, r)
     const T alpha = sh.alpha;
     T rza = T(0), rra = T(0);
@@ -132,7 +146,7 @@ __global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident(const ResidentArg
       T v[NV];
       v[NV - 1] = rra;
       if constexpr (!SCALED) v[0] = rza;
-      grid_sum<NV>(v, sh, bar, part2, lane, w, nw, [&](const double (&tot)[NV]) {
+      grid_sum_unit<NV>(v, sh.unit + 1, rs_words(A.sync, set, 1), sh, bar, part2, lane, w, nw, [&](const double (&tot)[NV]) {
         if (lane != 0) return;
         sh.rr = tot[NV - 1];
         ++sh.iter;
@@ -144,11 +158,12 @@ __global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident(const ResidentArg
           sh.stop = 1;
           sh.status = RP_BREAKDOWN;
         } else {
-          sh.beta = (T)(tot[0] / sh.rz);
+          sh.beta = ratio<T>(tot[0], sh.rz);
           sh.rz = tot[0];
         }
       });
     }
+    set = set == 2 ? 0 : set + 1;
     if (sh.bad || sh.stop) break;
     // C: p = z + beta p
     const T beta = sh.beta;
@@ -175,7 +190,9 @@ __global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident(const ResidentArg
     if (ALL) xg[i] = xs[k];
   }
   if (blockIdx.x == 0 && tid == 0) {
-    A.sync[32] = bar.target;
+    A.sync[kRsBase] = bar.target;
+    A.sync[kRsSet] = (unsigned int)set;
+    for (int k = 0; k < 3; ++k) A.sync[kRsUnit + k] = (unsigned int)sh.unit[k];
     c->iter = sh.iter;
     c->iter_total = sh.iter_total;
     c->pq = sh.pq;

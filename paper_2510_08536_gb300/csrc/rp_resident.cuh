@@ -10,6 +10,7 @@
 
 #include "rp_common.cuh"
 #include "rp_spmv.cuh"
+#include "rp_values.cuh"
 
 namespace rp {
 
@@ -24,10 +25,27 @@ constexpr int kRsThreads = sizeof(T) == 8 ? 768 : 1024;
 
 // Partial sums of a block's warps, and the flags every thread reads after a grid sum.
 struct RsFlags {
-  double warp[2][32];
+  union {
+    double warp[2][32];
+    uint32_t digit[2][kFixDigits][32];
+  };
   int stop;  // leave the loop (each kernel's own codes)
   int bad;   // a wait ran out
+  int over;  // a value past the range of its sum's unit
+  int again; // the sum has to be taken from the blocks' own sums
 };
+
+// Memory of the grid barrier and sums (rp_handle::rsync), cleared before each
+// solve: the arrival counter, its base of the next launch, the set of accumulators
+// that is next and the units of the sums; three sets of 4 words for each of two sums.
+constexpr int kRsCount = 0, kRsBase = 32, kRsSet = 33, kRsUnit = 34, kRsWords = 64, kRsSync = 128;
+__device__ __forceinline__ void rs_reset(unsigned int* sync) {
+  for (int k = threadIdx.x; k < kRsSync; k += blockDim.x)
+    sync[k] = k >= kRsUnit && k < kRsWords ? (unsigned int)kFixNoUnit : 0u;
+}
+__device__ __forceinline__ unsigned long long* rs_words(unsigned int* sync, int set, int sum) {
+  return reinterpret_cast<unsigned long long*>(sync + kRsWords) + set * 8 + sum * 4;
+}
 
 // One block's arrival at the grid barrier and its wait for all others (one
 // thread; the block's earlier writes are released, the others' acquired).
@@ -47,45 +65,161 @@ struct RsBarrier {
   }
 };
 
-// Grid sum of NV values a thread. Warp 0 of every block receives the totals in
-// tot[] (all lanes) and calls fin(tot, ok); then the block goes on together.
-template <int NV, typename T, typename Fin>
-__device__ __forceinline__ void grid_sum(const T (&v)[NV], RsFlags& sh, RsBarrier& bar, double* partials, int lane,
-                                         int w, int nw, Fin&& fin) {
+// Warp 0 of every block: the block's sums published, the grid met, all blocks'
+// sums added in block order (so all blocks hold the same totals).
+template <int NV>
+__device__ __forceinline__ bool grid_total(RsFlags& sh, RsBarrier& bar, double* partials, int lane, int nw,
+                                           double (&tot)[NV]) {
+#pragma unroll
+  for (int i = 0; i < NV; ++i) {
+    const double s = warp_sum(lane < nw ? sh.warp[i][lane] : 0.0);
+    if (lane == 0) __stcg(partials + (size_t)blockIdx.x * NV + i, s);
+  }
+  int ok = 1;
+  if (lane == 0) ok = bar.meet() ? 1 : 0;
+  ok = __shfl_sync(0xffffffffu, ok, 0);
+  __syncwarp();
+  constexpr int kPer = 5;  // 160 blocks a trip: one trip on 152 SMs
+#pragma unroll
+  for (int i = 0; i < NV; ++i) {
+    double s = 0.0;
+    for (unsigned int b0 = 0; b0 < gridDim.x; b0 += 32 * kPer) {
+      double x[kPer];
+#pragma unroll
+      for (int j = 0; j < kPer; ++j) {
+        const unsigned int b = b0 + 32 * j + lane;
+        x[j] = b < gridDim.x ? __ldcg(partials + (size_t)b * NV + i) : 0.0;
+      }
+      const double t = warp_sum_n(x);
+      s = b0 ? s + t : t;
+    }
+    tot[i] = s;
+  }
+  return ok != 0;
+}
+template <int NV, typename T>
+__device__ __forceinline__ void warp_sums(const T (&v)[NV], RsFlags& sh, int lane, int w) {
 #pragma unroll
   for (int i = 0; i < NV; ++i) {
     const double s = warp_sum(v[i]);
     if (lane == 0) sh.warp[i][w] = s;
   }
+}
+
+// Grid sum of NV values a thread. Warp 0 of every block receives the totals in
+// tot[] (all lanes) and calls fin(tot); then the block goes on together.
+template <int NV, typename T, typename Fin>
+__device__ __forceinline__ void grid_sum(const T (&v)[NV], RsFlags& sh, RsBarrier& bar, double* partials, int lane,
+                                         int w, int nw, Fin&& fin) {
+  warp_sums(v, sh, lane, w);
   __syncthreads();
   if (w == 0) {
-#pragma unroll
-    for (int i = 0; i < NV; ++i) {
-      const double s = warp_sum(lane < nw ? sh.warp[i][lane] : 0.0);
-      if (lane == 0) __stcg(partials + (size_t)blockIdx.x * NV + i, s);
-    }
-    int ok = 1;
-    if (lane == 0) ok = bar.meet() ? 1 : 0;
-    ok = __shfl_sync(0xffffffffu, ok, 0);
-    __syncwarp();
-    constexpr int kPer = 5;  // 160 blocks a trip: one trip on 152 SMs
     double tot[NV];
+    const bool ok = grid_total<NV>(sh, bar, partials, lane, nw, tot);
+    if (lane == 0 && !ok) sh.bad = 1;
+    fin(tot);
+  }
+  __syncthreads();
+}
+
+// The same for sums that change little from one iteration to the next: unit[i],
+// kept over the iterations, is 2^-80 of the last total. The threads' values
+// become integers in that unit (fix_digits), the warps and the block add
+// integers, and the block adds its sum, rounded to 2^-66 of the last total, to two
+// 64-bit words in L2: 40 low bits with the count of values out of range above
+// them, 48 high bits, and the count of arrivals in the top byte of both. A word
+// whose count is complete needs no fence and no second read: one exchange instead
+// of a release, an arrival, its poll, and 152 loads and their sum. Rounding: at most
+// 2^17 halves of 2^-80 and 152 halves of 2^-66 of the last total; the sum is taken
+// again the long way where a value reaches 2^9 of the last total, a block 2^20, or
+// the total falls below 2^-7 of it (and the first time): all blocks see the same
+// words and decide alike.
+// (32^3: 7.1k cycles a sum the long way, 600 and 740 of them the two warp sums, 2600
+// the meeting, 1800 the loads and their sum, 770 the division.)
+template <int NV, typename T, typename Fin>
+__device__ __forceinline__ void grid_sum_unit(const T (&v)[NV], int* unit, unsigned long long* words, RsFlags& sh,
+                                              RsBarrier& bar, double* partials, int lane, int w, int nw, Fin&& fin) {
+  bool quick = gridDim.x < 256;
+#pragma unroll
+  for (int i = 0; i < NV; ++i) quick = quick && unit[i] != kFixNoUnit;
+  if (quick) {
+    bool over = false;
 #pragma unroll
     for (int i = 0; i < NV; ++i) {
-      double s = 0.0;
-      for (unsigned int b0 = 0; b0 < gridDim.x; b0 += 32 * kPer) {
-        double x[kPer];
+      uint32_t u[kFixDigits];
+      over = !fix_digits(v[i], unit[i], u) || over;
 #pragma unroll
-        for (int j = 0; j < kPer; ++j) {
-          const unsigned int b = b0 + 32 * j + lane;
-          x[j] = b < gridDim.x ? __ldcg(partials + (size_t)b * NV + i) : 0.0;
-        }
-        const double t = warp_sum_n(x);
-        s = b0 ? s + t : t;
+      for (int k = 0; k < kFixDigits; ++k) {
+        u[k] = __reduce_add_sync(0xffffffffu, u[k]);
+        if (lane == 0) sh.digit[i][k][w] = u[k];
       }
-      tot[i] = s;
     }
-    if (lane == 0 && !ok) sh.bad = 1;
+    if (__any_sync(0xffffffffu, over) && lane == 0) sh.over = 1;
+    __syncthreads();
+    if (w == 0) {
+      unsigned long long word = 0ull;
+#pragma unroll
+      for (int i = 0; i < NV; ++i) {
+        uint32_t t[kFixDigits];
+#pragma unroll
+        for (int k = 0; k < kFixDigits; ++k)
+          t[k] = __reduce_add_sync(0xffffffffu, lane < nw ? sh.digit[i][k][lane] : 0u);
+        const unsigned long long a = (unsigned long long)t[0] + ((unsigned long long)t[1] << 20);
+        const long long b = (long long)t[2] + ((long long)t[3] << 20) + (long long)((unsigned long long)(long long)(int)t[4] << 40) +
+                            (long long)(a >> 40);  // the sum is b 2^40 + the 40 low bits of a
+        unsigned long long lo = (((a & 0xffffffffffull) + 0x2000u) >> 14) + ((unsigned long long)(b & 0x3fff) << 26);
+        long long hi = b >> 14;
+        const bool out = sh.over || hi >= (1ll << 46) || hi < -(1ll << 46);
+        if (out) {
+          lo = 1ull << 48;
+          hi = 0;
+        }
+        if (lane == 2 * i) word = lo + (1ull << 56);
+        if (lane == 2 * i + 1) word = (unsigned long long)(hi + (1ll << 47)) + (1ull << 56);
+      }
+      if (lane < 2 * NV) asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(words + lane), "l"(word) : "memory");
+      bool met = false;
+      for (int64_t k = 0; k < bar.spin && !met; ++k) {
+        if (lane < 2 * NV) asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(word) : "l"(words + lane) : "memory");
+        met = __all_sync(0xffffffffu, lane >= 2 * NV || (word >> 56) == gridDim.x);
+      }
+      bool good = true;
+      double tot[NV];
+#pragma unroll
+      for (int i = 0; i < NV; ++i) {
+        const unsigned long long w0 = __shfl_sync(0xffffffffu, word, 2 * i), w1 = __shfl_sync(0xffffffffu, word, 2 * i + 1);
+        const long long hi = (long long)(w1 & 0xffffffffffffffull) - ((long long)gridDim.x << 47);
+        const unsigned long long lo = w0 & 0xffffffffffffull, l = ((unsigned long long)hi << 40) + lo;
+        tot[i] = fix_value128((hi >> 24) + (l < lo ? 1 : 0), l, unit[i] + 14);
+        good = good && ((w0 >> 48) & 255u) == 0u && fix_unit(tot[i]) >= unit[i] - 7;
+      }
+      __syncwarp();
+      if (lane == 0) {
+        sh.over = 0;
+        sh.again = met && !good;
+        if (!met) sh.bad = 1;
+      }
+      if (met && good) {
+        if (lane == 0)
+#pragma unroll
+          for (int i = 0; i < NV; ++i) unit[i] = fix_unit(tot[i]);
+        fin(tot);
+      }
+    }
+    __syncthreads();
+    if (!sh.again) return;
+  }
+  warp_sums(v, sh, lane, w);
+  __syncthreads();
+  if (w == 0) {
+    double tot[NV];
+    const bool ok = grid_total<NV>(sh, bar, partials, lane, nw, tot);
+    if (lane == 0) {
+      if (!ok) sh.bad = 1;
+#pragma unroll
+      for (int i = 0; i < NV; ++i)
+        unit[i] = tot[i] != 0.0 && isfinite(tot[i]) ? fix_unit(tot[i]) : kFixNoUnit;
+    }
     fin(tot);
   }
   __syncthreads();
@@ -108,7 +242,7 @@ __device__ __forceinline__ uint32_t ldg_stream(const uint32_t* p) {
   return v;
 }
 
-// A slice of the uniform layout (4-bit indices, at most 8 entries a row) held
+// A slice of the uniform layout (4-bit indices, 1 to 8 entries a row) held
 // in registers: loaded one slice ahead, across the grid barriers too, so that
 // only the gathers of p wait on memory.
 template <typename T>
@@ -117,13 +251,13 @@ struct RsSlice {
   uint32_t wd;
   int32_t tv;
   int L;
-  __device__ __forceinline__ void load(const Sliced<T>& sl, uint2 d0, uint2 d1, uint32_t info, int lane) {
-    L = (int)((d1.x - d0.x) >> 5);
-    const T* p = sl.vals + d0.x + lane;
+  __device__ __forceinline__ void load(const Sliced<T>& sl, uint32_t x0, uint32_t x1, uint32_t y0, uint32_t info, int lane) {
+    L = (int)((x1 - x0) >> 5);
+    const T* p = sl.vals + x0 + lane;
 #pragma unroll
     for (int k = 0; k < 8; ++k)
       if (k < L) v[k] = ldg_stream(p + 32 * k);
-    wd = L > 0 ? ldg_stream(reinterpret_cast<const uint32_t*>(sl.ibuf) + d0.y + lane) : 0u;
+    wd = ldg_stream(reinterpret_cast<const uint32_t*>(sl.ibuf) + y0 + lane);
     tv = __ldg(sl.tabs + (info & ~kSliceW4) + (lane & 15));
   }
   // the row's products in entry order; x: the gathered vector at the lane's row
@@ -153,16 +287,18 @@ struct RsMatrix {
   const int32_t* col;
   const T* vals;
   int n, s0, cnt, lane, w, nw;
-  uint2* sdesc;     // [cnt + 1]
   int2* srow;       // MP
+  uint2* sdesc;     // [cnt + 1], not U4
+  uint32_t* sx;     // [cnt + 1], U4: slice s has its index words at 32 s
   uint32_t* sinfo;
   int32_t* snl;     // MP: first non-local entry of the slice's part
   RsSlice<T> f;     // U4: the slice fetched ahead
   NlRange fnl;
 
   // bytes of the records of `per` slices
-  static __host__ __device__ int64_t tail_bytes(bool csr, bool mp, int64_t per) {
-    return csr ? 0 : (per + 1) * 8 + per * 4 + (mp ? per * 12 : 0);
+  static int64_t tail_bytes(int lay, int64_t per) {
+    const bool mp = lay == kRsParts || lay == kRsPartsU4, u4 = lay == kRsU4 || lay == kRsPartsU4;
+    return lay == kRsCsr ? 0 : (per + 1) * (u4 ? 4 : 8) + per * 4 + (mp ? per * 12 : 0);
   }
   __device__ __forceinline__ RsMatrix(const Sliced<T>& sl_, const Parts<T>& parts_, const int32_t* rp, const int32_t* c,
                                       const T* v, int n_, unsigned char* tail, int per)
@@ -173,12 +309,16 @@ struct RsMatrix {
     const int S = LAY == kRsCsr ? (n + 31) / 32 : (int)sl.n_slices;
     s0 = (int)((int64_t)S * blockIdx.x / gridDim.x);
     cnt = (int)((int64_t)S * (blockIdx.x + 1) / gridDim.x) - s0;
-    sdesc = reinterpret_cast<uint2*>(tail);
-    srow = reinterpret_cast<int2*>(sdesc + per + 1);
-    sinfo = reinterpret_cast<uint32_t*>(srow + (MP ? per : 0));
+    srow = reinterpret_cast<int2*>(tail);
+    sdesc = reinterpret_cast<uint2*>(srow + (MP ? per : 0));
+    sx = reinterpret_cast<uint32_t*>(sdesc);
+    sinfo = U4 ? sx + per + 1 : reinterpret_cast<uint32_t*>(sdesc + per + 1);
     snl = reinterpret_cast<int32_t*>(sinfo + per);
     if (LAY != kRsCsr) {
-      for (int j = threadIdx.x; j <= cnt; j += blockDim.x) sdesc[j] = sl.desc[s0 + j];
+      for (int j = threadIdx.x; j <= cnt; j += blockDim.x) {
+        if (U4) sx[j] = sl.desc[s0 + j].x;
+        else sdesc[j] = sl.desc[s0 + j];
+      }
       for (int j = threadIdx.x; j < cnt; j += blockDim.x) {
         sinfo[j] = sl.tinfo[s0 + j];
         if (MP) {
@@ -201,7 +341,7 @@ struct RsMatrix {
     return i < n ? i : -1;
   }
   __device__ __forceinline__ void fetch(int j) {
-    f.load(sl, sdesc[j], sdesc[j + 1], sinfo[j], lane);
+    f.load(sl, sx[j], sx[j + 1], (uint32_t)(kSliceRows * (s0 + j)), sinfo[j], lane);
     if (MP) {
       const int i = row_of(j);
       fnl = i >= 0 ? nonlocal_range<T>(parts, srow[j].y >> 6, i) : NlRange{0, 0};
@@ -272,7 +412,7 @@ ResidentPlan plan_resident(const rp_handle* h, const Sliced<T>& sl, int64_t n, s
   const int64_t S = lay == kRsCsr ? (n + 31) / 32 : sl.n_slices;
   const int grid = (int)std::min<int64_t>(h->num_sms, S);
   const int64_t per = (S + grid - 1) / grid;  // slices a block at most
-  const int64_t tail = RsMatrix<T, kRsCsr>::tail_bytes(lay == kRsCsr, sl.srow != nullptr, per);
+  const int64_t tail = RsMatrix<T, kRsCsr>::tail_bytes(lay, per);
   for (int v : vecs) {
     void* fn = fn_of(lay, v);
     const int64_t need = per * 32 * v * (int64_t)sizeof(T) + tail;

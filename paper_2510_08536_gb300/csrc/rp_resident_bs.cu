@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident_bs(const Resident
   T* xg = V.x;
   if constexpr (sizeof(T) == 8) xg = a.io->x;
 
-  RsBarrier bar{A.sync, A.sync[32], A.spin};
+  RsBarrier bar{A.sync + kRsCount, A.sync[kRsBase], A.spin};
   const double thresh = c->ithresh;
   const int max_iter = c->max_iter;
   if (tid == 0) {
@@ -230,7 +230,7 @@ __global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident_bs(const Resident
     }
   }
   if (blockIdx.x == 0 && tid == 0) {
-    A.sync[32] = bar.target;
+    A.sync[kRsBase] = bar.target;
     c->iter = sh.iter;
     c->rho = sh.rho;
     c->rho_old = sh.rho_old;

@@ -482,7 +482,7 @@ rp_status build_sliced(rp_handle* h, cudaStream_t st) {
       t = it->second;
     }
     const bool w4 = D <= 16;
-    u4 = u4 && w4 && hw[s] <= 8;
+    u4 = u4 && w4 && hw[s] >= 1 && hw[s] <= 8;
     tinfo[s] = t | (w4 ? kSliceW4 : 0u);
     desc[s] = make_uint2((uint32_t)x, (uint32_t)y);
     const int per = w4 ? 8 : 4;

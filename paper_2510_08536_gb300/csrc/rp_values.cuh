@@ -105,6 +105,37 @@ __device__ __forceinline__ double recip_rn(double d) {
                               (((int64_t)(2045u - e) << 52) + (q - (1ll << 52))));
 }
 
+// a / b, a and b > 0, in the same way: 18, 17 and 17 bits (a's mantissa below b's:
+// one more) after the exact first step.
+__device__ __forceinline__ double quot_rn(double a, double b) {
+  const uint32_t ah = (uint32_t)__double2hiint(a), al = (uint32_t)__double2loint(a);
+  const uint32_t bh = (uint32_t)__double2hiint(b), bl = (uint32_t)__double2loint(b);
+  const int ea = (int)(ah >> 20), eb = (int)(bh >> 20);  // with the sign bit
+  if ((unsigned)(ea - 1) > 2045u || (unsigned)(eb - 1) > 2045u || (unsigned)(ea - eb + 1022) > 2043u) return a / b;
+  const uint64_t ma = (uint64_t)((ah & 0xfffffu) | 0x100000u) << 32 | al;
+  const uint64_t mb = (uint64_t)((bh & 0xfffffu) | 0x100000u) << 32 | bl;
+  const float f = __uint_as_float(0x3f800000u | (__funnelshift_l(bl, bh, 3) & 0x7fffffu));
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(f));
+  // q 2^52 (2^53) for a quotient in [1, 2) ([1/2, 1))
+  const int more = ma < mb ? 1 : 0;
+  int64_t r = (int64_t)(ma << more), q = 1;
+  r -= (int64_t)mb;  // the leading bit of the quotient: 0 <= r < mb
+  const float yq = y * 0x1p-1f;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const int t = k == 0 ? 18 : 17;
+    const int dgt = small_int(small_float((int)(r >> 33)) * (k == 0 ? yq : yq * 0.5f));  // r 2^t / mb
+    r = (int64_t)(((uint64_t)r << t) - (uint64_t)(int64_t)dgt * mb);
+    q = (q << t) + dgt;
+  }
+  // |r| < 3/2 mb: to nearest (ties do not occur: the quotient of two 53-bit integers is no odd
+  // multiple of half a 53-bit unit)
+  const int64_t h = (int64_t)(mb >> 1);
+  q += r > h ? 1 : r < -h ? -1 : 0;
+  return __longlong_as_double(((int64_t)(ea - eb - more + 1023) << 52) + (q - (1ll << 52)));
+}
+
 __device__ __forceinline__ double sqrt_rn(double d) {
   const uint32_t hi = (uint32_t)__double2hiint(d), lo = (uint32_t)__double2loint(d);
   if ((hi >> 20) - 1u > 2045u) return sqrt(d);  // zeros, subnormals, negative values, infinities, NaN
