@@ -87,13 +87,16 @@ __global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident(const ResidentArg
   const int cnt = M.cnt;
   for (int j = w; j < cnt; j += nw) {
     const int i = M.row_of(j), k = j * 32 + lane;
-    if (i < 0) continue;
-    rs[k] = a.r[i];
+    rs[k] = i >= 0 ? a.r[i] : T(0);
+    qs[k] = T(0);
     if (ALL) {
-      ps[k] = a.p[i];
-      xs[k] = xg[i];
+      ps[k] = i >= 0 ? a.p[i] : T(0);
+      xs[k] = i >= 0 ? xg[i] : T(0);
     }
   }
+  constexpr int W = ALL ? 16 / (int)sizeof(T) : 1;  // rows a thread takes at once outside the product
+  __syncthreads();
+
   double* part = a.partials;  // two sets of partial sums in turn
   double* part2 = a.partials + 2 * (size_t)gridDim.x;
   for (;;) {
@@ -127,20 +130,34 @@ __global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident(const ResidentArg
     // B: r -= alpha q, z = D^-1 r (kept in q's place), x += alpha p, (r, z), (r, r)
     const T alpha = sh.alpha;
     T rza = T(0), rra = T(0);
-    for (int j = w; j < cnt; j += nw) {
-      const int i = M.row_of(j), k = j * 32 + lane;
-      if (i < 0) continue;
-      const T ri = fma(-alpha, qs[k], rs[k]);
-      rs[k] = ri;
-      if (!SCALED) {
-        const T z = a.dinv[i] * ri;
-        qs[k] = z;
-        rza = fma(ri, z, rza);
+    M.template groups<W>([&](int k, int i, int m, bool whole) {
+      const RsPack<T, W> q = ld_pack<W>(qs + k);
+      RsPack<T, W> r = ld_pack<W>(rs + k);
+#pragma unroll
+      for (int e = 0; e < W; ++e) {
+        r.e[e] = fma(-alpha, q.e[e], r.e[e]);
+        rra = fma(r.e[e], r.e[e], rra);
       }
-      rra = fma(ri, ri, rra);
-      if (ALL) xs[k] = fma(alpha, ps[k], xs[k]);
-      else xg[i] = fma(alpha, a.p[i], xg[i]);
-    }
+      st_pack<W>(rs + k, r);
+      if constexpr (!SCALED) {
+        RsPack<T, W> z = ld_rows<W, true>(a.dinv + i, m, whole);
+#pragma unroll
+        for (int e = 0; e < W; ++e) {
+          z.e[e] *= r.e[e];
+          rza = fma(r.e[e], z.e[e], rza);
+        }
+        st_pack<W>(qs + k, z);
+      }
+      if constexpr (ALL) {
+        const RsPack<T, W> pv = ld_pack<W>(ps + k);
+        RsPack<T, W> x = ld_pack<W>(xs + k);
+#pragma unroll
+        for (int e = 0; e < W; ++e) x.e[e] = fma(alpha, pv.e[e], x.e[e]);
+        st_pack<W>(xs + k, x);
+      } else {
+        xg[i] = fma(alpha, a.p[i], xg[i]);
+      }
+    });
     {
       constexpr int NV = SCALED ? 1 : 2;
       T v[NV];
@@ -167,13 +184,16 @@ __global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident(const ResidentArg
     if (sh.bad || sh.stop) break;
     // C: p = z + beta p
     const T beta = sh.beta;
-    for (int j = w; j < cnt; j += nw) {
-      const int i = M.row_of(j), k = j * 32 + lane;
-      if (i < 0) continue;
-      const T pi = fma(beta, ALL ? ps[k] : a.p[i], SCALED ? rs[k] : qs[k]);
-      if (ALL) ps[k] = pi;
-      a.p[i] = pi;
-    }
+    M.template groups<W>([&](int k, int i, int m, bool whole) {
+      RsPack<T, W> p;
+      if constexpr (ALL) p = ld_pack<W>(ps + k);
+      else p.e[0] = a.p[i];
+      const RsPack<T, W> z = ld_pack<W>((SCALED ? rs : qs) + k);
+#pragma unroll
+      for (int e = 0; e < W; ++e) p.e[e] = fma(beta, p.e[e], z.e[e]);
+      if constexpr (ALL) st_pack<W>(ps + k, p);
+      st_rows<W>(a.p + i, p, m, whole);
+    });
     __syncthreads();
     if (tid == 0) {
       if (!bar.meet()) sh.bad = 1;
@@ -183,6 +203,7 @@ __global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident(const ResidentArg
     if (sh.bad || sh.stop) break;
   }
   // the state back to memory (p is there already)
+  __syncthreads();
   for (int j = w; j < cnt; j += nw) {
     const int i = M.row_of(j), k = j * 32 + lane;
     if (i < 0) continue;

@@ -1,8 +1,7 @@
 // Building blocks of the resident solver kernels (rp_resident.cu: PCG,
 // rp_bicgstab.cu: BiCGStab): one block an SM owns a contiguous run of 32-row
-// slices, a warp takes every nw-th of them in every phase (so a row's values
-// never leave its lane's hands between phases), and the grid meets at an arrival
-// counter.
+// slices, a warp takes every nw-th of them in the products and 16-byte groups of
+// rows in the passes over vectors, and the grid meets at an arrival counter.
 #pragma once
 
 #include <algorithm>
@@ -254,28 +253,81 @@ struct RsSlice {
   __device__ __forceinline__ void load(const Sliced<T>& sl, uint32_t x0, uint32_t x1, uint32_t y0, uint32_t info, int lane) {
     L = (int)((x1 - x0) >> 5);
     const T* p = sl.vals + x0 + lane;
-#pragma unroll
-    for (int k = 0; k < 8; ++k)
-      if (k < L) v[k] = ldg_stream(p + 32 * k);
     wd = ldg_stream(reinterpret_cast<const uint32_t*>(sl.ibuf) + y0 + lane);
     tv = __ldg(sl.tabs + (info & ~kSliceW4) + (lane & 15));
+    if (L == 7) {  // a cell and its six neighbours: most slices, without a test an entry
+#pragma unroll
+      for (int k = 0; k < 7; ++k) v[k] = ldg_stream(p + 32 * k);
+    } else {
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+        if (k < L) v[k] = ldg_stream(p + 32 * k);
+    }
   }
   // the row's products in entry order; x: the gathered vector at the lane's row
   __device__ __forceinline__ T sum(const T* x, bool valid) const {
-    T g[8];
+    T g[8], s = T(0);
+    if (L == 7 && __all_sync(0xffffffffu, valid)) {
+#pragma unroll
+      for (int k = 0; k < 7; ++k) g[k] = x[slice_offset<kIdx4>(wd, k, tv, nullptr, 0)];
+#pragma unroll
+      for (int k = 0; k < 7; ++k) s = fma(v[k], g[k], s);
+      return s;
+    }
 #pragma unroll
     for (int k = 0; k < 8; ++k)
       if (k < L) {
         const int off = slice_offset<kIdx4>(wd, k, tv, nullptr, 0);
         g[k] = valid ? x[off] : T(0);
       }
-    T s = T(0);
 #pragma unroll
     for (int k = 0; k < 8; ++k)
       if (k < L) s = fma(v[k], g[k], s);
     return s;
   }
 };
+
+// W values of one type, moved as one access of up to 16 bytes
+template <typename T, int W>
+struct alignas(W * sizeof(T)) RsPack {
+  T e[W];
+};
+template <int W, typename T>
+__device__ __forceinline__ RsPack<T, W> ld_pack(const T* p) {
+  return *reinterpret_cast<const RsPack<T, W>*>(p);
+}
+template <int W, typename T>
+__device__ __forceinline__ void st_pack(T* p, const RsPack<T, W>& v) {
+  *reinterpret_cast<RsPack<T, W>*>(p) = v;
+}
+// the same for the first m of them (global vectors: at the end of the rows, or of
+// a part whose rows do not start at a multiple of W); the others read as 0
+template <int W, bool RO, typename T>
+__device__ __forceinline__ RsPack<T, W> ld_rows(const T* p, int m, bool whole) {
+  RsPack<T, W> v;
+  if (whole) {
+    if constexpr (W * sizeof(T) == 16 && RO) {
+      const auto q = __ldg(reinterpret_cast<const typename Vec<T>::type*>(p));
+      for_each_comp<W>([&](auto c) { v.e[decltype(c)::value] = comp<decltype(c)::value>(const_cast<typename Vec<T>::type&>(q)); });
+    } else {
+      v = ld_pack<W>(p);
+    }
+    return v;
+  }
+#pragma unroll
+  for (int e = 0; e < W; ++e) v.e[e] = e < m ? (RO ? __ldg(p + e) : p[e]) : T(0);
+  return v;
+}
+template <int W, typename T>
+__device__ __forceinline__ void st_rows(T* p, const RsPack<T, W>& v, int m, bool whole) {
+  if (whole) {
+    st_pack<W>(p, v);
+    return;
+  }
+#pragma unroll
+  for (int e = 0; e < W; ++e)
+    if (e < m) p[e] = v.e[e];
+}
 
 // The block's slices and their products with a gathered vector.
 template <typename T, int LAY>
@@ -339,6 +391,25 @@ struct RsMatrix {
     }
     const int i = (s0 + j) * kSliceRows + lane;
     return i < n ? i : -1;
+  }
+  // The block's rows in groups of W, for the passes over vectors: f(k, i, m, whole)
+  // with the group's place k in shared memory, its first row i, its m rows (1 .. W)
+  // and whether rows i .. i + W - 1 can be moved as one aligned access. Rows past the
+  // end are zeros in shared memory.
+  template <int W, typename F>
+  __device__ __forceinline__ void groups(F&& f) const {
+    for (int k = threadIdx.x * W; k < cnt * kSliceRows; k += blockDim.x * W) {
+      int i, m;
+      if (MP) {
+        const int2 r = srow[k >> 5];
+        i = r.x + (k & 31);
+        m = min(W, (r.y & 63) - (k & 31));
+      } else {
+        i = s0 * kSliceRows + k;
+        m = min(W, n - i);
+      }
+      if (m > 0) f(k, i, m, W == 1 || (!MP && m == W));
+    }
   }
   __device__ __forceinline__ void fetch(int j) {
     f.load(sl, sx[j], sx[j + 1], (uint32_t)(kSliceRows * (s0 + j)), sinfo[j], lane);

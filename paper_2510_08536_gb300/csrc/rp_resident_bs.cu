@@ -57,6 +57,7 @@ __global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident_bs(const Resident
   T* ts = vs + A.rows;
   T* xg = V.x;
   if constexpr (sizeof(T) == 8) xg = a.io->x;
+  const bool x16 = (reinterpret_cast<uintptr_t>(xg) & 15) == 0;  // the caller's may not be
 
   RsBarrier bar{A.sync + kRsCount, A.sync[kRsBase], A.spin};
   const double thresh = c->ithresh;
@@ -79,11 +80,13 @@ __global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident_bs(const Resident
   const int cnt = M.cnt;
   for (int j = w; j < cnt; j += nw) {
     const int i = M.row_of(j), k = j * 32 + lane;
-    if (i < 0) continue;
-    rs[k] = V.r[i];
-    ps[k] = V.p[i];
-    vs[k] = V.v[i];
+    rs[k] = i >= 0 ? V.r[i] : T(0);
+    ps[k] = i >= 0 ? V.p[i] : T(0);
+    vs[k] = i >= 0 ? V.v[i] : T(0);
+    ts[k] = T(0);
   }
+  constexpr int W = 16 / (int)sizeof(T);  // rows a thread takes at once outside the products
+  __syncthreads();
 
   double* part = a.partials;  // two sets of partial sums in turn
   double* part2 = a.partials + 2 * (size_t)gridDim.x;
@@ -91,13 +94,17 @@ __global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident_bs(const Resident
     // B1
     {
       const T be = sh.be, om = sh.om;
-      for (int j = w; j < cnt; j += nw) {
-        const int i = M.row_of(j), k = j * 32 + lane;
-        if (i < 0) continue;
-        const T pi = fma(be, fma(-om, vs[k], ps[k]), rs[k]);
-        ps[k] = pi;
-        V.phat[i] = __ldg(V.dinv + i) * pi;
-      }
+      M.template groups<W>([&](int k, int i, int m, bool whole) {
+        RsPack<T, W> p = ld_pack<W>(ps + k), h = ld_rows<W, true>(V.dinv + i, m, whole);
+        const RsPack<T, W> v = ld_pack<W>(vs + k), r = ld_pack<W>(rs + k);
+#pragma unroll
+        for (int e = 0; e < W; ++e) {
+          p.e[e] = fma(be, fma(-om, v.e[e], p.e[e]), r.e[e]);
+          h.e[e] *= p.e[e];
+        }
+        st_pack<W>(ps + k, p);
+        st_rows<W>(V.phat + i, h, m, whole);
+      });
       __syncthreads();
       if (tid == 0 && !bar.meet()) sh.bad = 1;
       __syncthreads();
@@ -132,14 +139,18 @@ __global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident_bs(const Resident
     // B3
     {
       T acc = T(0);
-      for (int j = w; j < cnt; j += nw) {
-        const int i = M.row_of(j), k = j * 32 + lane;
-        if (i < 0) continue;
-        const T si = fma(-al, vs[k], rs[k]);
-        rs[k] = si;
-        V.shat[i] = __ldg(V.dinv + i) * si;
-        acc = fma(si, si, acc);
-      }
+      M.template groups<W>([&](int k, int i, int m, bool whole) {
+        RsPack<T, W> r = ld_pack<W>(rs + k), h = ld_rows<W, true>(V.dinv + i, m, whole);
+        const RsPack<T, W> v = ld_pack<W>(vs + k);
+#pragma unroll
+        for (int e = 0; e < W; ++e) {
+          r.e[e] = fma(-al, v.e[e], r.e[e]);
+          acc = fma(r.e[e], r.e[e], acc);
+          h.e[e] *= r.e[e];
+        }
+        st_pack<W>(rs + k, r);
+        st_rows<W>(V.shat + i, h, m, whole);
+      });
       const T v[1] = {acc};
       grid_sum<1>(v, sh, bar, part2, lane, w, nw, [&](const double (&tot)[1]) {
         if (lane != 0) return;
@@ -148,7 +159,7 @@ __global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident_bs(const Resident
       });
     }
     if (sh.bad) break;
-    if (sh.stop == 3) {
+    if (sh.stop == 3) {  // (the groups' rows are this block's: no wait since B1 is missing)
       for (int j = w; j < cnt; j += nw) {
         const int i = M.row_of(j), k = j * 32 + lane;
         if (i >= 0) xg[i] = fma(al, __ldg(V.dinv + i) * ps[k], xg[i]);
@@ -189,16 +200,22 @@ __global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident_bs(const Resident
     {
       const T om = sh.om;
       T arr = T(0), arh = T(0);
-      for (int j = w; j < cnt; j += nw) {
-        const int i = M.row_of(j), k = j * 32 + lane;
-        if (i < 0) continue;
-        const T d = __ldg(V.dinv + i), si = rs[k];
-        xg[i] = fma(om, d * si, fma(al, d * ps[k], xg[i]));
-        const T ri = fma(-om, ts[k], si);
-        rs[k] = ri;
-        arr = fma(ri, ri, arr);
-        arh = fma(__ldg(V.rhat + i), ri, arh);
-      }
+      M.template groups<W>([&](int k, int i, int m, bool whole) {
+        RsPack<T, W> r = ld_pack<W>(rs + k);
+        const RsPack<T, W> d = ld_rows<W, true>(V.dinv + i, m, whole), p = ld_pack<W>(ps + k), t = ld_pack<W>(ts + k);
+        const RsPack<T, W> rh = ld_rows<W, true>(V.rhat + i, m, whole);
+        const bool xw = whole && x16;
+        RsPack<T, W> x = ld_rows<W, false>(xg + i, m, xw);
+#pragma unroll
+        for (int e = 0; e < W; ++e) {
+          x.e[e] = fma(om, d.e[e] * r.e[e], fma(al, d.e[e] * p.e[e], x.e[e]));
+          r.e[e] = fma(-om, t.e[e], r.e[e]);
+          arr = fma(r.e[e], r.e[e], arr);
+          arh = fma(rh.e[e], r.e[e], arh);
+        }
+        st_rows<W>(xg + i, x, m, xw);
+        st_pack<W>(rs + k, r);
+      });
       const T v[2] = {arr, arh};
       grid_sum<2>(v, sh, bar, part2, lane, w, nw, [&](const double (&tot)[2]) {
         if (lane != 0) return;
