@@ -23,7 +23,10 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <cmath>
+#include <functional>
 #include <numeric>
+#include <queue>
 
 #include "rp_common.cuh"
 #include "rp_spmv.cuh"
@@ -823,6 +826,49 @@ rp_status build_batch_graph(rp_handle* h, int mode, int cluster, int threads, cu
   return RP_OK;
 }
 
+// The team size of a batch whose caller sets none. A system of n rows takes about
+// n^(1/3) iterations of 5000 + n / c rows' time on a team of c CTAs (the constant:
+// the barriers and sums of an iteration; fitted, within 10% of all the times below),
+// and the queue hands the largest systems out first, so the step ends with the last
+// team of that schedule. Few systems leave most SMs idle behind the largest one on
+// small teams; many, on large teams, pay the constant too often. ms a step
+// (continued refinement) with teams of 5, 8, 10, 12, 16 -- all batches took 5:
+//   48 systems of 8k-300k rows  125.5  84.6  67.4  59.1  66.9  (12 taken)
+//   48 of 1k-40k                 12.6  10.6   9.1  10.4  15.9  (10)
+//   32 of 4k-300k               114.7  79.2  64.1  52.5  43.9  (16)
+//    9 of 5k-300k                55.5  37.4  30.9  27.0  22.0  (16)
+//   96 of 4k-200k                72.4  54.8  53.8  59.3  81.2  (10)
+int team_size(rp_handle* h) {
+  std::vector<int64_t> rows(h->n_parts);
+  for (int p = 0; p < h->n_parts; ++p) rows[p] = h->part_row_off[p + 1] - h->part_row_off[p];
+  std::sort(rows.begin(), rows.end(), std::greater<int64_t>());
+  int best = h->batch_cluster;
+  double least = 0.0;
+  for (int c : {4, 5, 6, 8, 10, 12, 16}) {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr;
+    int nc = 0;
+    if (launch_config(h, 0, c, h->batch_threads, &cfg, &attr, &nc) != RP_OK) {
+      cudaGetLastError();
+      continue;
+    }
+    std::priority_queue<double, std::vector<double>, std::greater<double>> team(std::greater<double>(),
+                                                                                std::vector<double>(nc, 0.0));
+    double end = 0.0;
+    for (int64_t n : rows) {
+      const double t = team.top() + std::cbrt((double)n) * (5000.0 + (double)n / c);
+      team.pop();
+      team.push(t);
+      end = std::max(end, t);
+    }
+    if (least == 0.0 || end < least) {
+      least = end;
+      best = c;
+    }
+  }
+  return best;
+}
+
 }  // namespace
 
 rp_status batch_prepare(rp_handle* h) {
@@ -895,6 +941,7 @@ rp_status batch_prepare(rp_handle* h) {
   a.sl_entries = h->sl_entries;
   a.sl_ibuf_len = h->sl_ibuf_len;
   a.sl_tabs_len = h->sl_tabs_len;
+  h->batch_cluster = team_size(h);
   h->batch_ready = true;
   return RP_OK;
 }
@@ -996,7 +1043,7 @@ extern "C" rp_status rp_batch_autotune(rp_handle* h, const double* buffer, const
   // team counts between these shapes matter: with the largest systems first,
   // too many small teams leave the largest system's team running alone at
   // the end, too few large teams pay more barrier latency per iteration
-  const int clusters[] = {2, 3, 4, 5, 6, 8, 16};
+  const int clusters[] = {2, 3, 4, 5, 6, 8, 10, 12, 16};
   const int threads[] = {256, 512};
   cudaEvent_t e0, e1;
   RP_TRY_CUDA(cudaEventCreate(&e0));
