@@ -349,6 +349,7 @@ struct rp_handle {
   int64_t sl_ibuf_len = 0;   // index words
   int64_t sl_tabs_len = 0;   // int32 words of the distinct tables
   int sl_u4 = 0;             // every slice 4-bit with rows of at most 8 entries
+  int sl_width = 0;          // longest row of any slice
   int64_t* sl_part_soff = nullptr;  // [n_parts + 1] first slice of each part (device)
   int2* sl_srow = nullptr;           // [sl_slices] first row, part << 6 | rows (n_parts > 1)
   uint2* sl_desc = nullptr;  // [sl_slices + 1]

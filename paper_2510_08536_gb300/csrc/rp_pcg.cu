@@ -951,8 +951,8 @@ SolveSet solve_set(rp_handle* h, int mode, const double* vals, const double* din
     k.g3_32 = h->igrid32.k3;
   }
   k.resident = mixed ? resident_plan<float>(h, k.a32, k.scaled) : resident_plan<double>(h, k.a64, false);
-  k.rs64 = ResidentArgs<double>{k.a64, h->rsync, h->opts.spin_limit, k.resident.rows, INT32_MAX};
-  k.rs32 = ResidentArgs<float>{k.a32, h->rsync, h->opts.spin_limit, k.resident.rows, INT32_MAX};
+  k.rs64 = ResidentArgs<double>{k.a64, h->rsync, h->opts.spin_limit, k.resident.rows, k.resident.width, INT32_MAX};
+  k.rs32 = ResidentArgs<float>{k.a32, h->rsync, h->opts.spin_limit, k.resident.rows, k.resident.width, INT32_MAX};
   return k;
 }
 

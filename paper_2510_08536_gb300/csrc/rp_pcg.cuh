@@ -37,6 +37,7 @@ struct ResidentArgs {
   unsigned int* sync;  // memory of the grid barrier and sums, cleared before each solve
   int64_t spin;        // probe limit of a barrier wait
   int32_t rows;        // rows of shared memory a block holds (a multiple of 32)
+  int32_t width;       // longest row of a kept matrix
   int32_t cap;
 };
 // The launch of the resident kernel for these arguments, or fn = nullptr where

@@ -51,8 +51,10 @@ __device__ __forceinline__ T ratio(double a, double b) {
 }
 
 // LAY: layout of the product; SCALED: the system S A S (z = r); ALL: r, x, p
-// and q in shared memory, else r and q.
-template <typename T, int LAY, bool SCALED, bool ALL>
+// and q in shared memory, else r and q; MAT: the matrix too; FOLD: no barrier C (the
+// product gathers z + beta p of the two vectors, which are written to global memory
+// before the sum of B).
+template <typename T, int LAY, bool SCALED, bool ALL, bool MAT, bool FOLD>
 __global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident(const ResidentArgs<T> A) {
   const IterArgs<T>& a = A.it;
   Ctl* c = a.ctl;
@@ -82,9 +84,16 @@ __global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident(const ResidentArg
     sh.bad = sh.stop = sh.done = sh.over = 0;
     for (int k = 0; k < 3; ++k) sh.unit[k] = (int)A.sync[kRsUnit + k];
   }
-  RsMatrix<T, LAY> M(a.sl, a.parts, a.row_ptr, a.col, a.vals, (int)a.n,
-                     reinterpret_cast<unsigned char*>(rs + (ALL ? 4 : 2) * (size_t)A.rows), A.rows / 32);
+  using Matrix = RsMatrix<T, LAY, MAT>;
+  static_assert(!FOLD || (ALL && Matrix::U4), "folded: p on chip, any row gathered by a functor");
+  Matrix M(a.sl, a.parts, a.row_ptr, a.col, a.vals, (int)a.n,
+           reinterpret_cast<unsigned char*>(rs + (ALL ? 4 : 2) * (size_t)A.rows), A.rows / 32, A.width);
   const int cnt = M.cnt;
+  // FOLD: z, the last p and where it goes next; the first p is in memory as it is
+  T* const zbuf = SCALED ? a.r : a.q;
+  T* pcur = a.p;
+  const T *zg = a.p, *pold = a.p;
+  T fold_beta = T(0);
   for (int j = w; j < cnt; j += nw) {
     const int i = M.row_of(j), k = j * 32 + lane;
     rs[k] = i >= 0 ? a.r[i] : T(0);
@@ -102,9 +111,14 @@ __global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident(const ResidentArg
   for (;;) {
     // A: q = A p, (p, q)
     T acc = T(0);
+    auto gathers = [&] {
+      if constexpr (FOLD) return RsFold<T>{zg, pold, fold_beta};
+      else return RsGlobal<T>{a.p};
+    };
+    const auto from = gathers();
     for (int j = w; j < cnt; j += nw) {
       const int i = M.row_of(j), k = j * 32 + lane;
-      const T sum = M.product(j, i, a.p);
+      const T sum = M.product(j, i, from);
       if (i >= 0) {
         qs[k] = sum;
         acc = fma(ALL ? ps[k] : a.p[i], sum, acc);
@@ -112,7 +126,7 @@ __global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident(const ResidentArg
     }
     {
       const T v[1] = {acc};
-      grid_sum_unit<1>(v, sh.unit, rs_words(A.sync, set, 0), sh, bar, part, lane, w, nw, [&](const double (&tot)[1]) {
+      grid_sum_unit<1, false>(v, sh.unit, rs_words(A.sync, set, 0), sh, bar, part, lane, w, nw, [&](const double (&tot)[1]) {
         if (lane != 0) return;
         sh.pq = tot[0];
         sh.alpha = ratio<T>(sh.rz, tot[0]);
@@ -139,6 +153,7 @@ __global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident(const ResidentArg
         rra = fma(r.e[e], r.e[e], rra);
       }
       st_pack<W>(rs + k, r);
+      if constexpr (SCALED && FOLD) st_rows<W>(zbuf + i, r, m, whole);
       if constexpr (!SCALED) {
         RsPack<T, W> z = ld_rows<W, true>(a.dinv + i, m, whole);
 #pragma unroll
@@ -147,6 +162,7 @@ __global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident(const ResidentArg
           rza = fma(r.e[e], z.e[e], rza);
         }
         st_pack<W>(qs + k, z);
+        if constexpr (FOLD) st_rows<W>(zbuf + i, z, m, whole);
       }
       if constexpr (ALL) {
         const RsPack<T, W> pv = ld_pack<W>(ps + k);
@@ -163,7 +179,7 @@ __global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident(const ResidentArg
       T v[NV];
       v[NV - 1] = rra;
       if constexpr (!SCALED) v[0] = rza;
-      grid_sum_unit<NV>(v, sh.unit + 1, rs_words(A.sync, set, 1), sh, bar, part2, lane, w, nw, [&](const double (&tot)[NV]) {
+      grid_sum_unit<NV, FOLD>(v, sh.unit + 1, rs_words(A.sync, set, 1), sh, bar, part2, lane, w, nw, [&](const double (&tot)[NV]) {
         if (lane != 0) return;
         sh.rr = tot[NV - 1];
         ++sh.iter;
@@ -177,13 +193,15 @@ __global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident(const ResidentArg
         } else {
           sh.beta = ratio<T>(tot[0], sh.rz);
           sh.rz = tot[0];
+          if (sh.done >= A.cap) sh.stop = 3;  // after C; the next launch goes on
         }
       });
     }
     set = set == 2 ? 0 : set + 1;
-    if (sh.bad || sh.stop) break;
+    if (sh.bad || sh.stop == 1) break;
     // C: p = z + beta p
     const T beta = sh.beta;
+    T* const pnext = !FOLD || pcur != a.p ? a.p : SCALED ? a.q : a.r;
     M.template groups<W>([&](int k, int i, int m, bool whole) {
       RsPack<T, W> p;
       if constexpr (ALL) p = ld_pack<W>(ps + k);
@@ -192,23 +210,28 @@ __global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident(const ResidentArg
 #pragma unroll
       for (int e = 0; e < W; ++e) p.e[e] = fma(beta, p.e[e], z.e[e]);
       if constexpr (ALL) st_pack<W>(ps + k, p);
-      st_rows<W>(a.p + i, p, m, whole);
+      st_rows<W>(pnext + i, p, m, whole);
     });
     __syncthreads();
-    if (tid == 0) {
-      if (!bar.meet()) sh.bad = 1;
-      if (sh.done >= A.cap) sh.stop = 3;  // the next launch goes on
+    if constexpr (FOLD) {
+      zg = zbuf;
+      pold = pcur;
+      pcur = pnext;
+      fold_beta = beta;
+    } else {
+      if (tid == 0 && !bar.meet()) sh.bad = 1;
+      __syncthreads();
     }
-    __syncthreads();
     if (sh.bad || sh.stop) break;
   }
-  // the state back to memory (p is there already)
+  // the state back to memory (without FOLD p is there already)
   __syncthreads();
   for (int j = w; j < cnt; j += nw) {
     const int i = M.row_of(j), k = j * 32 + lane;
     if (i < 0) continue;
     a.r[i] = rs[k];
     if (ALL) xg[i] = xs[k];
+    if (FOLD) a.p[i] = ps[k];
   }
   if (blockIdx.x == 0 && tid == 0) {
     A.sync[kRsBase] = bar.target;
@@ -230,17 +253,29 @@ __global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident(const ResidentArg
 }
 
 template <typename T, bool ALL>
-void* resident_fn(int lay, bool scaled) {
+void* streamed_fn(int lay, bool scaled) {
   if constexpr (sizeof(T) == 4) {
     if (scaled)
-      return lay == kRsU4 ? (void*)k_resident<T, kRsU4, true, ALL> : (void*)k_resident<T, kRsSliced, true, ALL>;
+      return lay == kRsU4 ? (void*)k_resident<T, kRsU4, true, ALL, false, false>
+                          : (void*)k_resident<T, kRsSliced, true, ALL, false, false>;
   }
   switch (lay) {
-    case kRsU4: return (void*)k_resident<T, kRsU4, false, ALL>;
-    case kRsSliced: return (void*)k_resident<T, kRsSliced, false, ALL>;
-    case kRsParts: return (void*)k_resident<T, kRsParts, false, ALL>;
-    case kRsPartsU4: return (void*)k_resident<T, kRsPartsU4, false, ALL>;
-    default: return (void*)k_resident<T, kRsCsr, false, ALL>;
+    case kRsU4: return (void*)k_resident<T, kRsU4, false, ALL, false, false>;
+    case kRsSliced: return (void*)k_resident<T, kRsSliced, false, ALL, false, false>;
+    case kRsParts: return (void*)k_resident<T, kRsParts, false, ALL, false, false>;
+    case kRsPartsU4: return (void*)k_resident<T, kRsPartsU4, false, ALL, false, false>;
+    default: return (void*)k_resident<T, kRsCsr, false, ALL, false, false>;
+  }
+}
+template <typename T, bool FOLD>
+void* kept_fn(int lay, bool scaled) {
+  if constexpr (sizeof(T) == 4) {
+    if (scaled) return lay == kRsU4 ? (void*)k_resident<T, kRsU4, true, true, true, FOLD> : nullptr;
+    return lay == kRsPartsU4 ? (void*)k_resident<T, kRsPartsU4, false, true, true, FOLD> : nullptr;
+  } else {
+    return lay == kRsU4        ? (void*)k_resident<T, kRsU4, false, true, true, FOLD>
+           : lay == kRsPartsU4 ? (void*)k_resident<T, kRsPartsU4, false, true, true, FOLD>
+                               : nullptr;
   }
 }
 
@@ -248,16 +283,26 @@ void* resident_fn(int lay, bool scaled) {
 
 RP_CHECK_TU(resident)
 
+// The forms, best first. Folding doubles the product's gathers to save a barrier: only
+// where a warp has one slice.
+enum : int { kKeptFold, kKept, kStream4, kStream2 };
+template <typename T>
+constexpr int kFoldRows = kRsThreads<T>;
 template <typename T>
 ResidentPlan resident_plan(const rp_handle* h, const IterArgs<T>& a, bool scaled) {
   if (a.line.l != nullptr) return ResidentPlan{};
-  auto fn = [&](int lay, int vecs) {
+  auto fn = [&](int lay, const ResidentForm& f) -> void* {
     if constexpr (sizeof(T) == 8)
-      if (vecs == 2) return resident_fn<T, false>(lay, scaled);
-    return resident_fn<T, true>(lay, scaled);
+      if (f.id == kStream2) return streamed_fn<T, false>(lay, scaled);
+    if (f.id == kKept) return kept_fn<T, false>(lay, scaled);
+    return f.id == kKeptFold ? kept_fn<T, true>(lay, scaled) : streamed_fn<T, true>(lay, scaled);
   };
-  if constexpr (sizeof(T) == 8) return plan_resident<T>(h, a.sl, a.n, {4, 2}, fn);
-  else return plan_resident<T>(h, a.sl, a.n, {4}, fn);
+  if constexpr (sizeof(T) == 8)
+    return plan_resident<T>(h, a.sl, a.n,
+                            {{4, true, kFoldRows<T>, kKeptFold}, {4, true, INT32_MAX, kKept}, {4, false, INT32_MAX, kStream4},
+                             {2, false, INT32_MAX, kStream2}}, fn);
+  else
+    return plan_resident<T>(h, a.sl, a.n, {{4, true, kFoldRows<T>, kKeptFold}, {4, true, INT32_MAX, kKept}, {4, false, INT32_MAX, kStream4}}, fn);
 }
 template ResidentPlan resident_plan<double>(const rp_handle*, const IterArgs<double>&, bool);
 template ResidentPlan resident_plan<float>(const rp_handle*, const IterArgs<float>&, bool);

@@ -135,7 +135,8 @@ __device__ __forceinline__ void grid_sum(const T (&v)[NV], RsFlags& sh, RsBarrie
 // words and decide alike.
 // (32^3: 7.1k cycles a sum the long way, 600 and 740 of them the two warp sums, 2600
 // the meeting, 1800 the loads and their sum, 770 the division.)
-template <int NV, typename T, typename Fin>
+// FENCE: the block's earlier writes are released, the others' acquired.
+template <int NV, bool FENCE, typename T, typename Fin>
 __device__ __forceinline__ void grid_sum_unit(const T (&v)[NV], int* unit, unsigned long long* words, RsFlags& sh,
                                               RsBarrier& bar, double* partials, int lane, int w, int nw, Fin&& fin) {
   bool quick = gridDim.x < 256;
@@ -176,10 +177,14 @@ __device__ __forceinline__ void grid_sum_unit(const T (&v)[NV], int* unit, unsig
         if (lane == 2 * i) word = lo + (1ull << 56);
         if (lane == 2 * i + 1) word = (unsigned long long)(hi + (1ll << 47)) + (1ull << 56);
       }
+      if (FENCE) __threadfence();
       if (lane < 2 * NV) asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(words + lane), "l"(word) : "memory");
       bool met = false;
       for (int64_t k = 0; k < bar.spin && !met; ++k) {
-        if (lane < 2 * NV) asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(word) : "l"(words + lane) : "memory");
+        if (lane < 2 * NV) {
+          if (FENCE) asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(word) : "l"(words + lane) : "memory");
+          else asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(word) : "l"(words + lane) : "memory");
+        }
         met = __all_sync(0xffffffffu, lane >= 2 * NV || (word >> 56) == gridDim.x);
       }
       bool good = true;
@@ -241,6 +246,52 @@ __device__ __forceinline__ uint32_t ldg_stream(const uint32_t* p) {
   return v;
 }
 
+// Where a product takes its vector from: its value at a global row; at(i): the
+// vector seen from row i.
+// The vector itself:
+template <typename T>
+struct RsGlobal {
+  const T* x;
+  __device__ __forceinline__ T operator()(int g) const { return x[g]; }
+  __device__ __forceinline__ RsGlobal at(int i) const { return RsGlobal{x + i}; }
+};
+// z + beta p, before that sum is anywhere:
+template <typename T>
+struct RsFold {
+  const T* z;
+  const T* p;
+  T beta;
+  __device__ __forceinline__ T operator()(int g) const { return fma(beta, p[g], z[g]); }
+  __device__ __forceinline__ RsFold at(int i) const { return RsFold{z + i, p + i, beta}; }
+};
+
+// The products of a row of the uniform layout in entry order: x seen from the row, L
+// entries, their values val(e), index word wd, table entry tv.
+// (Taking the block's own rows from shared memory instead, under a predicate a lane,
+// lost 4 to 20%: the products are bound by their instructions, and rank boundaries
+// leave a far column in nearly every slice.)
+template <typename T, class G, class Val>
+__device__ __forceinline__ T rs_products(const G& x, bool valid, uint32_t wd, int32_t tv, int L, Val&& val) {
+  T g[8], s = T(0);
+  if (L == 7 && __all_sync(0xffffffffu, valid)) {  // most slices: without a test an entry
+#pragma unroll
+    for (int e = 0; e < 7; ++e) g[e] = x(slice_offset<kIdx4>(wd, e, tv, nullptr, 0));
+#pragma unroll
+    for (int e = 0; e < 7; ++e) s = fma(val(e), g[e], s);
+    return s;
+  }
+#pragma unroll
+  for (int e = 0; e < 8; ++e)
+    if (e < L) {
+      const int off = slice_offset<kIdx4>(wd, e, tv, nullptr, 0);
+      g[e] = valid ? x(off) : T(0);
+    }
+#pragma unroll
+  for (int e = 0; e < 8; ++e)
+    if (e < L) s = fma(val(e), g[e], s);
+  return s;
+}
+
 // A slice of the uniform layout (4-bit indices, 1 to 8 entries a row) held
 // in registers: loaded one slice ahead, across the grid barriers too, so that
 // only the gathers of p wait on memory.
@@ -250,11 +301,11 @@ struct RsSlice {
   uint32_t wd;
   int32_t tv;
   int L;
-  __device__ __forceinline__ void load(const Sliced<T>& sl, uint32_t x0, uint32_t x1, uint32_t y0, uint32_t info, int lane) {
+  __device__ __forceinline__ void load(const Sliced<T>& sl, uint32_t x0, uint32_t x1, uint32_t y0, uint32_t tab, int lane) {
     L = (int)((x1 - x0) >> 5);
     const T* p = sl.vals + x0 + lane;
     wd = ldg_stream(reinterpret_cast<const uint32_t*>(sl.ibuf) + y0 + lane);
-    tv = __ldg(sl.tabs + (info & ~kSliceW4) + (lane & 15));
+    tv = __ldg(sl.tabs + tab + (lane & 15));
     if (L == 7) {  // a cell and its six neighbours: most slices, without a test an entry
 #pragma unroll
       for (int k = 0; k < 7; ++k) v[k] = ldg_stream(p + 32 * k);
@@ -263,27 +314,6 @@ struct RsSlice {
       for (int k = 0; k < 8; ++k)
         if (k < L) v[k] = ldg_stream(p + 32 * k);
     }
-  }
-  // the row's products in entry order; x: the gathered vector at the lane's row
-  __device__ __forceinline__ T sum(const T* x, bool valid) const {
-    T g[8], s = T(0);
-    if (L == 7 && __all_sync(0xffffffffu, valid)) {
-#pragma unroll
-      for (int k = 0; k < 7; ++k) g[k] = x[slice_offset<kIdx4>(wd, k, tv, nullptr, 0)];
-#pragma unroll
-      for (int k = 0; k < 7; ++k) s = fma(v[k], g[k], s);
-      return s;
-    }
-#pragma unroll
-    for (int k = 0; k < 8; ++k)
-      if (k < L) {
-        const int off = slice_offset<kIdx4>(wd, k, tv, nullptr, 0);
-        g[k] = valid ? x[off] : T(0);
-      }
-#pragma unroll
-    for (int k = 0; k < 8; ++k)
-      if (k < L) s = fma(v[k], g[k], s);
-    return s;
   }
 };
 
@@ -329,10 +359,12 @@ __device__ __forceinline__ void st_rows(T* p, const RsPack<T, W>& v, int m, bool
     if (e < m) p[e] = v.e[e];
 }
 
-// The block's slices and their products with a gathered vector.
-template <typename T, int LAY>
+// The block's slices and their products with a gathered vector. MAT (uniform
+// layout): their values and index words stay in shared memory too.
+template <typename T, int LAY, bool MAT = false>
 struct RsMatrix {
   static constexpr bool MP = LAY == kRsParts || LAY == kRsPartsU4, U4 = LAY == kRsU4 || LAY == kRsPartsU4;
+  static_assert(!MAT || U4, "only the uniform layout is kept");
   const Sliced<T>& sl;
   const Parts<T>& parts;
   const int32_t* row_ptr;
@@ -344,16 +376,19 @@ struct RsMatrix {
   uint32_t* sx;     // [cnt + 1], U4: slice s has its index words at 32 s
   uint32_t* sinfo;
   int32_t* snl;     // MP: first non-local entry of the slice's part
-  RsSlice<T> f;     // U4: the slice fetched ahead
+  const T* mv;      // MAT
+  const uint32_t* mw;
+  RsSlice<T> f;     // U4, not MAT: the slice fetched ahead
   NlRange fnl;
 
-  // bytes of the records of `per` slices
-  static int64_t tail_bytes(int lay, int64_t per) {
+  // bytes of the records of `per` slices of at most `width` entries a row
+  static int64_t tail_bytes(int lay, int64_t per, bool mat, int width) {
     const bool mp = lay == kRsParts || lay == kRsPartsU4, u4 = lay == kRsU4 || lay == kRsPartsU4;
-    return lay == kRsCsr ? 0 : (per + 1) * (u4 ? 4 : 8) + per * 4 + (mp ? per * 12 : 0);
+    return (lay == kRsCsr ? 0 : (per + 1) * (u4 ? 4 : 8) + per * 4 + (mp ? per * 12 : 0)) +
+           (mat ? per * kSliceRows * ((int64_t)width * (int64_t)sizeof(T) + 4) : 0);
   }
   __device__ __forceinline__ RsMatrix(const Sliced<T>& sl_, const Parts<T>& parts_, const int32_t* rp, const int32_t* c,
-                                      const T* v, int n_, unsigned char* tail, int per)
+                                      const T* v, int n_, unsigned char* tail, int per, int width)
       : sl(sl_), parts(parts_), row_ptr(rp), col(c), vals(v), n(n_), fnl{0, 0} {
     lane = threadIdx.x & 31;
     w = threadIdx.x >> 5;
@@ -361,6 +396,12 @@ struct RsMatrix {
     const int S = LAY == kRsCsr ? (n + 31) / 32 : (int)sl.n_slices;
     s0 = (int)((int64_t)S * blockIdx.x / gridDim.x);
     cnt = (int)((int64_t)S * (blockIdx.x + 1) / gridDim.x) - s0;
+    if (MAT) {
+      T* m = reinterpret_cast<T*>(tail);
+      mv = m;
+      mw = reinterpret_cast<const uint32_t*>(m + (size_t)per * kSliceRows * width);
+      tail += (size_t)per * kSliceRows * (width * sizeof(T) + 4);
+    }
     srow = reinterpret_cast<int2*>(tail);
     sdesc = reinterpret_cast<uint2*>(srow + (MP ? per : 0));
     sx = reinterpret_cast<uint32_t*>(sdesc);
@@ -372,7 +413,7 @@ struct RsMatrix {
         else sdesc[j] = sl.desc[s0 + j];
       }
       for (int j = threadIdx.x; j < cnt; j += blockDim.x) {
-        sinfo[j] = sl.tinfo[s0 + j];
+        sinfo[j] = U4 ? sl.tinfo[s0 + j] & ~kSliceW4 : sl.tinfo[s0 + j];
         if (MP) {
           const int2 r = sl.srow[s0 + j];
           srow[j] = r;
@@ -381,7 +422,17 @@ struct RsMatrix {
       }
     }
     __syncthreads();
-    if (U4 && w < cnt) fetch(w);
+    if constexpr (MAT) {
+      const uint32_t x0 = sx[0], m = sx[cnt] - x0;
+      T* q = const_cast<T*>(mv);
+      for (uint32_t e = threadIdx.x; e < m; e += blockDim.x) q[e] = ldg_stream(sl.vals + x0 + e);
+      uint32_t* iw = const_cast<uint32_t*>(mw);
+      for (int e = threadIdx.x; e < cnt * kSliceRows; e += blockDim.x)
+        iw[e] = ldg_stream(reinterpret_cast<const uint32_t*>(sl.ibuf) + (size_t)kSliceRows * s0 + e);
+      __syncthreads();
+    } else if (U4 && w < cnt) {
+      fetch(w);
+    }
   }
   // row of slice j for this lane, or -1
   __device__ __forceinline__ int row_of(int j) const {
@@ -411,36 +462,42 @@ struct RsMatrix {
       if (m > 0) f(k, i, m, W == 1 || (!MP && m == W));
     }
   }
+  __device__ __forceinline__ NlRange nl_range(int j) const {
+    const int i = row_of(j);
+    return i >= 0 ? nonlocal_range<T>(parts, srow[j].y >> 6, i) : NlRange{0, 0};
+  }
   __device__ __forceinline__ void fetch(int j) {
     f.load(sl, sx[j], sx[j + 1], (uint32_t)(kSliceRows * (s0 + j)), sinfo[j], lane);
-    if (MP) {
-      const int i = row_of(j);
-      fnl = i >= 0 ? nonlocal_range<T>(parts, srow[j].y >> 6, i) : NlRange{0, 0};
-    }
+    if (MP) fnl = nl_range(j);
   }
-  // slice j's product with x (a vector this kernel writes); i: row_of(j)
-  __device__ __forceinline__ T product(int j, int i, const T* x) {
+  // slice j's product with x; i: row_of(j)
+  template <class G>
+  __device__ __forceinline__ T product(int j, int i, const G& x) {
     const bool valid = i >= 0;
     T sum = T(0);
     if constexpr (U4) {
-      const RsSlice<T> cur = f;
-      const NlRange nl = fnl;
-      fetch(j + nw < cnt ? j + nw : w);  // the last one fetches the first of the next product
-      int g = 0;
-      T gv = T(0);
-      const int nlo = MP ? snl[j] : 0;
-      if (MP && nl.j0 < nl.j1) {  // the first non-local entry alongside the gathers
-        g = __ldg(parts.nl_gcol + nlo + nl.j0);
-        gv = __ldg(parts.nl_vals + nlo + nl.j0);
+      const G xr = x.at(valid ? i : 0);
+      NlRange nl{0, 0};
+      if constexpr (MAT) {
+        if (MP) nl = nl_range(j);
+        const uint32_t x0 = sx[j];
+        const T* v = mv + (x0 - sx[0]) + lane;
+        const int32_t tv = __ldg(sl.tabs + sinfo[j] + (lane & 15));
+        sum = rs_products<T>(xr, valid, mw[j * kSliceRows + lane], tv, (int)((sx[j + 1] - x0) >> 5),
+                             [&](int e) { return v[kSliceRows * e]; });
+      } else {
+        const RsSlice<T> cur = f;
+        nl = fnl;
+        fetch(j + nw < cnt ? j + nw : w);  // the last one fetches the first of the next product
+        sum = rs_products<T>(xr, valid, cur.wd, cur.tv, cur.L, [&](int e) { return cur.v[e]; });
       }
-      sum = cur.sum(x + (valid ? i : 0), valid);
       if (MP && nl.j0 < nl.j1) {
-        sum = fma(gv, x[g], sum);
-        for (int e = nl.j0 + 1; e < nl.j1; ++e)
-          sum = fma(__ldg(parts.nl_vals + nlo + e), x[__ldg(parts.nl_gcol + nlo + e)], sum);
+        const int nlo = snl[j];
+        for (int e = nl.j0; e < nl.j1; ++e)
+          sum = fma(__ldg(parts.nl_vals + nlo + e), x(__ldg(parts.nl_gcol + nlo + e)), sum);
       }
     } else if constexpr (LAY == kRsCsr) {
-      if (valid) sum = row_dot_any<T, true>(parts, row_ptr, col, vals, x, i, n);
+      if (valid) sum = row_dot_any<T, true>(parts, row_ptr, col, vals, x.x, i, n);
     } else {
       const int part_id = MP ? srow[j].y >> 6 : 0;
       NlRange nl{0, 0};
@@ -449,23 +506,32 @@ struct RsMatrix {
       const SliceCk ck = slice_ck<T, MP>(sl, parts, part_id, i, n);
       const uint2 d0 = sdesc[j], d1 = sdesc[j + 1];
       sum = slice_sum<T, true>(d0, d1, sinfo[j], sl.vals + d0.x + lane,
-                               reinterpret_cast<const uint32_t*>(sl.ibuf) + d0.y + lane, sl.tabs, x + (valid ? i : 0),
+                               reinterpret_cast<const uint32_t*>(sl.ibuf) + d0.y + lane, sl.tabs, x.x + (valid ? i : 0),
                                valid, lane, ck);
       if constexpr (MP)
-        if (valid) sum = nonlocal_sum<T, true>(parts, part_id, nl, x, sum);
+        if (valid) sum = nonlocal_sum<T, true>(parts, part_id, nl, x.x, sum);
     }
     return sum;
   }
 };
 
-// The launch of a resident kernel: fn(layout, vectors kept) returns the instance,
-// or nullptr where there is none; the first of the `vecs` counts that fits.
+// The launch of a resident kernel, in one of its forms (the first that fits): how
+// many vectors it keeps in shared memory, whether the matrix too, and at most how
+// many rows a block.
 struct ResidentPlan {
   void* fn = nullptr;  // nullptr: the streaming kernels run
-  int grid = 0, threads = 0, smem = 0, rows = 0;
+  int grid = 0, threads = 0, smem = 0, rows = 0, width = 0;
 };
+struct ResidentForm {
+  int vecs;
+  bool mat;
+  int max_rows;
+  int id;
+};
+// fn_of(layout, form): the instance, or nullptr where there is none
 template <typename T, typename Fn>
-ResidentPlan plan_resident(const rp_handle* h, const Sliced<T>& sl, int64_t n, std::initializer_list<int> vecs, Fn&& fn_of) {
+ResidentPlan plan_resident(const rp_handle* h, const Sliced<T>& sl, int64_t n, std::initializer_list<ResidentForm> forms,
+                           Fn&& fn_of) {
   ResidentPlan p;
   int coop = 0, smem_max = 0;
   if (n == 0) return p;
@@ -483,10 +549,12 @@ ResidentPlan plan_resident(const rp_handle* h, const Sliced<T>& sl, int64_t n, s
   const int64_t S = lay == kRsCsr ? (n + 31) / 32 : sl.n_slices;
   const int grid = (int)std::min<int64_t>(h->num_sms, S);
   const int64_t per = (S + grid - 1) / grid;  // slices a block at most
-  const int64_t tail = RsMatrix<T, kRsCsr>::tail_bytes(lay, per);
-  for (int v : vecs) {
-    void* fn = fn_of(lay, v);
-    const int64_t need = per * 32 * v * (int64_t)sizeof(T) + tail;
+  for (const ResidentForm& f : forms) {
+    if ((f.mat && !u4) || per * 32 > f.max_rows) continue;
+    void* fn = fn_of(lay, f);
+    if (!fn) continue;
+    const int64_t need =
+        per * 32 * f.vecs * (int64_t)sizeof(T) + RsMatrix<T, kRsCsr>::tail_bytes(lay, per, f.mat, h->sl_width);
     const int threads = 32 * (int)std::min<int64_t>(std::max<int64_t>(per, 4), kRsThreads<T> / 32);
     cudaFuncAttributes at;
     int nb = 0;
@@ -495,7 +563,7 @@ ResidentPlan plan_resident(const rp_handle* h, const Sliced<T>& sl, int64_t n, s
         cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max - (int)at.sharedSizeBytes) ==
             cudaSuccess &&
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, threads, (size_t)need) == cudaSuccess && nb >= 1)
-      return ResidentPlan{fn, grid, threads, (int)need, (int)(per * 32)};
+      return ResidentPlan{fn, grid, threads, (int)need, (int)(per * 32), h->sl_width};
     cudaGetLastError();
   }
   return p;

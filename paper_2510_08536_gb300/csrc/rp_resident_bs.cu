@@ -76,7 +76,7 @@ __global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident_bs(const Resident
     sh.be = (T)((sh.rho / sh.rho_old) * (sh.alpha / sh.omega));
   }
   RsMatrix<T, LAY> M(V.sl, V.parts, a.row_ptr, a.col, V.vals, (int)a.n,
-                     reinterpret_cast<unsigned char*>(ts + A.rows), A.rows / 32);
+                     reinterpret_cast<unsigned char*>(ts + A.rows), A.rows / 32, 0);
   const int cnt = M.cnt;
   for (int j = w; j < cnt; j += nw) {
     const int i = M.row_of(j), k = j * 32 + lane;
@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident_bs(const Resident
       for (int j = w; j < cnt; j += nw) {
         const int i = M.row_of(j), k = j * 32 + lane;
         const T rh = i >= 0 ? __ldg(V.rhat + i) : T(0);
-        const T y = M.product(j, i, V.phat);
+        const T y = M.product(j, i, RsGlobal<T>{V.phat});
         if (i >= 0) {
           vs[k] = y;
           acc = fma(rh, y, acc);
@@ -175,7 +175,7 @@ __global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident_bs(const Resident
       T ats = T(0), att = T(0);
       for (int j = w; j < cnt; j += nw) {
         const int i = M.row_of(j), k = j * 32 + lane;
-        const T y = M.product(j, i, V.shat);
+        const T y = M.product(j, i, RsGlobal<T>{V.shat});
         if (i >= 0) {
           ts[k] = y;
           ats = fma(y, rs[k], ats);
@@ -271,7 +271,7 @@ RP_CHECK_TU(resident_bs)
 
 template <typename T>
 ResidentPlan resident_bs_plan(const rp_handle* h, const BsVecs<T>& v) {
-  return plan_resident<T>(h, v.sl, h->n, {4}, [](int lay, int) -> void* {
+  return plan_resident<T>(h, v.sl, h->n, {{4, false, INT32_MAX, 0}}, [](int lay, const ResidentForm&) -> void* {
     switch (lay) {
       case kRsU4: return (void*)k_resident_bs<T, kRsU4>;
       case kRsSliced: return (void*)k_resident_bs<T, kRsSliced>;

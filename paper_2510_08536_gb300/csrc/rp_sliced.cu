@@ -546,6 +546,7 @@ rp_status build_sliced(rp_handle* h, cudaStream_t st) {
   if (herr) return undo(fail(RP_ECUDA, "sliced layout: slice sizes differ between passes"));
   h->sl_slices = S;
   h->sl_u4 = u4 ? 1 : 0;
+  h->sl_width = *std::max_element(hw.begin(), hw.end());
   h->sl_entries = (int64_t)x;
   h->sl_ibuf_len = (int64_t)y;
   h->sl_tabs_len = (int64_t)tabs.size();

@@ -49,16 +49,23 @@ def _solve(h, b, precision, stream=None):
     ((19, 23, 29), (2, 3, 2), {"n_parts": 3}),
     ((37, 29, 31), (2, 2, 2), {"layout": repart.RP_LAYOUT_CSR}),
     ((61, 53, 67), (3, 2, 4), {"symmetric": True}),
+    ((83, 79, 71), (2, 1, 2), {"n_parts": 2}),  # FP32: matrix on chip, FP64: streamed
+    ((97, 96, 95), (2, 2, 2), {}),            # matrix streamed
     ((109, 103, 101), (2, 2, 2), {}),         # FP64: r and q on chip only
 ])
 def test_resident_solves(dims, ranks, kw):
     c = Case(dims, ranks, symmetric=kw.get("symmetric", False))
     ref = pcg_omp.pcg(c.map.row_ptr, c.map.col_idx, c.vals, c.dinv, c.b, tol=1e-9)
     h = repart.build_repartition(c.mesh.ranks, **kw)
-    repart.update_values_packed(h, _t(c.staging))
+    single = repart.build_repartition(c.mesh.ranks, host_loop=1, **kw)
     b = _t(c.b)
     for precision in ("fp64", "mixed", "mixed_ru"):
+        repart.update_values_packed(h, _t(c.staging))
         x, info = _solve(h, b, precision)
+        if c.mesh.n_cells < 100000:  # one iteration a launch: the same sums and states
+            repart.update_values_packed(single, _t(c.staging))
+            x1, info1 = _solve(single, b, precision)
+            assert torch.equal(x, x1) and info == info1, precision
         xs = x.cpu().numpy()
         assert info["status"] == 0, (precision, info)
         assert c.true_rel_residual(xs) <= 1e-9, precision
@@ -66,6 +73,7 @@ def test_resident_solves(dims, ranks, kw):
             assert np.linalg.norm(xs - ref.x) <= 1e-7 * np.linalg.norm(ref.x)
             assert abs(info["iterations"] - ref.iterations) <= 2
     h.close()
+    single.close()
 
 
 @pytest.mark.parametrize("dims,ranks,kw", [
