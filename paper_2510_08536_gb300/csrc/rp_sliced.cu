@@ -217,9 +217,9 @@ __global__ void __launch_bounds__(kThreads)
   }
 }
 
-// The value update of the sliced layout: CSR values, FP32 copies and sliced
-// values of both precisions (SCALED: and the FP32 values of S A S) from the
-// buffer in one pass.
+// The value update of the sliced layout: CSR values, FP32 copies, the inverse
+// diagonal and sliced values of both precisions (SCALED: and the FP32 values of
+// S A S) from the buffer in one pass.
 struct FillArgs {
   int64_t S, n;
   const double* buf;
@@ -235,6 +235,9 @@ struct FillArgs {
   const uint32_t* ibuf;
   const double* s64;
   const float2* s2;
+  const int32_t* diag_pos;
+  double* dinv;
+  float* dinv32;
   double* vals;
   float* vals32;
   double* out;
@@ -242,89 +245,169 @@ struct FillArgs {
   float* out32s;
 };
 
-// One warp a slice. Its rows are one run of CSR entries: the warp reads the
-// run's slots and gathers the buffer coalesced (eight of each in flight),
-// writes the CSR values, keeps the run in shared memory and writes the slice
-// from there, a row a lane. (A permutation to CSR, a gather from CSR to the slices
-// and a third pass for S A S moved 60 bytes an entry where this moves 40: 2.30 ms
-// an update at 256^3 with S A S, 1.27 ms now; 120 us of it here at 128^3, 60% of
-// HBM, bound by the chain row pointer, slot, buffer.) Runs of more than kRun entries (rows longer than 8 on
-// average) gather the slice's entries from the buffer again, rows of more than 8
-// entries and 8-bit indices take the general loop.
+// A slice as the update sees it: its rows, the lane's CSR run (positions in its
+// part) and its place in the layout.
+struct FillSlice {
+  int i, beg, len, dp;
+  uint32_t x0, y0, info;
+  int L;
+  bool valid;
+};
+// The CSR run of a whole slice: m entries from beg of its part.
+struct FillRun {
+  int beg, m, part;
+};
+struct FillRows {
+  int row0, rows, part;
+};
+__device__ __forceinline__ FillRows fill_rows(const FillArgs& A, int s) {
+  if (A.srow) {
+    const int2 r = __ldg(A.srow + s);
+    return FillRows{r.x, r.y & 63, r.y >> 6};
+  }
+  return FillRows{s * kSliceRows, min(kSliceRows, (int)A.n - s * kSliceRows), 0};
+}
+__device__ __forceinline__ FillRun fill_run(const FillArgs& A, int s) {
+  const FillRows r = fill_rows(A, s);
+  const int32_t* rp = A.row_ptr + r.row0 + r.part;
+  const int beg = __ldg(rp);
+  return FillRun{beg, __ldg(rp + r.rows) - beg, r.part};
+}
+template <bool SCALED>
+__device__ __forceinline__ FillSlice fill_slice(const FillArgs& A, int s, int lane) {
+  const FillRows r = fill_rows(A, s);
+  FillSlice v;
+  v.valid = lane < r.rows;
+  v.i = r.row0 + lane;
+  const int32_t* rp = A.row_ptr + v.i + r.part;
+  v.beg = v.valid ? __ldg(rp) : 0;
+  v.len = v.valid ? __ldg(rp + 1) - v.beg : 0;
+  v.dp = v.valid ? __ldg(A.diag_pos + v.i) : 0;
+  const uint2 d0 = __ldg(A.desc + s), d1 = __ldg(A.desc + s + 1);
+  v.x0 = d0.x;
+  v.y0 = d0.y;
+  v.L = (int)((d1.x - d0.x) >> 5);
+  v.info = SCALED ? __ldg(A.tinfo + s) : kSliceW4;
+  return v;
+}
+__device__ __forceinline__ void cp_async4(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async8(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+
+// One warp a slice. Its rows are one run of CSR entries: the run's slots are copied
+// to shared memory two slices ahead, the buffer's values they name one slice ahead
+// (cp.async: the bytes in flight cost no registers), and the warp writes the CSR
+// values, the slice and the diagonal's reciprocals from there. (A permutation to CSR,
+// a gather from CSR to the slices and a third pass for S A S moved 60 bytes an entry
+// where this moves 40.) Runs of more than kRun entries (rows longer than 8 on average)
+// are gathered straight from the buffer; rows of more than 8 entries and 8-bit
+// indices take the general loop.
 constexpr int kRun = 8 * kSliceRows;
+constexpr int kFillSmem = kWarpsPerBlock * kRun * 2 * (8 + 4);
 template <bool FP32, bool SCALED>
 __global__ void __launch_bounds__(kThreads, 4) k_fill_slices(const FillArgs A) {
-  __shared__ double sval[kWarpsPerBlock][kRun];
-  __shared__ float sval32[FP32 ? kWarpsPerBlock : 1][kRun];
+  extern __shared__ __align__(16) unsigned char fbuf[];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  double* sv = sval[w];
-  float* sf = sval32[FP32 ? w : 0];
+  double* sv = reinterpret_cast<double*>(fbuf) + w * 2 * kRun;                                      // [2][kRun]
+  int32_t* ss = reinterpret_cast<int32_t*>(fbuf + kWarpsPerBlock * 2 * kRun * 8) + w * 2 * kRun;    // [2][kRun]
   const int S = (int)A.S, step = gridDim.x * kWarpsPerBlock;
-  for (int s = blockIdx.x * kWarpsPerBlock + w; s < S; s += step) {
-    int row0 = s * kSliceRows, rows = min(kSliceRows, (int)A.n - s * kSliceRows), part = 0;
-    if (A.srow) {
-      const int2 r = __ldg(A.srow + s);
-      row0 = r.x;
-      rows = r.y & 63;
-      part = r.y >> 6;
-    }
-    const bool valid = lane < rows;
-    const int i = row0 + lane;
-    const int32_t* rp = A.row_ptr + i + part;
-    const int beg = valid ? __ldg(rp) : 0, len = valid ? __ldg(rp + 1) - beg : 0;
-    const uint2 d0 = __ldg(A.desc + s), d1 = __ldg(A.desc + s + 1);
-    const uint32_t info = SCALED ? __ldg(A.tinfo + s) : kSliceW4;
-    const int32_t* tab = A.tabs + (info & ~kSliceW4);
-    const int L = (int)((d1.x - d0.x) >> 5);
-    const int beg0 = __shfl_sync(0xffffffffu, beg, 0), m = (int)__reduce_add_sync(0xffffffffu, (unsigned)len);
-    const int at = beg - beg0;
-    const int64_t q0 = __ldg(A.nnz_off + part) + beg0;
+  int s = blockIdx.x * kWarpsPerBlock + w;
+  if (s >= S) return;
+  auto buffer = [&](int part, int64_t& len) {
     const int64_t b0 = __ldg(A.slot_off + (int64_t)part * A.alpha);
-    const int64_t blen = __ldg(A.slot_off + (int64_t)(part + 1) * A.alpha) - b0;
-    const double* buf = A.buf + b0;
+    len = __ldg(A.slot_off + (int64_t)(part + 1) * A.alpha) - b0;
+    return A.buf + b0;
+  };
+  // slots of a run (m entries at most kRun; longer ones are not kept), then their values
+  auto copy_slots = [&](const FillRun& r, int32_t* to) {
+    if (r.m <= kRun) {
+      const int32_t* src = A.src_of + __ldg(A.nnz_off + r.part) + r.beg + lane;
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (32 * u + lane < r.m) cp_async4(to + 32 * u + lane, src + 32 * u);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  auto copy_values = [&](const FillRun& r, const int32_t* from, double* to) {
+    if (r.m <= kRun) {
+      int64_t blen;
+      const double* buf = buffer(r.part, blen);
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (32 * u + lane < r.m) {
+          const int32_t t = from[32 * u + lane];
+          if (RP_IN(t, 0, blen, kChkPermute)) cp_async8(to + 32 * u + lane, buf + t);
+          else to[32 * u + lane] = 0.0;
+        }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  const FillRun none{0, 0, 0};
+  FillRun r0 = fill_run(A, s), r1 = s + step < S ? fill_run(A, s + step) : none,
+          r2 = s + 2 * step < S ? fill_run(A, s + 2 * step) : none;
+  copy_slots(r0, ss);
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  copy_values(r0, ss, sv);
+  copy_slots(r1, ss + kRun);
+  FillSlice next = fill_slice<SCALED>(A, s, lane);
+  for (int b = 0; s < S; s += step, b ^= 1) {
+    const FillSlice v = next;
+    const FillRun run = r0;
+    double* cur = sv + b * kRun;
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncwarp();  // every lane's copies are there, and the slice before is done with its half
+    r0 = r1;
+    copy_values(r0, ss + (b ^ 1) * kRun, sv + (b ^ 1) * kRun);
+    r1 = r2;
+    copy_slots(r1, ss + b * kRun);
+    if (s + step < S) next = fill_slice<SCALED>(A, s + step, lane);
+    r2 = s + 3 * step < S ? fill_run(A, s + 3 * step) : none;
+
+    const int i = v.i, at = v.beg - run.beg;
+    const int32_t* tab = A.tabs + (v.info & ~kSliceW4);
+    const int64_t q0 = __ldg(A.nnz_off + run.part) + run.beg;
     float2 si = make_float2(0.f, 0.f);
-    if (SCALED && valid) si = __ldg(A.s2 + i);
-    // entry v with the column's scale sj, offset id of the slice's table
-    auto scaled = [&](double v, float2 sj, uint32_t id) {
+    if (SCALED && v.valid) si = __ldg(A.s2 + i);
+    // entry x with the column's scale sj, offset id of the slice's table
+    auto scaled = [&](double x, float2 sj, uint32_t id) {
       bool ok;
-      float f = scaled_value(v, si, sj, ok);
+      float f = scaled_value(x, si, sj, ok);
       if (!ok) {
         const int j = i + __ldg(tab + id);
-        f = RP_IN(j, 0, A.n, kChkGather) ? (float)(v * (__ldg(A.s64 + i) * __ldg(A.s64 + j))) : 0.f;
+        f = RP_IN(j, 0, A.n, kChkGather) ? (float)(x * (__ldg(A.s64 + i) * __ldg(A.s64 + j))) : 0.f;
       }
       return f;
     };
-    const int32_t* src = A.src_of + q0 + lane;
-    double* cv = A.vals + q0 + lane;
-    double* out = A.out + d0.x + lane;
-    float* out32 = FP32 ? A.out32 + d0.x + lane : nullptr;
-    float* out32s = SCALED ? A.out32s + d0.x + lane : nullptr;
-    __syncwarp();  // the previous slice's readers of sv are done
-    for (int c = 0; c < m; c += kRun, src += kRun, cv += kRun) {
-      const int rest = m - c - lane;
-      int32_t t[8];
-      double v[8];
+    const bool kept = run.m <= kRun;
+    int64_t blen = 0;
+    const double* buf = kept ? nullptr : buffer(run.part, blen);
+    auto entry = [&](int k) { return kept ? cur[k] : slot_value(buf, __ldg(A.src_of + q0 + k), blen); };
+    for (int c = 0; c < run.m; c += kRun) {
+      double* cv = A.vals + q0 + c + lane;
+      float* cv32 = FP32 ? A.vals32 + q0 + c + lane : nullptr;
 #pragma unroll
       for (int u = 0; u < 8; ++u)
-        if (32 * u < rest) t[u] = __ldcs(src + 32 * u);
-#pragma unroll
-      for (int u = 0; u < 8; ++u)
-        if (32 * u < rest) v[u] = slot_value(buf, t[u], blen);
-#pragma unroll
-      for (int u = 0; u < 8; ++u)
-        if (32 * u < rest) {
-          __stcs(cv + 32 * u, v[u]);
-          sv[32 * u + lane] = v[u];
-          if (FP32) {
-            const float f = f32_rn(v[u]);
-            __stcs(A.vals32 + (cv - A.vals) + 32 * u, f);
-            sf[32 * u + lane] = f;
-          }
+        if (c + 32 * u + lane < run.m) {
+          const double x = entry(c + 32 * u + lane);
+          __stcs(cv + 32 * u, x);
+          if (FP32) __stcs(cv32 + 32 * u, f32_rn(x));
         }
     }
-    __syncwarp();
-    if (m <= kRun && L <= 8 && (info & kSliceW4)) {
-      const uint32_t wd = SCALED ? __ldg(A.ibuf + d0.y + lane) : 0u;
+    if (v.valid && RP_IN(v.dp, v.beg, v.beg + v.len, kChkSliceValues)) {
+      const double d = entry(v.dp - run.beg);
+      A.dinv[i] = recip_rn(d);
+      if (FP32) A.dinv32[i] = 1.0f / f32_rn(d);
+    }
+    double* out = A.out + v.x0 + lane;
+    float* out32 = FP32 ? A.out32 + v.x0 + lane : nullptr;
+    float* out32s = SCALED ? A.out32s + v.x0 + lane : nullptr;
+    if (kept && v.L <= 8 && (v.info & kSliceW4)) {
+      const uint32_t wd = SCALED ? __ldg(A.ibuf + v.y0 + lane) : 0u;
       const int32_t tv = SCALED ? __ldg(tab + (lane & 15)) : 0;
 #pragma unroll
       for (int u0 = 0; u0 < 8; u0 += 4) {  // in halves: the gathered scales of all eight spill
@@ -332,40 +415,40 @@ __global__ void __launch_bounds__(kThreads, 4) k_fill_slices(const FillArgs A) {
         if (SCALED) {
 #pragma unroll
           for (int u = u0; u < u0 + 4; ++u)
-            if (u < L) {
+            if (u < v.L) {
               const int off = __shfl_sync(0xffffffffu, tv, (int)(wd >> (4 * u)), 16);
-              sj[u - u0] = u < len && RP_IN(i + off, 0, A.n, kChkGather) ? __ldg(A.s2 + i + off) : make_float2(0.f, 0.f);
+              sj[u - u0] = u < v.len && RP_IN(i + off, 0, A.n, kChkGather) ? __ldg(A.s2 + i + off) : make_float2(0.f, 0.f);
             }
         }
 #pragma unroll
         for (int u = u0; u < u0 + 4; ++u)
-          if (u < L) {
-            const bool has = u < len;
-            const double v = has ? sv[at + u] : 0.0;
-            __stcs(out + kSliceRows * u, v);
-            if (FP32) __stcs(out32 + kSliceRows * u, has ? sf[at + u] : 0.f);
-            if (SCALED) __stcs(out32s + kSliceRows * u, has ? scaled(v, sj[u - u0], (wd >> (4 * u)) & 15u) : 0.f);
+          if (u < v.L) {
+            const bool has = u < v.len;
+            const double x = has ? cur[at + u] : 0.0;
+            __stcs(out + kSliceRows * u, x);
+            if (FP32) __stcs(out32 + kSliceRows * u, has ? f32_rn(x) : 0.f);
+            if (SCALED) __stcs(out32s + kSliceRows * u, has ? scaled(x, sj[u - u0], (wd >> (4 * u)) & 15u) : 0.f);
           }
       }
     } else {
-      const int per = (info & kSliceW4) ? 8 : 4, bits = (info & kSliceW4) ? 4 : 8;
-      for (int k = 0; k < L; ++k) {
-        const bool has = k < len;
-        double v = 0.0;
-        if (has) v = m <= kRun ? sv[at + k] : slot_value(buf, A.src_of[q0 + at + k], blen);
-        __stcs(out + kSliceRows * k, v);
-        if (FP32) __stcs(out32 + kSliceRows * k, has ? f32_rn(v) : 0.f);
+      const int per = (v.info & kSliceW4) ? 8 : 4, bits = (v.info & kSliceW4) ? 4 : 8;
+      for (int k = 0; k < v.L; ++k) {
+        const bool has = k < v.len;
+        const double x = has ? entry(at + k) : 0.0;
+        __stcs(out + kSliceRows * k, x);
+        if (FP32) __stcs(out32 + kSliceRows * k, has ? f32_rn(x) : 0.f);
         if (SCALED) {
           float f = 0.f;
-          const uint32_t wd = __ldg(A.ibuf + d0.y + (uint32_t)(kSliceRows * (k / per)) + lane);
+          const uint32_t wd = __ldg(A.ibuf + v.y0 + (uint32_t)(kSliceRows * (k / per)) + lane);
           const uint32_t id = (wd >> (bits * (k % per))) & ((1u << bits) - 1u);
           const int off = __ldg(tab + id);
-          if (has && RP_IN(i + off, 0, A.n, kChkGather)) f = scaled(v, __ldg(A.s2 + i + off), id);
+          if (has && RP_IN(i + off, 0, A.n, kChkGather)) f = scaled(x, __ldg(A.s2 + i + off), id);
           __stcs(out32s + kSliceRows * k, f);
         }
       }
     }
   }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
 
 template <typename T>
@@ -554,7 +637,7 @@ rp_status build_sliced(rp_handle* h, cudaStream_t st) {
 }
 
 // s_i = 1 / sqrt(a_ii): FP64 square root and division (both correctly rounded), from
-// the current values (the value update computes them itself, k_dinv)
+// the current values (the value update computes them itself, k_diagonal)
 __global__ void __launch_bounds__(kThreads)
     k_scaling(int64_t n, const int32_t* __restrict__ diag_pos, const double* __restrict__ vals, int64_t nnz,
               double* __restrict__ s64, float2* __restrict__ s2) {
@@ -627,12 +710,17 @@ RP_CHECK_TU(sliced)
 rp_status fill_sliced(rp_handle* h, const double* buf, cudaStream_t s) {
   const FillArgs a{h->sl_slices, h->n, buf, h->d_slot_off, h->k / h->n_parts, h->d_part_nnz_off, h->sl_srow,
                    h->row_ptr, h->src_of, h->sl_desc, h->sl_tinfo, h->sl_tabs,
-                   reinterpret_cast<const uint32_t*>(h->sl_ibuf), h->s64, h->s2, h->vals, h->vals32, h->sl_vals,
+                   reinterpret_cast<const uint32_t*>(h->sl_ibuf), h->s64, h->s2, h->diag_pos, h->dinv, h->dinv32, h->vals, h->vals32, h->sl_vals,
                    h->sl_vals32, h->sl_vals32s};
-  const int g = slice_grid(h, h->sl_slices);
-  if (h->sl_vals32s) k_fill_slices<true, true><<<g, kThreads, 0, s>>>(a);
-  else if (h->sl_vals32) k_fill_slices<true, false><<<g, kThreads, 0, s>>>(a);
-  else k_fill_slices<false, false><<<g, kThreads, 0, s>>>(a);
+  // four blocks an SM (shared memory and registers)
+  const int64_t want = (h->sl_slices + kWarpsPerBlock - 1) / kWarpsPerBlock;
+  const int g = (int)std::min<int64_t>(want, (int64_t)h->num_sms * 4);
+  void* fn = h->sl_vals32s  ? (void*)k_fill_slices<true, true>
+             : h->sl_vals32 ? (void*)k_fill_slices<true, false>
+                            : (void*)k_fill_slices<false, false>;
+  RP_TRY_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kFillSmem));
+  void* args[1] = {const_cast<FillArgs*>(&a)};
+  RP_TRY_CUDA(cudaLaunchKernel(fn, dim3((unsigned)g), dim3(kThreads), args, (size_t)kFillSmem, s));
   RP_TRY_CUDA(cudaGetLastError());
   return RP_OK;
 }

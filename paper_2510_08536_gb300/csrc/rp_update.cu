@@ -61,20 +61,21 @@ __global__ void __launch_bounds__(kThreads)
   }
 }
 
-// Jacobi diagonal straight from the diagonal block of each rank (contiguous
-// in the buffer): dinv[i] = 1 / a_ii, and 1/(float)a_ii for the FP32 copy.
-// s64: also the scaling s_i = 1/sqrt(a_ii) of S A S and its FP32 pair (one
-// part; the same values the merged diagonal holds).
-template <bool FP32>
+// From the diagonal straight out of the diagonal block of each rank (contiguous in
+// the buffer), DINV: dinv[i] = 1 / a_ii, and 1/(float)a_ii for the FP32 copy (where the
+// sliced update does not write them); s64: the scaling s_i = 1/sqrt(a_ii) of S A S and
+// its FP32 pair (one part; the same values the merged diagonal holds).
+template <bool DINV>
 __global__ void __launch_bounds__(kThreads)
-    k_dinv(const double* __restrict__ buf, const int64_t* __restrict__ row_off,
-           const int64_t* __restrict__ slot_off, int k, double* __restrict__ dinv,
-           float* __restrict__ dinv32, double* __restrict__ s64, float2* __restrict__ s2) {
+    k_diagonal(const double* __restrict__ buf, const int64_t* __restrict__ row_off,
+               const int64_t* __restrict__ slot_off, int k, double* __restrict__ dinv, float* __restrict__ dinv32,
+               double* __restrict__ s64, float2* __restrict__ s2) {
   for_ranked(row_off, k, [&](int r, int64_t i) {
     const double d = __ldcs(buf + __ldg(slot_off + r) + (i - __ldg(row_off + r)));
-    dinv[i] = recip_rn(d);
-    if (FP32) dinv32[i] = 1.0f / f32_rn(d);
-    if (s64) {
+    if (DINV) {
+      dinv[i] = recip_rn(d);
+      if (dinv32) dinv32[i] = 1.0f / f32_rn(d);
+    } else {
       const double sc = recip_rn(sqrt_rn(d));
       s64[i] = sc;
       s2[i] = scale_pair(sc);
@@ -83,14 +84,12 @@ __global__ void __launch_bounds__(kThreads)
 }
 
 static rp_status permute_all(rp_handle* h, const double* buf, cudaStream_t s) {
-  if (h->n > 0) {
-    if (h->want_fp32)
-      k_dinv<true><<<grid_for(h, h->n / 4), kThreads, 0, s>>>(buf, h->d_row_off, h->d_slot_off, h->k, h->dinv, h->dinv32,
-                                                              h->sl_vals32s ? h->s64 : nullptr, h->s2);
-    else
-      k_dinv<false><<<grid_for(h, h->n / 4), kThreads, 0, s>>>(buf, h->d_row_off, h->d_slot_off, h->k, h->dinv, nullptr,
-                                                               nullptr, nullptr);
-  }
+  const int gd = grid_for(h, h->n / 4);
+  if (h->n > 0 && h->sl_vals32s)
+    k_diagonal<false><<<gd, kThreads, 0, s>>>(buf, h->d_row_off, h->d_slot_off, h->k, nullptr, nullptr, h->s64, h->s2);
+  if (h->n > 0 && h->sl_slices == 0)
+    k_diagonal<true><<<gd, kThreads, 0, s>>>(buf, h->d_row_off, h->d_slot_off, h->k, h->dinv,
+                                             h->want_fp32 ? h->dinv32 : nullptr, nullptr, nullptr);
   if (h->sl_slices > 0) {
     RP_TRY(fill_sliced(h, buf, s));
   } else {
