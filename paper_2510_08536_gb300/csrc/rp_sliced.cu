@@ -306,7 +306,11 @@ __device__ __forceinline__ void cp_async8(void* dst, const void* src) {
 // a gather from CSR to the slices and a third pass for S A S moved 60 bytes an entry
 // where this moves 40.) Runs of more than kRun entries (rows longer than 8 on average)
 // are gathered straight from the buffer; rows of more than 8 entries and 8-bit
-// indices take the general loop.
+// indices take the general loop. Plain stores: streaming ones (evict first) cost 2%,
+// the runs' ends share sectors. 256^3 with S A S: 1.21 ms an update, 0.19 ms of it the
+// diagonal pass, 4.7 GB at 0.7 of the copy rate (bound by issue and the mix of nine
+// streams read and written; two separate gathers took 2.30 ms, one without the copies
+// ahead 1.28 ms).
 constexpr int kRun = 8 * kSliceRows;
 constexpr int kFillSmem = kWarpsPerBlock * kRun * 2 * (8 + 4);
 template <bool FP32, bool SCALED>
@@ -394,8 +398,8 @@ __global__ void __launch_bounds__(kThreads, 4) k_fill_slices(const FillArgs A) {
       for (int u = 0; u < 8; ++u)
         if (c + 32 * u + lane < run.m) {
           const double x = entry(c + 32 * u + lane);
-          __stcs(cv + 32 * u, x);
-          if (FP32) __stcs(cv32 + 32 * u, f32_rn(x));
+          cv[32 * u] = x;
+          if (FP32) cv32[32 * u] = f32_rn(x);
         }
     }
     if (v.valid && RP_IN(v.dp, v.beg, v.beg + v.len, kChkSliceValues)) {
@@ -425,9 +429,9 @@ __global__ void __launch_bounds__(kThreads, 4) k_fill_slices(const FillArgs A) {
           if (u < v.L) {
             const bool has = u < v.len;
             const double x = has ? cur[at + u] : 0.0;
-            __stcs(out + kSliceRows * u, x);
-            if (FP32) __stcs(out32 + kSliceRows * u, has ? f32_rn(x) : 0.f);
-            if (SCALED) __stcs(out32s + kSliceRows * u, has ? scaled(x, sj[u - u0], (wd >> (4 * u)) & 15u) : 0.f);
+            out[kSliceRows * u] = x;
+            if (FP32) out32[kSliceRows * u] = has ? f32_rn(x) : 0.f;
+            if (SCALED) out32s[kSliceRows * u] = has ? scaled(x, sj[u - u0], (wd >> (4 * u)) & 15u) : 0.f;
           }
       }
     } else {
@@ -435,15 +439,15 @@ __global__ void __launch_bounds__(kThreads, 4) k_fill_slices(const FillArgs A) {
       for (int k = 0; k < v.L; ++k) {
         const bool has = k < v.len;
         const double x = has ? entry(at + k) : 0.0;
-        __stcs(out + kSliceRows * k, x);
-        if (FP32) __stcs(out32 + kSliceRows * k, has ? f32_rn(x) : 0.f);
+        out[kSliceRows * k] = x;
+        if (FP32) out32[kSliceRows * k] = has ? f32_rn(x) : 0.f;
         if (SCALED) {
           float f = 0.f;
           const uint32_t wd = __ldg(A.ibuf + v.y0 + (uint32_t)(kSliceRows * (k / per)) + lane);
           const uint32_t id = (wd >> (bits * (k % per))) & ((1u << bits) - 1u);
           const int off = __ldg(tab + id);
           if (has && RP_IN(i + off, 0, A.n, kChkGather)) f = scaled(x, __ldg(A.s2 + i + off), id);
-          __stcs(out32s + kSliceRows * k, f);
+          out32s[kSliceRows * k] = f;
         }
       }
     }
