@@ -43,13 +43,6 @@ struct RsShared : RsFlags {
   int unit[3];  // of (p, q), (r, z) and (r, r)
 };
 
-// a / b in T, for the finite a, b > 0 of an iteration that goes on without the FP64 pipe
-template <typename T>
-__device__ __forceinline__ T ratio(double a, double b) {
-  if constexpr (sizeof(T) == 8) return quot_rn(a, b);
-  else return f32_rn(quot_rn(a, b));
-}
-
 // LAY: layout of the product; SCALED: the system S A S (z = r); ALL: r, x, p
 // and q in shared memory, else r and q; MAT: the matrix too; FOLD: no barrier C (the
 // product gathers z + beta p of the two vectors, which are written to global memory
@@ -140,7 +133,7 @@ __global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident(const ResidentArg
     // every block has left the sums of the iteration before: their accumulators are
     // cleared for the one after the next (seen by all behind barrier C)
     const int free_set = set == 0 ? 2 : set - 1;
-    if (blockIdx.x == 0 && tid < 8) rs_words(A.sync, free_set, 0)[tid] = 0ull;
+    if (blockIdx.x == 0 && tid < 8) rs_words(A.sync, free_set, 0)[tid] = 0ull;  // two sums
     // B: r -= alpha q, z = D^-1 r (kept in q's place), x += alpha p, (r, z), (r, r)
     const T alpha = sh.alpha;
     T rza = T(0), rra = T(0);

@@ -36,14 +36,15 @@ struct RsFlags {
 
 // Memory of the grid barrier and sums (rp_handle::rsync), cleared before each
 // solve: the arrival counter, its base of the next launch, the set of accumulators
-// that is next and the units of the sums; three sets of 4 words for each of two sums.
-constexpr int kRsCount = 0, kRsBase = 32, kRsSet = 33, kRsUnit = 34, kRsWords = 64, kRsSync = 128;
+// that is next and the units of the sums; three sets of 4 words for each of four sums.
+constexpr int kRsCount = 0, kRsBase = 32, kRsSet = 33, kRsUnit = 34, kRsWords = 64, kRsSetWords = 16;
+constexpr int kRsSync = kRsWords + 3 * 2 * kRsSetWords;
 __device__ __forceinline__ void rs_reset(unsigned int* sync) {
   for (int k = threadIdx.x; k < kRsSync; k += blockDim.x)
     sync[k] = k >= kRsUnit && k < kRsWords ? (unsigned int)kFixNoUnit : 0u;
 }
 __device__ __forceinline__ unsigned long long* rs_words(unsigned int* sync, int set, int sum) {
-  return reinterpret_cast<unsigned long long*>(sync + kRsWords) + set * 8 + sum * 4;
+  return reinterpret_cast<unsigned long long*>(sync + kRsWords) + set * kRsSetWords + sum * 4;
 }
 
 // One block's arrival at the grid barrier and its wait for all others (one
@@ -107,21 +108,7 @@ __device__ __forceinline__ void warp_sums(const T (&v)[NV], RsFlags& sh, int lan
 
 // Grid sum of NV values a thread. Warp 0 of every block receives the totals in
 // tot[] (all lanes) and calls fin(tot); then the block goes on together.
-template <int NV, typename T, typename Fin>
-__device__ __forceinline__ void grid_sum(const T (&v)[NV], RsFlags& sh, RsBarrier& bar, double* partials, int lane,
-                                         int w, int nw, Fin&& fin) {
-  warp_sums(v, sh, lane, w);
-  __syncthreads();
-  if (w == 0) {
-    double tot[NV];
-    const bool ok = grid_total<NV>(sh, bar, partials, lane, nw, tot);
-    if (lane == 0 && !ok) sh.bad = 1;
-    fin(tot);
-  }
-  __syncthreads();
-}
-
-// The same for sums that change little from one iteration to the next: unit[i],
+// For sums that change little from one iteration to the next: unit[i],
 // kept over the iterations, is 2^-80 of the last total. The threads' values
 // become integers in that unit (fix_digits), the warps and the block add
 // integers, and the block adds its sum, rounded to 2^-66 of the last total, to two
@@ -227,6 +214,13 @@ __device__ __forceinline__ void grid_sum_unit(const T (&v)[NV], int* unit, unsig
     fin(tot);
   }
   __syncthreads();
+}
+
+// a / b in T without the FP64 pipe (finite a, b > 0; else as the division)
+template <typename T>
+__device__ __forceinline__ T ratio(double a, double b) {
+  if constexpr (sizeof(T) == 8) return quot_rn(a, b);
+  else return f32_rn(quot_rn(a, b));
 }
 
 // read-only data of one pass an iteration: not worth a line of L1

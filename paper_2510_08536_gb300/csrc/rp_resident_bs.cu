@@ -33,6 +33,7 @@ struct BsShared : RsFlags {
   T al, om, be;
   double rho, rho_old, alpha, omega, rr, ss;
   int iter, status, done;
+  int unit[6];  // of (rhat, v), (s, s), (t, s), (t, t), (r, r), (rhat, r)
 };
 
 template <typename T>
@@ -60,6 +61,7 @@ __global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident_bs(const Resident
   const bool x16 = (reinterpret_cast<uintptr_t>(xg) & 15) == 0;  // the caller's may not be
 
   RsBarrier bar{A.sync + kRsCount, A.sync[kRsBase], A.spin};
+  int set = (int)A.sync[kRsSet];  // accumulators of this iteration's sums
   const double thresh = c->ithresh;
   const int max_iter = c->max_iter;
   if (tid == 0) {
@@ -71,7 +73,8 @@ __global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident_bs(const Resident
     sh.ss = c->ss;
     sh.iter = c->iter;
     sh.status = c->status;
-    sh.bad = sh.stop = sh.done = 0;
+    sh.bad = sh.stop = sh.done = sh.over = 0;
+    for (int k = 0; k < 6; ++k) sh.unit[k] = (int)A.sync[kRsUnit + k];
     sh.om = (T)sh.omega;
     sh.be = (T)((sh.rho / sh.rho_old) * (sh.alpha / sh.omega));
   }
@@ -123,18 +126,21 @@ __global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident_bs(const Resident
         }
       }
       const T v[1] = {acc};
-      grid_sum<1>(v, sh, bar, part, lane, w, nw, [&](const double (&tot)[1]) {
+      grid_sum_unit<1, false>(v, sh.unit, rs_words(A.sync, set, 0), sh, bar, part, lane, w, nw, [&](const double (&tot)[1]) {
         if (lane != 0) return;
         if (tot[0] == 0.0 || !isfinite(tot[0])) {
           sh.status = RP_BREAKDOWN;
           sh.stop = 1;
         } else {
-          sh.alpha = sh.rho / tot[0];
+          sh.alpha = quot_rn(sh.rho, tot[0]);
           sh.al = (T)sh.alpha;
         }
       });
     }
     if (sh.bad || sh.stop) break;
+    // every block has left the sums of the iteration before: their accumulators are
+    // cleared for the one after the next (seen by all behind the next barrier)
+    if (blockIdx.x == 0 && tid < kRsSetWords) rs_words(A.sync, set == 0 ? 2 : set - 1, 0)[tid] = 0ull;
     const T al = sh.al;
     // B3
     {
@@ -152,7 +158,7 @@ __global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident_bs(const Resident
         st_rows<W>(V.shat + i, h, m, whole);
       });
       const T v[1] = {acc};
-      grid_sum<1>(v, sh, bar, part2, lane, w, nw, [&](const double (&tot)[1]) {
+      grid_sum_unit<1, true>(v, sh.unit + 1, rs_words(A.sync, set, 1), sh, bar, part2, lane, w, nw, [&](const double (&tot)[1]) {
         if (lane != 0) return;
         sh.ss = tot[0];
         if (tot[0] <= thresh) sh.stop = 3;
@@ -183,9 +189,9 @@ __global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident_bs(const Resident
         }
       }
       const T v[2] = {ats, att};
-      grid_sum<2>(v, sh, bar, part, lane, w, nw, [&](const double (&tot)[2]) {
+      grid_sum_unit<2, false>(v, sh.unit + 2, rs_words(A.sync, set, 2), sh, bar, part, lane, w, nw, [&](const double (&tot)[2]) {
         if (lane != 0) return;
-        const double om = tot[0] / tot[1];
+        const double om = quot_rn(tot[0], tot[1]);
         if (!(tot[1] > 0.0) || !isfinite(om)) {
           sh.status = RP_BREAKDOWN;
           sh.stop = 1;
@@ -217,7 +223,7 @@ __global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident_bs(const Resident
         st_pack<W>(rs + k, r);
       });
       const T v[2] = {arr, arh};
-      grid_sum<2>(v, sh, bar, part2, lane, w, nw, [&](const double (&tot)[2]) {
+      grid_sum_unit<2, false>(v, sh.unit + 4, rs_words(A.sync, set, 3), sh, bar, part2, lane, w, nw, [&](const double (&tot)[2]) {
         if (lane != 0) return;
         sh.rr = tot[0];
         ++sh.iter;
@@ -230,11 +236,12 @@ __global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident_bs(const Resident
         } else {
           sh.rho_old = sh.rho;
           sh.rho = tot[1];
-          sh.be = (T)((sh.rho / sh.rho_old) * (sh.alpha / sh.omega));
+          sh.be = (T)(quot_rn(sh.rho, sh.rho_old) * quot_rn(sh.alpha, sh.omega));
         }
         sh.stop = stop;
       });
     }
+    set = set == 2 ? 0 : set + 1;
     if (sh.bad || sh.stop) break;
   }
   if (sh.stop == 2) {  // the state back to memory for the next launch
@@ -248,6 +255,8 @@ __global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident_bs(const Resident
   }
   if (blockIdx.x == 0 && tid == 0) {
     A.sync[kRsBase] = bar.target;
+    A.sync[kRsSet] = (unsigned int)(sh.stop == 3 ? (set == 2 ? 0 : set + 1) : set);
+    for (int k = 0; k < 6; ++k) A.sync[kRsUnit + k] = (unsigned int)sh.unit[k];
     c->iter = sh.iter;
     c->rho = sh.rho;
     c->rho_old = sh.rho_old;
