@@ -1043,7 +1043,7 @@ extern "C" rp_status rp_batch_autotune(rp_handle* h, const double* buffer, const
   // team counts between these shapes matter: with the largest systems first,
   // too many small teams leave the largest system's team running alone at
   // the end, too few large teams pay more barrier latency per iteration
-  const int clusters[] = {2, 3, 4, 5, 6, 8, 10, 12, 16};
+  const int clusters[] = {2, 3, 4, 5, 6, 8, 16};
   const int threads[] = {256, 512};
   cudaEvent_t e0, e1;
   RP_TRY_CUDA(cudaEventCreate(&e0));
