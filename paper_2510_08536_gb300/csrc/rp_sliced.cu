@@ -312,7 +312,8 @@ __device__ __forceinline__ void cp_async8(void* dst, const void* src) {
 // streams read and written; two separate gathers took 2.30 ms, one without the copies
 // ahead 1.28 ms).
 constexpr int kRun = 8 * kSliceRows;
-constexpr int kFillSmem = kWarpsPerBlock * kRun * 2 * (8 + 4);
+constexpr int kFillSmem = kWarpsPerBlock * kRun * 2 * (8 + 4);  // 48 KB, no more than a launch may ask for by default
+static_assert(kFillSmem <= 48 * 1024, "opt in");
 template <bool FP32, bool SCALED>
 __global__ void __launch_bounds__(kThreads, 4) k_fill_slices(const FillArgs A) {
   extern __shared__ __align__(16) unsigned char fbuf[];
@@ -719,12 +720,9 @@ rp_status fill_sliced(rp_handle* h, const double* buf, cudaStream_t s) {
   // four blocks an SM (shared memory and registers)
   const int64_t want = (h->sl_slices + kWarpsPerBlock - 1) / kWarpsPerBlock;
   const int g = (int)std::min<int64_t>(want, (int64_t)h->num_sms * 4);
-  void* fn = h->sl_vals32s  ? (void*)k_fill_slices<true, true>
-             : h->sl_vals32 ? (void*)k_fill_slices<true, false>
-                            : (void*)k_fill_slices<false, false>;
-  RP_TRY_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kFillSmem));
-  void* args[1] = {const_cast<FillArgs*>(&a)};
-  RP_TRY_CUDA(cudaLaunchKernel(fn, dim3((unsigned)g), dim3(kThreads), args, (size_t)kFillSmem, s));
+  if (h->sl_vals32s) k_fill_slices<true, true><<<g, kThreads, kFillSmem, s>>>(a);
+  else if (h->sl_vals32) k_fill_slices<true, false><<<g, kThreads, kFillSmem, s>>>(a);
+  else k_fill_slices<false, false><<<g, kThreads, kFillSmem, s>>>(a);
   RP_TRY_CUDA(cudaGetLastError());
   return RP_OK;
 }
