@@ -726,8 +726,10 @@ def run_ours(args):
 
     def launches(prec, info):
         per_pass = {"fp64": 1, "mixed": 2, "mixed_ru": 3}[prec]  # residual (+ correction, + p continuation)
-        solve = 1 + 3 * info["iterations"] + per_pass * info["passes"]
-        return 2 + (1 if sliced else 0) + solve  # permutation + Jacobi diagonal (+ sliced values)
+        # three kernels an iteration, or the resident kernel once a pass (vectors that fit the chip)
+        inner = info["passes"] if mesh.n_cells <= 2_100_000 else 3 * info["iterations"]
+        update = (1 if prec == "fp64" else 2) if sliced else 2  # all values (+ scaling); permutation + diagonal
+        return update + 1 + inner + per_pass * info["passes"]
 
     results = {}
     clocks = {}

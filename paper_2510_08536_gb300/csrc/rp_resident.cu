@@ -5,28 +5,37 @@
 // 20 us an iteration however small the system is: three launches, two block
 // elections and the latency of cold pipelines. Systems whose vectors fit the
 // SMs' shared memory (152 x 227 KB) need none of it: block b owns a contiguous
-// run of 32-row slices and keeps r, x, p and q of those rows in shared memory
-// (FP64 beyond 7,200 rows an SM: r and q); only p, which the products gather
-// across blocks, is also written to global memory, and the matrix streams from
-// L2. The grid meets three times an iteration:
+// run of 32-row slices and keeps r, x, p and q of those rows in shared memory;
+// only p, which the products gather across blocks, is also written to global
+// memory. The grid meets three times an iteration:
 //   A  q = A p,                             (p, q)          | sum -> alpha
 //   B  r -= alpha q, z = D^-1 r, x += alpha p, (r, z), (r, r) | sum -> beta, stop test
 //   C  p = z + beta p                                       | barrier
-// with the arithmetic of K1-K3, row by row the same fused multiply-adds; the
-// dot products are summed per thread, warp and block and over the blocks in
-// block order (rp_reduce.cuh), every block summing all partials itself, so all
-// blocks hold the same scalars and take the same branches.
+// with the arithmetic of K1-K3, row by row the same fused multiply-adds. The sums
+// are the same integers in every block (grid_sum_unit), so all blocks hold the same
+// scalars and take the same branches.
+//
+// Forms (resident_plan takes the first that fits):
+//   matrix kept too, C folded into the next A: at most one slice a warp (117k rows
+//     in FP64, 156k in FP32); the product gathers z + beta p
+//   matrix kept: to 380k rows in FP64, 725k in FP32; its values stay off L2
+//   vectors kept, matrix from L2 one slice ahead: to 1.1M rows in FP64, 2.2M in FP32
+//   r and q kept (FP64): to 2.2M rows
+// us an iteration (streaming kernels, then this): 32^3 FP64 19.7 -> 6.8, 97x61x83 FP32
+// 32.6 -> 9.1, 64^3 FP64 34.5 -> 13.5, 128^3 FP64 91.7 -> 61.9, 128^3 FP32 on 8 parts
+// 51.4 -> 39.
 //
 // The barrier is an arrival counter in L2 (red.release, ld.acquire polls of one
-// thread a block): 1.3 us on 152 SMs. (Flags with the partial sums as payload,
-// polled by all blocks, took 5-8 us: the polls delay the writes they wait for.)
-// The launch is cooperative, so all blocks are resident; every wait is bounded
-// by spin probes all the same and ends the solve with RP_DEVICE_TIMEOUT.
+// thread a block): 1.3 us on 152 SMs. (Flags with the partial sums as payload took
+// 5400 to 6700 cycles a sum with any number of replicas polled: the polls delay the
+// writes they wait for.) The launch is cooperative, so all blocks are resident; every
+// wait is bounded by spin probes all the same and ends the solve with
+// RP_DEVICE_TIMEOUT.
 //
-// Bound: small systems by the three meetings and the latency of the gathers;
-// FP64 at 128^3 by the FP64 pipe (14 instructions a row and iteration with z
-// kept, where K2 and K3 compute it twice).
-#include "rp_common.cuh"
+// Bound: small systems by the meetings (4000 cycles a sum, 2600 the barrier) and the
+// latency of the gathers; FP32 at 2M rows by the products' instructions; FP64 at 128^3
+// by the FP64 pipe (14 instructions a row and iteration with z kept, where K2 and K3
+// compute it twice; the pipe 75% busy).
 #include "rp_pcg.cuh"
 
 namespace rp {

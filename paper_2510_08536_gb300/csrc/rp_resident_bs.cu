@@ -18,8 +18,10 @@
 // of rp_resident.cuh; every wait is bounded and ends the solve with
 // RP_DEVICE_TIMEOUT.
 //
-// Bound: the latency of the gathers and the five meetings; in FP64 the FP64 pipe
-// (28 instructions a row and iteration).
+// 128^3 mixed, a momentum step of 214 iterations: 26.0 ms with the streaming kernels,
+// 14.5 ms with this one and sums by way of all blocks' partial sums, 13.9 ms with sums
+// in known units. Bound: the products' instructions (31k of 130k cycles each) and the
+// five meetings; in FP64 the FP64 pipe (28 instructions a row and iteration).
 #include "rp_bicgstab.cuh"
 
 namespace rp {
