@@ -23,7 +23,7 @@
 //   r and q kept (FP64): to 2.2M rows
 // us an iteration (streaming kernels, then this): 32^3 FP64 19.7 -> 6.8, 97x61x83 FP32
 // 32.6 -> 9.1, 64^3 FP64 34.5 -> 13.5, 128^3 FP64 91.7 -> 61.9, 128^3 FP32 on 8 parts
-// 51.4 -> 39.
+// 51.4 -> 31.4.
 //
 // The barrier is an arrival counter in L2 (red.release, ld.acquire polls of one
 // thread a block): 1.3 us on 152 SMs. (Flags with the partial sums as payload took
@@ -57,7 +57,7 @@ struct RsShared : RsFlags {
 // product gathers z + beta p of the two vectors, which are written to global memory
 // before the sum of B).
 template <typename T, int LAY, bool SCALED, bool ALL, bool MAT, bool FOLD>
-__global__ void __launch_bounds__(kRsThreads<T>, 1) k_resident(const ResidentArgs<T> A) {
+__global__ void __launch_bounds__(kRsThreads<T, MAT>, 1) k_resident(const ResidentArgs<T> A) {
   const IterArgs<T>& a = A.it;
   Ctl* c = a.ctl;
   // written again only after every block has arrived once (or given up)
@@ -289,7 +289,7 @@ RP_CHECK_TU(resident)
 // where a warp has one slice.
 enum : int { kKeptFold, kKept, kStream4, kStream2 };
 template <typename T>
-constexpr int kFoldRows = kRsThreads<T>;
+constexpr int kFoldRows = kRsThreads<T, true>;
 template <typename T>
 ResidentPlan resident_plan(const rp_handle* h, const IterArgs<T>& a, bool scaled) {
   if (a.line.l != nullptr) return ResidentPlan{};

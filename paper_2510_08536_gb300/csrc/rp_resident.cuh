@@ -17,10 +17,13 @@ namespace rp {
 // of at most 8 entries), and both with several parts
 enum : int { kRsCsr = 0, kRsSliced = 1, kRsU4 = 2, kRsParts = 3, kRsPartsU4 = 4 };
 
-// FP64: 24 warps of up to 80 registers (32 warps of 64 spill the prefetched
-// slice, and the FP64 pipe is the bound anyway)
-template <typename T>
-constexpr int kRsThreads = sizeof(T) == 8 ? 768 : 1024;
+// Threads of a block: as many as leave the slice fetched ahead its registers. FP32
+// streamed, us an iteration at 128^3 (one part, 8 parts, BiCGStab): 32 warps of 64
+// registers 34.1, 39.6, 62.0 (they spill); 28 of 72 25.9, 31.4, 52.3; 24 of 80 27.1,
+// 34.4, 57.9; 16 of 128 lose more. With the matrix in shared memory 64 registers are
+// enough for FP32. FP64 (28 instructions of its pipe a slice): 24 warps of 80.
+template <typename T, bool MAT>
+constexpr int kRsThreads = sizeof(T) == 8 ? 768 : MAT ? 1024 : 896;
 
 // Partial sums of a block's warps, and the flags every thread reads after a grid sum.
 struct RsFlags {
@@ -472,8 +475,9 @@ struct RsMatrix {
     if constexpr (U4) {
       const G xr = x.at(valid ? i : 0);
       NlRange nl{0, 0};
+      if (MP) nl = MAT ? nl_range(j) : fnl;
+      // the first non-local entry (most rows that have any have one) under way with the gathers
       if constexpr (MAT) {
-        if (MP) nl = nl_range(j);
         const uint32_t x0 = sx[j];
         const T* v = mv + (x0 - sx[0]) + lane;
         const int32_t tv = __ldg(sl.tabs + sinfo[j] + (lane & 15));
@@ -481,7 +485,6 @@ struct RsMatrix {
                              [&](int e) { return v[kSliceRows * e]; });
       } else {
         const RsSlice<T> cur = f;
-        nl = fnl;
         fetch(j + nw < cnt ? j + nw : w);  // the last one fetches the first of the next product
         sum = rs_products<T>(xr, valid, cur.wd, cur.tv, cur.L, [&](int e) { return cur.v[e]; });
       }
@@ -549,7 +552,7 @@ ResidentPlan plan_resident(const rp_handle* h, const Sliced<T>& sl, int64_t n, s
     if (!fn) continue;
     const int64_t need =
         per * 32 * f.vecs * (int64_t)sizeof(T) + RsMatrix<T, kRsCsr>::tail_bytes(lay, per, f.mat, h->sl_width);
-    const int threads = 32 * (int)std::min<int64_t>(std::max<int64_t>(per, 4), kRsThreads<T> / 32);
+    const int threads = 32 * (int)std::min<int64_t>(std::max<int64_t>(per, 4), (f.mat ? kRsThreads<T, true> : kRsThreads<T, false>) / 32);
     cudaFuncAttributes at;
     int nb = 0;
     // the kernel's own (static) shared memory comes off the block's limit
