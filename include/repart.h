@@ -240,7 +240,7 @@ rp_status rp_spmv_noalloc(int64_t n, const int32_t* row_ptr, const int32_t* col_
 
 /* The sliced layout the PCG iteration multiplies with (the paper has no
  * counterpart: it is this library's device format of the merged matrix, built
- * once next to the CSR map by rp_build_repartition and refilled from the CSR
+ * once next to the CSR map by rp_build_repartition and refilled with the CSR
  * values by every value update). Rows in slices of 32 (n_slices = ceil(n/32)
  * for one part, the sum of ceil(n_p/32) over parts; 0 when the layout is not
  * in use), one row per lane. Slice s: desc[2s] = x_s,
