@@ -106,12 +106,14 @@ __device__ __forceinline__ double recip_rn(double d) {
 }
 
 // a / b, a and b > 0, in the same way: 18, 17 and 17 bits (a's mantissa below b's:
-// one more) after the exact first step.
+// one more) after the exact first step. Exponents 1021 apart at most, so that the
+// quotient is a normal number in either case (1022 below, a smaller mantissa makes
+// it subnormal); else the division itself.
 __device__ __forceinline__ double quot_rn(double a, double b) {
   const uint32_t ah = (uint32_t)__double2hiint(a), al = (uint32_t)__double2loint(a);
   const uint32_t bh = (uint32_t)__double2hiint(b), bl = (uint32_t)__double2loint(b);
   const int ea = (int)(ah >> 20), eb = (int)(bh >> 20);  // with the sign bit
-  if ((unsigned)(ea - 1) > 2045u || (unsigned)(eb - 1) > 2045u || (unsigned)(ea - eb + 1022) > 2043u) return a / b;
+  if ((unsigned)(ea - 1) > 2045u || (unsigned)(eb - 1) > 2045u || (unsigned)(ea - eb + 1021) > 2042u) return a / b;
   const uint64_t ma = (uint64_t)((ah & 0xfffffu) | 0x100000u) << 32 | al;
   const uint64_t mb = (uint64_t)((bh & 0xfffffu) | 0x100000u) << 32 | bl;
   const float f = __uint_as_float(0x3f800000u | (__funnelshift_l(bl, bh, 3) & 0x7fffffu));
