@@ -723,7 +723,7 @@ rp_status bs_host_loop(rp_handle* h, bool mixed, cudaStream_t s) {
     RP_TRY_CUDA(cudaMemcpyAsync(&c, h->bs->ctl, sizeof(BsCtl), cudaMemcpyDeviceToHost, s));
     RP_TRY_CUDA(cudaStreamSynchronize(s));
     if (c.stop) break;
-    while (!c.stop) {
+    while (inner_runs(c.stop, c.status)) {
       void* args[1] = {&a};
       void* rargs[1] = {r.args(mixed)};
       if (r.plan.fn)

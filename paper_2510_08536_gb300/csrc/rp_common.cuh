@@ -407,6 +407,10 @@ struct rp_handle {
 
 namespace rp {
 
+// Does a host loop launch another inner iteration on this control block? A block
+// that reports a timeout raises both words; either one ends the loop.
+inline bool inner_runs(int32_t stop, int32_t status) { return !stop && status != RP_DEVICE_TIMEOUT; }
+
 // streaming-grid size for n rows
 inline int grid_for(const rp_handle* h, int64_t n) {
   int64_t want = (n + kThreads - 1) / kThreads;

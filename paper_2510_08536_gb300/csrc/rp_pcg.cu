@@ -1187,7 +1187,7 @@ rp_status host_loop_solve(rp_handle* h, int mode, const double* vals, const doub
     if (mode == 2) RP_TRY(launch1(k.rup, h->grid, kThreads, 0, &k.ru, s));
     RP_TRY(read());
     const bool go = !c.stop;
-    while (!c.stop) {
+    while (inner_runs(c.stop, c.status)) {
       if (k.resident.fn) {  // one iteration a launch
         k.rs64.cap = k.rs32.cap = 1;
         void* args[1] = {mixed ? (void*)&k.rs32 : (void*)&k.rs64};

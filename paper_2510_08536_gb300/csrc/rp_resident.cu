@@ -245,7 +245,7 @@ __global__ void __launch_bounds__(kRsThreads<T, MAT>, 1) k_resident(const Reside
     c->rz = sh.rz;
     c->rr = sh.rr;
     atomicMax(&c->status, sh.status);  // a timeout, the largest status, stands whoever writes last
-    c->stop = sh.stop == 3 ? 0 : 1;
+    if (sh.stop != 3) c->stop = 1;  // 0 at the launch and only ever raised: another block's report stands
     if (sh.stop == 2) c->skip_x = 1;
   }
   if (tid == 0 && sh.bad) {  // any block may have given up

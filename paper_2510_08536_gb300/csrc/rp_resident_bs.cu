@@ -268,7 +268,7 @@ __global__ void __launch_bounds__(kRsThreads<T, false>, 1) k_resident_bs(const R
     c->ss = sh.ss;
     c->half = sh.stop == 3;
     atomicMax(&c->status, sh.status);  // a timeout, the largest status, stands whoever writes last
-    c->stop = sh.stop == 2 ? 0 : 1;
+    if (sh.stop != 2) c->stop = 1;  // 0 at the launch and only ever raised: another block's report stands
   }
   if (tid == 0 && sh.bad) {  // any block may have given up
     atomicMax(&c->status, (int)RP_DEVICE_TIMEOUT);
