@@ -338,6 +338,21 @@ rp_status rp_solve(rp_handle* h, const double* b, double* x, double tol, int32_t
  * solve has run on the handle. */
 rp_status rp_get_solve_info(rp_handle* h, rp_solve_info* info, void* stream);
 
+/* Which kernels ran the inner iterations of the latest rp_solve,
+ * rp_solve_adjoint or rp_solve_bicgstab(_mixed) on this handle (for counting
+ * launches and for tests): RP_FORM_STREAMING one launch a step of every
+ * iteration (three of PCG, five of BiCGStab), the others one cooperative launch
+ * for a whole inner run, the vectors in shared memory -- and the matrix
+ * (RP_FORM_RESIDENT_MATRIX), its product taking z + beta p by itself
+ * (RP_FORM_RESIDENT_FOLDED). RP_EINVAL if no solve has run on the handle. */
+enum {
+  RP_FORM_STREAMING = 0,
+  RP_FORM_RESIDENT = 1,
+  RP_FORM_RESIDENT_MATRIX = 2,
+  RP_FORM_RESIDENT_FOLDED = 3
+};
+rp_status rp_get_solve_form(const rp_handle* h, int32_t* form);
+
 /* Solve a non-symmetric system A x = b (the momentum equation, which the paper
  * solves with BiCGStab; Sec. 4) to ||b - A x||_2 <= tol ||b||_2 (true
  * residual, FP64) with Jacobi-preconditioned BiCGStab (van der Vorst, 1992;
@@ -461,6 +476,12 @@ rp_status rp_face_grad(rp_handle* h, const double* lambda, const double* x, doub
  * clears the counters. The normal build returns RP_EUNSUPPORTED with
  * *count = 0. */
 rp_status rp_check_violations(uint64_t* count, int32_t* first_site, int64_t* first_index, int32_t reset);
+
+/* Bounds-checked build only, for its tests: refuse != 0 makes every cooperative
+ * launch of this handle's solves fail as a driver that refuses it would, so that
+ * they take the streaming kernels. Takes effect at the next solve. The normal
+ * build returns RP_EUNSUPPORTED. */
+rp_status rp_check_resident(rp_handle* h, int32_t refuse);
 
 void rp_destroy(rp_handle* h);
 const char* rp_status_str(rp_status s);

@@ -34,7 +34,7 @@ struct BsState {
   float *rhat32 = nullptr, *s32 = nullptr, *t32 = nullptr, *phat32 = nullptr, *shat32 = nullptr;
   BsCtl* ctl = nullptr;
   SolveIO* io = nullptr;
-  cudaGraphExec_t graph = nullptr, graph_mixed = nullptr;
+  SolveGraph graph, graph_mixed;
   int grid_vec = 1, grid_sl = 1, grid_sl32 = 1;
 };
 
@@ -665,7 +665,7 @@ BsResident bs_resident(const rp_handle* h, bool mixed, const BsArgs& a, int cap)
 // while (outer) { residual pass; while (inner) { B1 .. B5 }; [x += d] }, the inner
 // while replaced by the resident kernel where it takes the system (and may be
 // used: a cooperative node is refused under MPS); mixed: FP32 inner loop
-rp_status build_bs_graph(rp_handle* h, bool mixed, bool may_reside, cudaGraphExec_t* exec) {
+rp_status build_bs_graph(rp_handle* h, bool mixed, bool may_reside, SolveGraph* out) {
   cudaGraph_t top = nullptr;
   RP_TRY_CUDA(cudaGraphCreate(&top, 0));
   struct Guard {
@@ -688,9 +688,7 @@ rp_status build_bs_graph(rp_handle* h, bool mixed, bool may_reside, cudaGraphExe
   RP_TRY(node(obody, &nres, nullptr, mixed ? (void*)k_bs_res_mixed : (void*)k_bs_res, h->grid, kThreads, 0, &a));
   if (resident) {
     RP_TRY(node(obody, &win, &nres, r.plan.fn, r.plan.grid, r.plan.threads, r.plan.smem, r.args(mixed)));
-    cudaLaunchAttributeValue coop{};
-    coop.cooperative = 1;
-    RP_TRY_CUDA(cudaGraphKernelNodeSetAttribute(win, cudaLaunchAttributeCooperative, &coop));
+    RP_TRY_CUDA(cooperative_node(h, win));
   } else {
     RP_TRY(while_node(obody, &win, &nres, hin, &ibody));
     BsLaunch k[5];
@@ -703,7 +701,8 @@ rp_status build_bs_graph(rp_handle* h, bool mixed, bool may_reside, cudaGraphExe
     cudaGraphNode_t ncor;
     RP_TRY(node(obody, &ncor, &win, (void*)k_bs_correct, h->bs->grid_vec, kThreads, 0, &a));
   }
-  RP_TRY_CUDA(cudaGraphInstantiate(exec, top, 0));
+  RP_TRY_CUDA(cudaGraphInstantiate(&out->exec, top, 0));
+  out->form = resident ? r.plan.form : RP_FORM_STREAMING;
   return RP_OK;
 }
 
@@ -725,11 +724,11 @@ rp_status bs_host_loop(rp_handle* h, bool mixed, cudaStream_t s) {
     if (c.stop) break;
     while (inner_runs(c.stop, c.status)) {
       void* args[1] = {&a};
-      void* rargs[1] = {r.args(mixed)};
-      if (r.plan.fn)
-        RP_TRY_CUDA(cudaLaunchCooperativeKernel(r.plan.fn, dim3((unsigned)r.plan.grid),
-                                                dim3((unsigned)r.plan.threads), rargs, (size_t)r.plan.smem, s));
-      else
+      if (r.plan.fn && launch_resident(h, r.plan, r.args(mixed), s) != cudaSuccess) {
+        cudaGetLastError();  // refused: the same state serves the streaming kernels
+        r.plan = ResidentPlan{};
+      }
+      if (!r.plan.fn)
         for (auto& kk : k)
           RP_TRY_CUDA(cudaLaunchKernel(kk.fn, dim3((unsigned)kk.grid), dim3((unsigned)kk.threads), args,
                                        (size_t)kk.smem, s));
@@ -741,6 +740,7 @@ rp_status bs_host_loop(rp_handle* h, bool mixed, cudaStream_t s) {
       RP_TRY_CUDA(cudaGetLastError());
     }
   }
+  h->solve_form = r.plan.form;
   return RP_OK;
 }
 
@@ -748,11 +748,8 @@ rp_status bs_host_loop(rp_handle* h, bool mixed, cudaStream_t s) {
 
 void drop_bicgstab_graph(rp_handle* h) {
   if (!h->bs) return;
-  for (cudaGraphExec_t* g : {&h->bs->graph, &h->bs->graph_mixed})
-    if (*g) {
-      cudaGraphExecDestroy(*g);
-      *g = nullptr;
-    }
+  h->bs->graph.drop();
+  h->bs->graph_mixed.drop();
 }
 
 void free_bicgstab(rp_handle* h) {
@@ -788,10 +785,10 @@ rp_status bicgstab_run(rp_handle* h, bool mixed, const double* b, double* x, dou
   cudaStream_t s = (cudaStream_t)stream;
   RP_TRY(ensure_bs(h));
   BsState* bs = h->bs;
-  cudaGraphExec_t& graph = mixed ? bs->graph_mixed : bs->graph;
-  if (!graph && !h->opts.host_loop && build_bs_graph(h, mixed, true, &graph) != RP_OK) {
+  SolveGraph& graph = mixed ? bs->graph_mixed : bs->graph;
+  if (!graph.exec && !h->opts.host_loop && build_bs_graph(h, mixed, true, &graph) != RP_OK) {
     cudaGetLastError();
-    graph = nullptr;
+    graph.exec = nullptr;
     RP_TRY(build_bs_graph(h, mixed, false, &graph));
   }
   const double* bd = b;
@@ -809,8 +806,12 @@ rp_status bicgstab_run(rp_handle* h, bool mixed, const double* b, double* x, dou
   k_bs_setup<<<1, kRsSync, 0, s>>>(bs->ctl, bs->io, bd, xd, tol, x_is_guess ? 0 : 1, h->opts.max_iter,
                              h->opts.max_restarts, h->opts.max_outer, h->opts.inner_tol, h->rsync);
   RP_TRY_CUDA(cudaGetLastError());
-  if (h->opts.host_loop) RP_TRY(bs_host_loop(h, mixed, s));
-  else RP_TRY_CUDA(cudaGraphLaunch(graph, s));
+  if (h->opts.host_loop) {
+    RP_TRY(bs_host_loop(h, mixed, s));
+  } else {
+    RP_TRY_CUDA(cudaGraphLaunch(graph.exec, s));
+    h->solve_form = graph.form;
+  }
   if (where == RP_MEM_HOST) RP_TRY_CUDA(cudaMemcpyAsync(x, h->x_host_stage, 8 * h->n, cudaMemcpyDeviceToHost, s));
   if (!info) return RP_OK;
   BsCtl c;

@@ -145,11 +145,16 @@ struct SolveIO {
   double* x;
 };
 
+struct SolveGraph {
+  cudaGraphExec_t exec = nullptr;
+  int32_t form = RP_FORM_STREAMING;  // the kernels of its inner iterations
+  void drop() {
+    if (exec) cudaGraphExecDestroy(exec);
+    exec = nullptr;
+  }
+};
 struct Graphs {
-  cudaGraphExec_t fp64 = nullptr;
-  cudaGraphExec_t mixed = nullptr;
-  cudaGraphExec_t mixed_ru = nullptr;
-  cudaGraphExec_t adjoint = nullptr;
+  SolveGraph fp64, mixed, mixed_ru, adjoint;
 };
 
 // The matrix split into GPU parts (Sec. 3): per part a local CSR over the
@@ -383,6 +388,8 @@ struct rp_handle {
   rp::Graphs graphs;
   cudaStream_t capture_stream = nullptr;
   bool solve_ran = false;          // an rp_solve has filled the control block
+  int32_t solve_form = -1;         // kernels of the latest solve (rp_get_solve_form); -1: none yet
+  int32_t check_refuse = 0;        // bounds-checked build: rp_check_resident
 
   // line preconditioner (precond == RP_PRECOND_LINE)
   int precond = RP_PRECOND_JACOBI;

@@ -967,7 +967,7 @@ rp_status launch1(void* fn, int grid, int threads, int smem, void* argp, cudaStr
 // may be used: a cooperative node is refused under MPS).
 // mode: 0 FP64, 1 mixed (restarted inner PCG), 2 mixed with continued inner PCG
 rp_status build_solve_graph(rp_handle* h, int mode, const double* vals, const double* dinv, bool may_reside,
-                            cudaGraphExec_t* exec) {
+                            SolveGraph* out) {
   const bool mixed = mode != 0;
   GraphGuard top;
   RP_TRY_CUDA(cudaGraphCreate(&top.g, 0));
@@ -992,11 +992,10 @@ rp_status build_solve_graph(rp_handle* h, int mode, const double* vals, const do
   if (resident) {
     RP_TRY(add_kernel(obody, &win, &before_inner, k.resident.fn, k.resident.grid,
                       mixed ? (void*)&k.rs32 : (void*)&k.rs64, k.resident.smem, k.resident.threads));
-    cudaLaunchAttributeValue coop{};
-    coop.cooperative = 1;
-    RP_TRY_CUDA(cudaGraphKernelNodeSetAttribute(win, cudaLaunchAttributeCooperative, &coop));
+    RP_TRY_CUDA(cooperative_node(h, win));
     if (mixed) RP_TRY(add_kernel(obody, &ncor, &win, (void*)k_correct, h->grid, &k.ca));
-    RP_TRY_CUDA(cudaGraphInstantiate(exec, top.g, 0));
+    RP_TRY_CUDA(cudaGraphInstantiate(&out->exec, top.g, 0));
+    out->form = k.resident.form;
     return RP_OK;
   }
   RP_TRY(add_while(obody, &win, &before_inner, hin, &ibody));
@@ -1012,7 +1011,8 @@ rp_status build_solve_graph(rp_handle* h, int mode, const double* vals, const do
     RP_TRY(add_kernel(ibody, &n2, &n1, k.k2_64, k.g2_64, &ia));
     RP_TRY(add_kernel(ibody, &n3, &n2, k.k3_64, k.g3_64, &ia));
   }
-  RP_TRY_CUDA(cudaGraphInstantiate(exec, top.g, 0));
+  RP_TRY_CUDA(cudaGraphInstantiate(&out->exec, top.g, 0));
+  out->form = RP_FORM_STREAMING;
   return RP_OK;
 }
 
@@ -1140,11 +1140,7 @@ void free_solver(rp_handle* h) {
   h->ticket = nullptr;
   h->rsync = nullptr;
   h->ctl_spmv = nullptr;
-  if (h->graphs.fp64) cudaGraphExecDestroy(h->graphs.fp64);
-  if (h->graphs.mixed) cudaGraphExecDestroy(h->graphs.mixed);
-  if (h->graphs.mixed_ru) cudaGraphExecDestroy(h->graphs.mixed_ru);
-  if (h->graphs.adjoint) cudaGraphExecDestroy(h->graphs.adjoint);
-  h->graphs = Graphs{};
+  for (SolveGraph* g : {&h->graphs.fp64, &h->graphs.mixed, &h->graphs.mixed_ru, &h->graphs.adjoint}) g->drop();
 }
 
 rp_status launch_solve(rp_handle* h, cudaGraphExec_t exec, const double* b, double* x, double tol, bool x_zero,
@@ -1175,6 +1171,7 @@ rp_status read_info(rp_handle* h, rp_solve_info* info, cudaStream_t s) {
 rp_status host_loop_solve(rp_handle* h, int mode, const double* vals, const double* dinv, cudaStream_t s) {
   const bool mixed = mode != 0;
   SolveSet k = solve_set(h, mode, vals, dinv, 0, 0, 0);
+  k.rs64.cap = k.rs32.cap = 1;  // resident: one iteration a launch
   Ctl c;
   auto read = [&]() -> rp_status {
     RP_TRY_CUDA(cudaMemcpyAsync(&c, h->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, s));
@@ -1188,11 +1185,11 @@ rp_status host_loop_solve(rp_handle* h, int mode, const double* vals, const doub
     RP_TRY(read());
     const bool go = !c.stop;
     while (inner_runs(c.stop, c.status)) {
-      if (k.resident.fn) {  // one iteration a launch
-        k.rs64.cap = k.rs32.cap = 1;
-        void* args[1] = {mixed ? (void*)&k.rs32 : (void*)&k.rs64};
-        RP_TRY_CUDA(cudaLaunchCooperativeKernel(k.resident.fn, dim3((unsigned)k.resident.grid),
-                                                dim3((unsigned)k.resident.threads), args, (size_t)k.resident.smem, s));
+      if (k.resident.fn && launch_resident(h, k.resident, mixed ? (void*)&k.rs32 : (void*)&k.rs64, s) != cudaSuccess) {
+        cudaGetLastError();  // refused: the same state serves the streaming kernels
+        k.resident = ResidentPlan{};
+      }
+      if (k.resident.fn) {
       } else if (mixed) {
         launch_k1(k.a32, k1_grid(k.a32, h->igrid32), s);
         RP_TRY(launch1(k.k2_32, k.g2_32, kThreads, 0, &k.a32, s));
@@ -1209,15 +1206,16 @@ rp_status host_loop_solve(rp_handle* h, int mode, const double* vals, const doub
     if (!go) break;
   }
   RP_TRY_CUDA(cudaGetLastError());
+  h->solve_form = k.resident.form;
   return RP_OK;
 }
 
-rp_status solve_common(rp_handle* h, int mode, const double* vals, const double* dinv, cudaGraphExec_t* slot,
+rp_status solve_common(rp_handle* h, int mode, const double* vals, const double* dinv, SolveGraph* slot,
                        const double* b, double* x, double tol, int32_t x_is_guess, int32_t where,
                        rp_solve_info* info, cudaStream_t s) {
-  if (!*slot && !h->opts.host_loop && build_solve_graph(h, mode, vals, dinv, true, slot) != RP_OK) {
+  if (!slot->exec && !h->opts.host_loop && build_solve_graph(h, mode, vals, dinv, true, slot) != RP_OK) {
     cudaGetLastError();
-    *slot = nullptr;
+    slot->exec = nullptr;
     RP_TRY(build_solve_graph(h, mode, vals, dinv, false, slot));
   }
   const double* bd = b;
@@ -1235,7 +1233,8 @@ rp_status solve_common(rp_handle* h, int mode, const double* vals, const double*
                             h->opts.max_restarts, h->opts.max_outer, h->opts.ru_delta, h->rsync);
     RP_TRY(host_loop_solve(h, mode, vals, dinv, s));
   } else {
-    RP_TRY(launch_solve(h, *slot, bd, xd, tol, !x_is_guess, h->opts.max_iter, info, s));
+    RP_TRY(launch_solve(h, slot->exec, bd, xd, tol, !x_is_guess, h->opts.max_iter, info, s));
+    h->solve_form = slot->form;
   }
   if (where == RP_MEM_HOST) RP_TRY_CUDA(cudaMemcpyAsync(x, h->x_host_stage, 8 * h->n, cudaMemcpyDeviceToHost, s));
   h->solve_ran = true;
@@ -1287,6 +1286,13 @@ extern "C" rp_status rp_get_solve_info(rp_handle* h, rp_solve_info* info, void* 
   return (rp_status)info->status;
 }
 
+extern "C" rp_status rp_get_solve_form(const rp_handle* h, int32_t* form) {
+  if (!h || !form) return fail(RP_EINVAL, "null argument");
+  if (h->solve_form < 0) return fail(RP_EINVAL, "no solve has run on this handle");
+  *form = h->solve_form;
+  return RP_OK;
+}
+
 extern "C" rp_status rp_set_solver_options(rp_handle* h, const rp_options* o) {
   if (!h || !o) return fail(RP_EINVAL, "null argument");
   if (o->max_iter < 0 || o->max_outer < 0 || o->max_restarts < 0 || !(o->inner_tol > 0.0) ||
@@ -1307,11 +1313,7 @@ extern "C" rp_status rp_set_solver_options(rp_handle* h, const rp_options* o) {
     h->precond = o->precond;
     h->opts.precond = o->precond;
     h->opts.spin_limit = o->spin_limit;
-    for (cudaGraphExec_t* g : {&h->graphs.fp64, &h->graphs.mixed, &h->graphs.mixed_ru, &h->graphs.adjoint})
-      if (*g) {
-        cudaGraphExecDestroy(*g);
-        *g = nullptr;
-      }
+    for (SolveGraph* g : {&h->graphs.fp64, &h->graphs.mixed, &h->graphs.mixed_ru, &h->graphs.adjoint}) g->drop();
     drop_bicgstab_graph(h);
     if (new_precond) {
       RP_TRY(line_factors(h, 0));  // from the current values
@@ -1331,6 +1333,19 @@ extern "C" rp_status rp_set_solver_options(rp_handle* h, const rp_options* o) {
       }
   }
   return RP_OK;
+}
+
+extern "C" rp_status rp_check_resident(rp_handle* h, int32_t refuse) {
+  if (!h) return fail(RP_EINVAL, "null handle");
+#ifdef RP_CHECK
+  h->check_refuse = refuse;
+  for (SolveGraph* g : {&h->graphs.fp64, &h->graphs.mixed, &h->graphs.mixed_ru, &h->graphs.adjoint}) g->drop();
+  drop_bicgstab_graph(h);
+  return RP_OK;
+#else
+  (void)refuse;
+  return fail(RP_EUNSUPPORTED, "this library was built without RP_CHECK");
+#endif
 }
 
 extern "C" rp_status rp_spmv(rp_handle* h, const double* x, double* y, double* xy, void* stream) {

@@ -518,13 +518,36 @@ struct RsMatrix {
 struct ResidentPlan {
   void* fn = nullptr;  // nullptr: the streaming kernels run
   int grid = 0, threads = 0, smem = 0, rows = 0, width = 0;
+  int32_t form = RP_FORM_STREAMING;
 };
 struct ResidentForm {
   int vecs;
   bool mat;
   int max_rows;
   int id;
+  int32_t form = RP_FORM_RESIDENT;
 };
+// A cooperative launch can be refused (in a graph under MPS, for instance): the
+// caller takes the streaming kernels then.
+inline cudaError_t cooperative_node(const rp_handle* h, cudaGraphNode_t node) {
+#ifdef RP_CHECK
+  if (h->check_refuse) return cudaErrorNotSupported;
+#else
+  (void)h;
+#endif
+  cudaLaunchAttributeValue coop{};
+  coop.cooperative = 1;
+  return cudaGraphKernelNodeSetAttribute(node, cudaLaunchAttributeCooperative, &coop);
+}
+inline cudaError_t launch_resident(const rp_handle* h, const ResidentPlan& p, void* argp, cudaStream_t s) {
+#ifdef RP_CHECK
+  if (h->check_refuse) return cudaErrorNotSupported;
+#else
+  (void)h;
+#endif
+  void* args[1] = {argp};
+  return cudaLaunchCooperativeKernel(p.fn, dim3((unsigned)p.grid), dim3((unsigned)p.threads), args, (size_t)p.smem, s);
+}
 // fn_of(layout, form): the instance, or nullptr where there is none
 template <typename T, typename Fn>
 ResidentPlan plan_resident(const rp_handle* h, const Sliced<T>& sl, int64_t n, std::initializer_list<ResidentForm> forms,
@@ -560,7 +583,7 @@ ResidentPlan plan_resident(const rp_handle* h, const Sliced<T>& sl, int64_t n, s
         cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max - (int)at.sharedSizeBytes) ==
             cudaSuccess &&
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, threads, (size_t)need) == cudaSuccess && nb >= 1)
-      return ResidentPlan{fn, grid, threads, (int)need, (int)(per * 32), h->sl_width};
+      return ResidentPlan{fn, grid, threads, (int)need, (int)(per * 32), h->sl_width, f.form};
     cudaGetLastError();
   }
   return p;

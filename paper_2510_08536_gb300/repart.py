@@ -106,6 +106,8 @@ def load(path: str = LIB_PATH) -> ctypes.CDLL:
         "rp_entry_grad": (i32, [vp, vp, vp, vp, vp]),
         "rp_face_grad": (i32, [vp, vp, vp, vp, vp]),
         "rp_check_violations": (i32, [ctypes.POINTER(ctypes.c_uint64), ctypes.POINTER(i32), ctypes.POINTER(i64), i32]),
+        "rp_check_resident": (i32, [vp, i32]),
+        "rp_get_solve_form": (i32, [vp, ctypes.POINTER(i32)]),
         "rp_destroy": (None, [vp]),
         "rp_status_str": (ctypes.c_char_p, [i32]),
         "rp_last_error": (ctypes.c_char_p, []),
@@ -435,6 +437,14 @@ def solve_bicgstab(h: Handle, b, x, tol: float = 1e-9, x_is_guess: bool = False,
     return info.as_dict() if wait else None
 
 
+def solve_form(h: Handle) -> str:
+    """rp_get_solve_form: the kernels of the latest solve's iterations ("streaming",
+    "resident", "resident_matrix" or "resident_folded")."""
+    form = ctypes.c_int32()
+    _check(load().rp_get_solve_form(h.ptr, ctypes.byref(form)), "rp_get_solve_form")
+    return ("streaming", "resident", "resident_matrix", "resident_folded")[form.value]
+
+
 def profile_iteration(h: Handle, b, precision: str = "fp64", iters: int = 20, stream=None):
     """rp_profile_iteration: average ms of the SpMV, residual and x/p kernels."""
     ms = (ctypes.c_float * 3)()
@@ -468,6 +478,11 @@ def check_violations(reset: bool = False):
     return c.value, site.value, idx.value
 
 
+def check_resident(h: Handle, refuse: bool):
+    """rp_check_resident (bounds-checked library only): refuse cooperative launches."""
+    _check(load().rp_check_resident(h.ptr, int(refuse)), "rp_check_resident")
+
+
 @dataclasses.dataclass
 class Exports:
     """Names the header declares (checked against the loaded library)."""
@@ -477,4 +492,4 @@ class Exports:
                     "rp_last_error", "rp_spmv_noalloc", "rp_batch_build", "rp_batch_update_solve",
                     "rp_batch_set_config", "rp_batch_autotune", "rp_set_solver_options", "rp_iter_spmv",
                     "rp_get_sliced_view", "rp_solve_bicgstab", "rp_solve_bicgstab_mixed", "rp_get_solve_info",
-                    "rp_check_violations")
+                    "rp_check_violations", "rp_check_resident", "rp_get_solve_form")

@@ -1,0 +1,100 @@
+"""The two forms of the inner iterations in the bounds-checked build: cooperative
+launches refused (as a driver under MPS refuses them) from the solve graph and
+from the host loop, which then run the streaming kernels to the same residual.
+
+A child process loads that library (the binding holds one library per process).
+True residuals are recomputed with the oracle's matrix; 1e-9 is what the solves
+are asked for."""
+import multiprocessing as mp
+import os
+import sys
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+
+
+class _Systems:
+    """A pressure and a momentum system on one ragged mesh, solved by a handle of the checked library."""
+
+    def __init__(self, dims=(19, 17, 23), ranks=(2, 2, 2)):
+        import torch
+
+        from gpu_util import Case
+        from oracle import repart_oracle as O
+        from paper_2510_08536_gb300 import synth
+        self.torch = torch
+        c = Case(dims, ranks)
+        self.ranks, self.n, self.b = c.mesh.ranks, c.mesh.n_cells, c.b
+        mst = synth.momentum_staging(c.mesh, 0.5, 100)
+        Am = O.csr_matrix(c.map.row_ptr, c.map.col_idx, O.update_values(c.map.src_of, mst))
+        self.systems = {"pcg": (c.staging, c.A), "bicgstab": (mst, Am)}
+
+    def dev(self, a):
+        return self.torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+    def solve(self, h, kind, precision):
+        """(status, true relative residual, form)"""
+        from paper_2510_08536_gb300 import repart
+        stg, A = self.systems[kind]
+        repart.update_values_packed(h, self.dev(stg))
+        x = self.dev(np.zeros(self.n))
+        f = repart.solve if kind == "pcg" else repart.solve_bicgstab
+        info = f(h, self.dev(self.b), x, tol=1e-9, precision=precision)
+        r = self.b - A @ x.cpu().numpy()
+        return info["status"], float(np.linalg.norm(r) / np.linalg.norm(self.b)), repart.solve_form(h)
+
+
+ALL = [("pcg", "fp64"), ("pcg", "mixed"), ("pcg", "mixed_ru"), ("bicgstab", "fp64"), ("bicgstab", "mixed")]
+
+
+def _refused():
+    from paper_2510_08536_gb300 import repart
+    out = {}
+    s = _Systems()
+    for host_loop in (0, 1):
+        h = repart.build_repartition(s.ranks, host_loop=host_loop)
+        for refuse in (0, 1):
+            repart.check_resident(h, refuse)
+            for kind, precision in ALL:
+                out[host_loop, refuse, kind, precision] = s.solve(h, kind, precision)
+        h.close()
+    return out
+
+
+def _child(q, name):
+    sys.path[:0] = [ROOT, HERE]
+    try:
+        from paper_2510_08536_gb300 import build, repart
+        repart.load(build.build(check=True))
+        repart.check_violations(reset=True)
+        out = globals()[name]()
+        out["violations"] = repart.check_violations(reset=True)
+    except Exception:  # report to the parent
+        import traceback
+        out = {"error": traceback.format_exc()[-3000:]}
+    q.put(out)
+
+
+def _run(name):
+    ctx = mp.get_context("spawn")
+    q = ctx.Queue()
+    p = ctx.Process(target=_child, args=(q, name))
+    p.start()
+    out = q.get(timeout=600)
+    p.join(60)
+    assert "error" not in out, out["error"]
+    assert p.exitcode == 0
+    assert out.pop("violations")[0] == 0
+    return out
+
+
+def test_refused_cooperative_launches():
+    for (host_loop, refuse, kind, precision), (status, residual, form) in _run("_refused").items():
+        case = (host_loop, refuse, kind, precision, form)
+        assert status == 0 and residual <= 1e-9, case
+        assert (form == "streaming") == bool(refuse), case
