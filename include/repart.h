@@ -127,10 +127,14 @@ typedef struct rp_options {
   int32_t max_restarts;   /* residual-replacement restarts allowed per solve      */
   int32_t device;         /* CUDA device ordinal (-1: current device)             */
   double inner_tol;       /* relative tolerance of the FP32 inner solve           */
-  int64_t spin_limit;     /* probe limit of every device-side wait; a wait that
+  int64_t spin_limit;     /* probe limit of every device-side wait (an mbarrier
+                             probe, or an L2 poll of the resident kernels' grid
+                             meetings); a wait that
                              runs out ends the solve with RP_DEVICE_TIMEOUT after
                              its block's own copies have landed (0: every wait
-                             gives up at once -- tests the timeout path)         */
+                             gives up at once -- tests the timeout path). Limits
+                             below 65536 are too small for grid meetings: solves
+                             keep to the streaming kernels                       */
   int32_t host_loop;      /* 1: rp_solve launches the same kernels from the host,
                              reading the control block after every iteration
                              (slow; for profilers that cannot look inside
@@ -479,9 +483,10 @@ rp_status rp_check_violations(uint64_t* count, int32_t* first_site, int64_t* fir
 
 /* Bounds-checked build only, for its tests: refuse != 0 makes every cooperative
  * launch of this handle's solves fail as a driver that refuses it would, so that
- * they take the streaming kernels. Takes effect at the next solve. The normal
- * build returns RP_EUNSUPPORTED. */
-rp_status rp_check_resident(rp_handle* h, int32_t refuse);
+ * they take the streaming kernels; spin >= 0 replaces spin_limit in the waits of
+ * the resident kernels. Takes effect at the next solve. The normal build returns
+ * RP_EUNSUPPORTED. */
+rp_status rp_check_resident(rp_handle* h, int32_t refuse, int64_t spin);
 
 void rp_destroy(rp_handle* h);
 const char* rp_status_str(rp_status s);

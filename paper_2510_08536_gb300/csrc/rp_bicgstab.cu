@@ -657,8 +657,8 @@ struct BsResident {
 BsResident bs_resident(const rp_handle* h, bool mixed, const BsArgs& a, int cap) {
   BsResident r;
   r.plan = mixed ? resident_bs_plan<float>(h, a.f) : resident_bs_plan<double>(h, a.d);
-  r.a64 = ResidentBsArgs<double>{a, h->rsync, h->opts.spin_limit, r.plan.rows, cap};
-  r.a32 = ResidentBsArgs<float>{a, h->rsync, h->opts.spin_limit, r.plan.rows, cap};
+  r.a64 = ResidentBsArgs<double>{a, h->rsync, resident_spin(h), r.plan.rows, cap};
+  r.a32 = ResidentBsArgs<float>{a, h->rsync, resident_spin(h), r.plan.rows, cap};
   return r;
 }
 

@@ -390,6 +390,7 @@ struct rp_handle {
   bool solve_ran = false;          // an rp_solve has filled the control block
   int32_t solve_form = -1;         // kernels of the latest solve (rp_get_solve_form); -1: none yet
   int32_t check_refuse = 0;        // bounds-checked build: rp_check_resident
+  int64_t check_spin = -1;
 
   // line preconditioner (precond == RP_PRECOND_LINE)
   int precond = RP_PRECOND_JACOBI;

@@ -951,8 +951,8 @@ SolveSet solve_set(rp_handle* h, int mode, const double* vals, const double* din
     k.g3_32 = h->igrid32.k3;
   }
   k.resident = mixed ? resident_plan<float>(h, k.a32, k.scaled) : resident_plan<double>(h, k.a64, false);
-  k.rs64 = ResidentArgs<double>{k.a64, h->rsync, h->opts.spin_limit, k.resident.rows, k.resident.width, INT32_MAX};
-  k.rs32 = ResidentArgs<float>{k.a32, h->rsync, h->opts.spin_limit, k.resident.rows, k.resident.width, INT32_MAX};
+  k.rs64 = ResidentArgs<double>{k.a64, h->rsync, resident_spin(h), k.resident.rows, k.resident.width, INT32_MAX};
+  k.rs32 = ResidentArgs<float>{k.a32, h->rsync, resident_spin(h), k.resident.rows, k.resident.width, INT32_MAX};
   return k;
 }
 
@@ -1335,15 +1335,16 @@ extern "C" rp_status rp_set_solver_options(rp_handle* h, const rp_options* o) {
   return RP_OK;
 }
 
-extern "C" rp_status rp_check_resident(rp_handle* h, int32_t refuse) {
+extern "C" rp_status rp_check_resident(rp_handle* h, int32_t refuse, int64_t spin) {
   if (!h) return fail(RP_EINVAL, "null handle");
 #ifdef RP_CHECK
   h->check_refuse = refuse;
+  h->check_spin = spin;
   for (SolveGraph* g : {&h->graphs.fp64, &h->graphs.mixed, &h->graphs.mixed_ru, &h->graphs.adjoint}) g->drop();
   drop_bicgstab_graph(h);
   return RP_OK;
 #else
-  (void)refuse;
+  (void)refuse, (void)spin;
   return fail(RP_EUNSUPPORTED, "this library was built without RP_CHECK");
 #endif
 }

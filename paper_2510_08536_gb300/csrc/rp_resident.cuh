@@ -527,6 +527,17 @@ struct ResidentForm {
   int id;
   int32_t form = RP_FORM_RESIDENT;
 };
+// Limits below this keep to the streaming kernels. A poll of the arrival counter is
+// an L2 round trip (0.4 us), a block waits for the slowest one's pass of up to 0.1
+// ms; a caller's small limit was chosen for the mbarrier probes of the streaming
+// products, or for kernels without any wait (CSR), which it suffices for.
+constexpr int64_t kResidentSpin = int64_t(1) << 16;
+inline int64_t resident_spin(const rp_handle* h) {
+#ifdef RP_CHECK
+  if (h->check_spin >= 0) return h->check_spin;
+#endif
+  return h->opts.spin_limit;
+}
 // A cooperative launch can be refused (in a graph under MPS, for instance): the
 // caller takes the streaming kernels then.
 inline cudaError_t cooperative_node(const rp_handle* h, cudaGraphNode_t node) {
@@ -554,7 +565,7 @@ ResidentPlan plan_resident(const rp_handle* h, const Sliced<T>& sl, int64_t n, s
                            Fn&& fn_of) {
   ResidentPlan p;
   int coop = 0, smem_max = 0;
-  if (n == 0) return p;
+  if (n == 0 || h->opts.spin_limit < kResidentSpin) return p;
   if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, h->device) != cudaSuccess || !coop ||
       cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device) != cudaSuccess) {
     cudaGetLastError();

@@ -106,7 +106,7 @@ def load(path: str = LIB_PATH) -> ctypes.CDLL:
         "rp_entry_grad": (i32, [vp, vp, vp, vp, vp]),
         "rp_face_grad": (i32, [vp, vp, vp, vp, vp]),
         "rp_check_violations": (i32, [ctypes.POINTER(ctypes.c_uint64), ctypes.POINTER(i32), ctypes.POINTER(i64), i32]),
-        "rp_check_resident": (i32, [vp, i32]),
+        "rp_check_resident": (i32, [vp, i32, i64]),
         "rp_get_solve_form": (i32, [vp, ctypes.POINTER(i32)]),
         "rp_destroy": (None, [vp]),
         "rp_status_str": (ctypes.c_char_p, [i32]),
@@ -478,9 +478,10 @@ def check_violations(reset: bool = False):
     return c.value, site.value, idx.value
 
 
-def check_resident(h: Handle, refuse: bool):
-    """rp_check_resident (bounds-checked library only): refuse cooperative launches."""
-    _check(load().rp_check_resident(h.ptr, int(refuse)), "rp_check_resident")
+def check_resident(h: Handle, refuse: bool = False, spin: int = -1):
+    """rp_check_resident (bounds-checked library only): refuse cooperative
+    launches; limit of the resident kernels' waits (-1: spin_limit)."""
+    _check(load().rp_check_resident(h.ptr, int(refuse), int(spin)), "rp_check_resident")
 
 
 @dataclasses.dataclass

@@ -1,6 +1,9 @@
 """The two forms of the inner iterations in the bounds-checked build: cooperative
 launches refused (as a driver under MPS refuses them) from the solve graph and
-from the host loop, which then run the streaming kernels to the same residual.
+from the host loop, which then run the streaming kernels to the same residual;
+and grid meetings that run out (their limit set to 0: every block gives up at its
+first one), which end each solve with RP_DEVICE_TIMEOUT and leave the handle as good
+as a fresh one.
 
 A child process loads that library (the binding holds one library per process).
 True residuals are recomputed with the oracle's matrix; 1e-9 is what the solves
@@ -66,6 +69,25 @@ def _refused():
     return out
 
 
+def _timeouts():
+    from paper_2510_08536_gb300 import repart
+    out = {}
+    s = _Systems()
+    for host_loop in (0, 1):
+        h, fresh = (repart.build_repartition(s.ranks, host_loop=host_loop) for _ in range(2))
+        for kind, precision in ALL:
+            repart.check_resident(h, spin=0)
+            try:
+                out[host_loop, kind, precision, 0] = s.solve(h, kind, precision)
+            except repart.RepartError as e:
+                out[host_loop, kind, precision, 0] = e.status, repart.solve_form(h)
+            repart.check_resident(h)
+            out[host_loop, kind, precision, 1] = s.solve(h, kind, precision) == s.solve(fresh, kind, precision)
+        h.close()
+        fresh.close()
+    return out
+
+
 def _child(q, name):
     sys.path[:0] = [ROOT, HERE]
     try:
@@ -91,6 +113,16 @@ def _run(name):
     assert p.exitcode == 0
     assert out.pop("violations")[0] == 0
     return out
+
+
+def test_grid_meetings_run_out():
+    from paper_2510_08536_gb300 import repart
+    for (host_loop, kind, precision, again), got in _run("_timeouts").items():
+        case = (host_loop, kind, precision, got)
+        if again:
+            assert got is True, case
+        else:
+            assert got[0] == repart.RP_DEVICE_TIMEOUT and got[1] != "streaming", case
 
 
 def test_refused_cooperative_launches():
