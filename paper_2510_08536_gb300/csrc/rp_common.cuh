@@ -301,7 +301,7 @@ struct rp_handle {
   rp_options opts{};
 
   // per rank (host)
-  std::vector<int64_t> row_off, slot_off, face_off, iface_off;
+  std::vector<int64_t> row_off, slot_off, face_off, iface_off, out_off;
   std::vector<int32_t> n_cells, n_faces, n_iface;
   // per part (host)
   std::vector<int64_t> part_row_off, part_nnz_off, part_nl_off, part_buf_off, part_nlcol_off;
@@ -322,6 +322,7 @@ struct rp_handle {
   int64_t* d_slot_off = nullptr;
   int64_t* d_face_off = nullptr;
   int64_t* d_iface_off = nullptr;
+  int64_t* d_out_off = nullptr;     // per-rank offsets of the face-gradient output
   int32_t* d_lower = nullptr;  // concatenated addressing, kept for face gradients
   int32_t* d_upper = nullptr;
   int32_t* d_iface_row = nullptr;
@@ -520,20 +521,40 @@ __device__ __forceinline__ int find_rank(const int64_t* __restrict__ off, int k,
   return lo;
 }
 
-// Elements t of a table off[0..k] (off[r] <= t < off[r + 1]: rank r), a run of
-// 128 a warp, four a lane: f(r, t) for every t. One search serves the run
-// where it lies in one rank (a search an element took 7 dependent loads).
-template <typename F>
-__device__ __forceinline__ void for_ranked(const int64_t* __restrict__ off, int k, F&& f) {
-  const int lane = threadIdx.x & 31;
-  const int64_t total = __ldg(off + k), step = ((int64_t)gridDim.x * blockDim.x) * 4;
-  for (int64_t t0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 128; t0 < total; t0 += step) {
-    const int r0 = find_rank(off, k, t0);
-    const bool one = __ldg(off + r0 + 1) >= t0 + 128;
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int64_t t = t0 + 32 * u + lane;
-      if (t < total) f(one ? r0 : find_rank(off, k, t), t);
+// A thread's way through the grid's elements: `trips` trips of the block through
+// elements that follow one another, then on behind those of the other blocks.
+struct Walk {
+  int64_t t;
+  int left, trips;
+};
+__device__ __forceinline__ Walk grid_walk(int trips) {
+  return Walk{(int64_t)blockIdx.x * (trips * (int)blockDim.x) + threadIdx.x, trips, trips};
+}
+// Four trips serve four elements with one search of a rank (many ranks: eight); where
+// the grid has threads for every second element there is nothing to serve.
+inline int walk_trips(const rp_handle* h, int64_t total) {
+  return total <= 2ll * h->num_sms * kBlocksPerSm * kThreads ? 1 : h->k > 128 ? 8 : 4;
+}
+// The walk through elements first .. first + count - 1, whose table off[0..k] gives
+// their ranks (off[r] <= e < off[r + 1], e from 0): at(r) when a thread's rank changes,
+// then f(e).
+template <typename At, typename F>
+__device__ __forceinline__ void for_ranked(Walk& w, int64_t first, int64_t count, const int64_t* __restrict__ off, int k,
+                                           At&& at, F&& f) {
+  const int64_t end = first + count;
+  int64_t next = w.t;  // where the rank after the present one begins
+  while (w.t < end) {
+    const int64_t e = w.t - first;
+    if (w.t >= next) {
+      const int r = find_rank(off, k, e);
+      next = first + __ldg(off + r + 1);
+      at(r);
+    }
+    f(e);
+    w.t += blockDim.x;
+    if (--w.left == 0) {
+      w.left = w.trips;
+      w.t += (int64_t)(gridDim.x - 1) * (w.trips * (int)blockDim.x);
     }
   }
 }

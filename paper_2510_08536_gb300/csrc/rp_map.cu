@@ -554,7 +554,7 @@ extern "C" const char* rp_status_str(rp_status s) {
 static void free_handle_memory(rp_handle* h) {
   void* ptrs[] = {h->row_ptr, h->col_idx, h->src_of, h->diag_pos, h->tpos, h->nl_row_ptr, h->nl_col_idx,
                   h->nl_src_of, h->nl_cols, h->nl_gcol, h->d_row_off, h->d_slot_off, h->d_face_off, h->d_iface_off,
-                  h->d_lower, h->d_upper, h->d_iface_row, h->d_iface_gcol, h->staging, h->vals,
+                  h->d_out_off, h->d_lower, h->d_upper, h->d_iface_row, h->d_iface_gcol, h->staging, h->vals,
                   h->vals32, h->nl_vals, h->valsT, h->dinv, h->dinv32, h->dinvT, h->nl_vals32,
                   h->d_part_row_off, h->d_part_nnz_off, h->d_part_nl_off, h->d_part_nlcol_off};
   for (void* p : ptrs)
@@ -616,6 +616,8 @@ extern "C" rp_status rp_build_repartition(const rp_ldu_desc* ranks, int32_t k, c
   h->n = h->row_off[k];
   h->n_slots = h->slot_off[k];
   h->n_face_out = h->face_off[k] + h->iface_off[k];
+  h->out_off.resize(k + 1);
+  for (int32_t r = 0; r <= k; ++r) h->out_off[r] = h->face_off[r] + h->iface_off[r];
   const int64_t n = h->n, n_entries = ent_off[k];
   const int64_t F = h->face_off[k], E = h->iface_off[k];
   h->part_row_off.assign(o.n_parts + 1, 0);
@@ -668,6 +670,7 @@ extern "C" rp_status rp_build_repartition(const rp_ldu_desc* ranks, int32_t k, c
   ALLOC(H->d_slot_off, k + 1);
   ALLOC(H->d_face_off, k + 1);
   ALLOC(H->d_iface_off, k + 1);
+  ALLOC(H->d_out_off, k + 1);
   ALLOC(H->d_lower, F);
   ALLOC(H->d_upper, F);
   ALLOC(H->d_iface_row, E);
@@ -676,6 +679,7 @@ extern "C" rp_status rp_build_repartition(const rp_ldu_desc* ranks, int32_t k, c
   CU(cudaMemcpyAsync(H->d_slot_off, H->slot_off.data(), 8 * (k + 1), cudaMemcpyHostToDevice, st));
   CU(cudaMemcpyAsync(H->d_face_off, H->face_off.data(), 8 * (k + 1), cudaMemcpyHostToDevice, st));
   CU(cudaMemcpyAsync(H->d_iface_off, H->iface_off.data(), 8 * (k + 1), cudaMemcpyHostToDevice, st));
+  CU(cudaMemcpyAsync(H->d_out_off, H->out_off.data(), 8 * (k + 1), cudaMemcpyHostToDevice, st));
   if (F) {
     CU(cudaMemcpyAsync(H->d_lower, lower.data(), 4 * F, cudaMemcpyHostToDevice, st));
     CU(cudaMemcpyAsync(H->d_upper, upper.data(), 4 * F, cudaMemcpyHostToDevice, st));

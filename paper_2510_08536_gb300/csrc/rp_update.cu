@@ -68,27 +68,31 @@ __global__ void __launch_bounds__(kThreads)
 template <bool DINV>
 __global__ void __launch_bounds__(kThreads)
     k_diagonal(const double* __restrict__ buf, const int64_t* __restrict__ row_off,
-               const int64_t* __restrict__ slot_off, int k, double* __restrict__ dinv, float* __restrict__ dinv32,
+               const int64_t* __restrict__ slot_off, int k, int64_t n, int trips, double* __restrict__ dinv, float* __restrict__ dinv32,
                double* __restrict__ s64, float2* __restrict__ s2) {
-  for_ranked(row_off, k, [&](int r, int64_t i) {
-    const double d = __ldcs(buf + __ldg(slot_off + r) + (i - __ldg(row_off + r)));
-    if (DINV) {
-      dinv[i] = recip_rn(d);
-      if (dinv32) dinv32[i] = 1.0f / f32_rn(d);
-    } else {
-      const double sc = recip_rn(sqrt_rn(d));
-      s64[i] = sc;
-      s2[i] = scale_pair(sc);
-    }
-  });
+  Walk w = grid_walk(trips);
+  const double* from = buf;
+  for_ranked(
+      w, 0, n, row_off, k, [&](int r) { from = buf + (__ldg(slot_off + r) - __ldg(row_off + r)); },
+      [&](int64_t i) {
+        const double d = __ldcs(from + i);
+        if (DINV) {
+          dinv[i] = recip_rn(d);
+          if (dinv32) dinv32[i] = 1.0f / f32_rn(d);
+        } else {
+          const double sc = recip_rn(sqrt_rn(d));
+          s64[i] = sc;
+          s2[i] = scale_pair(sc);
+        }
+      });
 }
 
 static rp_status permute_all(rp_handle* h, const double* buf, cudaStream_t s) {
-  const int gd = grid_for(h, h->n / 4);
+  const int gd = grid_for(h, h->n);
   if (h->n > 0 && h->sl_vals32s)
-    k_diagonal<false><<<gd, kThreads, 0, s>>>(buf, h->d_row_off, h->d_slot_off, h->k, nullptr, nullptr, h->s64, h->s2);
+    k_diagonal<false><<<gd, kThreads, 0, s>>>(buf, h->d_row_off, h->d_slot_off, h->k, h->n, walk_trips(h, h->n), nullptr, nullptr, h->s64, h->s2);
   if (h->n > 0 && h->sl_slices == 0)
-    k_diagonal<true><<<gd, kThreads, 0, s>>>(buf, h->d_row_off, h->d_slot_off, h->k, h->dinv,
+    k_diagonal<true><<<gd, kThreads, 0, s>>>(buf, h->d_row_off, h->d_slot_off, h->k, h->n, walk_trips(h, h->n), h->dinv,
                                              h->want_fp32 ? h->dinv32 : nullptr, nullptr, nullptr);
   if (h->sl_slices > 0) {
     RP_TRY(fill_sliced(h, buf, s));
