@@ -356,6 +356,7 @@ struct rp_handle {
   int64_t sl_tabs_len = 0;   // int32 words of the distinct tables
   int sl_u4 = 0;             // every slice 4-bit with rows of at most 8 entries
   int sl_width = 0;          // longest row of any slice
+  bool sl_one_pass = false, sl_one_pass_scaled = false;  // see fill_one_pass
   int64_t* sl_part_soff = nullptr;  // [n_parts + 1] first slice of each part (device)
   int2* sl_srow = nullptr;           // [sl_slices] first row, part << 6 | rows (n_parts > 1)
   uint2* sl_desc = nullptr;  // [sl_slices + 1]
@@ -431,7 +432,11 @@ inline int grid_for(const rp_handle* h, int64_t n) {
 rp_status ensure_solver_buffers(rp_handle* h);
 rp_status build_sliced(rp_handle* h, cudaStream_t s);  // after the CSR map
 rp_status fill_sliced_transposed(rp_handle* h, cudaStream_t s);  // sl_valsT from valsT
-rp_status fill_sliced(rp_handle* h, const double* buf, cudaStream_t s);  // the value update of a sliced handle
+// the value update of a sliced handle: all values from the buffer in one pass, or the
+// sliced values from the CSR ones (and s64) after a permutation
+bool fill_one_pass(const rp_handle* h);
+rp_status fill_sliced(rp_handle* h, const double* buf, cudaStream_t s);
+rp_status gather_sliced(rp_handle* h, cudaStream_t s);
 // the scaled inner system of the mixed PCG solves: allocated and filled from the
 // current values on first use (then refilled by fill_sliced); false when the
 // handle does not take it (several parts, CSR layout, no FP32 copy)

@@ -115,7 +115,9 @@ __device__ int slice_table(const int32_t* __restrict__ row_ptr, const int32_t* _
 }
 
 // pass 1: width L_s and table length D_s of every slice; err bit 1: a
-// row longer than kSliceMaxWidth, bit 2: a table longer than kSliceMaxDict
+// row longer than kSliceMaxWidth, bit 2: a table longer than kSliceMaxDict;
+// err[1]: slices of more than kRun entries, err[2]: the most entries of a slice
+constexpr int kRun = 8 * kSliceRows;
 __global__ void __launch_bounds__(kThreads)
     k_slice_count(SlParts q, int64_t S, uint8_t* __restrict__ width, uint16_t* __restrict__ tlen, int32_t* err) {
   __shared__ int32_t sdict[kWarpsPerBlock][kSliceMaxDict];
@@ -134,9 +136,14 @@ __global__ void __launch_bounds__(kThreads)
       if (lane == 0) atomicOr(err, 2);
       continue;
     }
+    const int run = __reduce_add_sync(0xffffffffu, len);
     if (lane == 0) {
       width[s] = (uint8_t)L;
       tlen[s] = (uint16_t)D;
+      if (run > kRun) {
+        atomicAdd(err + 1, 1);
+        atomicMax(err + 2, run);
+      }
     }
   }
 }
@@ -204,9 +211,10 @@ __global__ void __launch_bounds__(kThreads)
 }
 
 // sliced values from the CSR values: v[q] = vals[pos[q]], 0 for padding
+template <bool FP32>
 __global__ void __launch_bounds__(kThreads)
     k_slice_vals(int64_t nq4, const int4* __restrict__ pos, const double* __restrict__ vals,
-                 double2* __restrict__ out, int64_t nnz) {
+                 double2* __restrict__ out, float4* __restrict__ out32, int64_t nnz) {
   // a CSR position, or -1 for padding (bounds-checked build: anything else reads 0)
   auto at = [&](int32_t q) { return q >= 0 && RP_IN(q, 0, nnz, kChkSliceValues) ? __ldg(vals + q) : 0.0; };
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nq4; i += (int64_t)gridDim.x * blockDim.x) {
@@ -214,6 +222,7 @@ __global__ void __launch_bounds__(kThreads)
     const double a = at(p.x), b = at(p.y), c = at(p.z), d = at(p.w);
     __stcs(out + 2 * i, make_double2(a, b));
     __stcs(out + 2 * i + 1, make_double2(c, d));
+    if (FP32) __stcs(out32 + i, make_float4(f32_rn(a), f32_rn(b), f32_rn(c), f32_rn(d)));
   }
 }
 
@@ -305,13 +314,13 @@ __device__ __forceinline__ void cp_async8(void* dst, const void* src) {
 // values, the slice and the diagonal's reciprocals from there. (A permutation to CSR,
 // a gather from CSR to the slices and a third pass for S A S moved 60 bytes an entry
 // where this moves 40.) Runs of more than kRun entries (rows longer than 8 on average)
-// are gathered straight from the buffer; rows of more than 8 entries and 8-bit
+// are gathered straight from the buffer, one entry after another: handles with more
+// than a few take two passes (fill_one_pass). Rows of more than 8 entries and 8-bit
 // indices take the general loop. Plain stores: streaming ones (evict first) cost 2%,
 // the runs' ends share sectors. 256^3 with S A S: 1.21 ms an update, 0.19 ms of it the
 // diagonal pass, 4.7 GB at 0.7 of the copy rate (bound by issue and the mix of nine
 // streams read and written; two separate gathers took 2.30 ms, one without the copies
 // ahead 1.28 ms).
-constexpr int kRun = 8 * kSliceRows;
 constexpr int kFillSmem = kWarpsPerBlock * kRun * 2 * (8 + 4);  // 48 KB, no more than a launch may ask for by default
 static_assert(kFillSmem <= 48 * 1024, "opt in");
 template <bool FP32, bool SCALED>
@@ -523,19 +532,19 @@ rp_status build_sliced(rp_handle* h, cudaStream_t st) {
   int32_t* err;
   RP_TRY(tmp.alloc(&width, S));
   RP_TRY(tmp.alloc(&tlen, S));
-  RP_TRY(tmp.alloc(&err, 1));
-  RP_TRY_CUDA(cudaMemsetAsync(err, 0, 4, st));
+  RP_TRY(tmp.alloc(&err, 3));
+  RP_TRY_CUDA(cudaMemsetAsync(err, 0, 12, st));
   const int g = slice_grid(h, S);
   k_slice_count<<<g, kThreads, 0, st>>>(q, S, width, tlen, err);
   RP_TRY_CUDA(cudaGetLastError());
   std::vector<uint8_t> hw(S);
   std::vector<uint16_t> ht(S);
-  int32_t herr = 0;
+  int32_t counted[3] = {0, 0, 0}, herr = 0;
   RP_TRY_CUDA(cudaMemcpyAsync(hw.data(), width, S, cudaMemcpyDeviceToHost, st));
   RP_TRY_CUDA(cudaMemcpyAsync(ht.data(), tlen, 2 * S, cudaMemcpyDeviceToHost, st));
-  RP_TRY_CUDA(cudaMemcpyAsync(&herr, err, 4, cudaMemcpyDeviceToHost, st));
+  RP_TRY_CUDA(cudaMemcpyAsync(counted, err, 12, cudaMemcpyDeviceToHost, st));
   RP_TRY_CUDA(cudaStreamSynchronize(st));
-  if (herr) return RP_OK;  // a row or a slice does not fit: CSR iteration
+  if (counted[0]) return RP_OK;  // a row or a slice does not fit: CSR iteration
 
   // every slice's table into one scratch array, then distinct tables kept once
   std::vector<int64_t> toff(S + 1, 0);
@@ -634,6 +643,13 @@ rp_status build_sliced(rp_handle* h, cudaStream_t st) {
   if (herr) return undo(fail(RP_ECUDA, "sliced layout: slice sizes differ between passes"));
   h->sl_slices = S;
   h->sl_u4 = u4 ? 1 : 0;
+  // lines of fill_one_pass, from both ways' times (1M rows; slices of long rows among
+  // rows of 7; one pass, two, us): rows of 11 in 0 of 32 slices 50, 66, in 4 63, 72, in 6 78,
+  // 75, in all 146, 102; rows of 21 in 1 79, 72, in 4 87, 83, in all 291, 182; with S A S
+  // rows of 11 in 8 110, 148, in 16 147, 164, in all 199, 189; rows of 21 in 8 163, 183, in
+  // 16 244, 238
+  h->sl_one_pass = counted[1] == 0 || ((int64_t)counted[1] * 8 <= S && counted[2] <= 3 * kRun / 2);
+  h->sl_one_pass_scaled = (int64_t)counted[1] * 4 <= S;
   h->sl_width = *std::max_element(hw.begin(), hw.end());
   h->sl_entries = (int64_t)x;
   h->sl_ibuf_len = (int64_t)y;
@@ -691,9 +707,8 @@ __global__ void __launch_bounds__(kThreads)
   }
 }
 
-// the values of S A S from the current ones, for the first mixed solve
+// the values of S A S from the sliced ones and s64
 static rp_status fill_scaled(rp_handle* h, cudaStream_t s) {
-  k_scaling<<<grid_for(h, h->n), kThreads, 0, s>>>(h->n, h->diag_pos, h->vals, h->nnz, h->s64, h->s2);
   k_slice_vals_scaled<<<grid_for(h, h->sl_slices * kSliceRows), kThreads, 0, s>>>(
       h->sl_slices, h->sl_desc, h->sl_tinfo, h->sl_tabs, reinterpret_cast<const uint32_t*>(h->sl_ibuf), h->sl_vals,
       h->s64, h->n, h->sl_vals32s);
@@ -707,6 +722,7 @@ rp_status ensure_scaled(rp_handle* h, cudaStream_t s, bool* ok) {
   if (!h->s64) RP_TRY(salloc(&h->s64, h->n + 64));
   if (!h->s2) RP_TRY(salloc(&h->s2, h->n + 64));
   RP_TRY(salloc(&h->sl_vals32s, h->sl_entries));
+  k_scaling<<<grid_for(h, h->n), kThreads, 0, s>>>(h->n, h->diag_pos, h->vals, h->nnz, h->s64, h->s2);
   return fill_scaled(h, s);
 }
 
@@ -727,6 +743,25 @@ rp_status fill_sliced(rp_handle* h, const double* buf, cudaStream_t s) {
   return RP_OK;
 }
 
+bool fill_one_pass(const rp_handle* h) {
+  return h->sl_slices > 0 && (h->sl_vals32s ? h->sl_one_pass_scaled : h->sl_one_pass);
+}
+
+// The second of two passes: k_slice_vals over 1M rows of 9.4, 14.7 and 20.4 entries makes
+// an update of 98, 154 and 210 us, where one pass takes 137, 225 and 324.
+rp_status gather_sliced(rp_handle* h, cudaStream_t s) {
+  const int64_t nq4 = h->sl_entries / 4;  // a multiple of 32 entries
+  const int g = grid_for(h, nq4);
+  const int4* pos = reinterpret_cast<const int4*>(h->sl_pos);
+  double2* out = reinterpret_cast<double2*>(h->sl_vals);
+  if (h->sl_vals32)
+    k_slice_vals<true><<<g, kThreads, 0, s>>>(nq4, pos, h->vals, out, reinterpret_cast<float4*>(h->sl_vals32), h->nnz);
+  else
+    k_slice_vals<false><<<g, kThreads, 0, s>>>(nq4, pos, h->vals, out, nullptr, h->nnz);
+  RP_TRY_CUDA(cudaGetLastError());
+  return h->sl_vals32s ? fill_scaled(h, s) : RP_OK;
+}
+
 // The transposed matrix of a structurally symmetric pattern (every entry has
 // its transposed position) has the same slices: entry q of the layout takes
 // valsT at the same CSR position.
@@ -734,8 +769,8 @@ rp_status fill_sliced_transposed(rp_handle* h, cudaStream_t s) {
   if (h->sl_slices == 0 || !h->valsT) return RP_OK;
   if (!h->sl_valsT) RP_TRY(salloc(&h->sl_valsT, h->sl_entries));
   const int64_t nq4 = h->sl_entries / 4;
-  k_slice_vals<<<grid_for(h, nq4), kThreads, 0, s>>>(nq4, reinterpret_cast<const int4*>(h->sl_pos), h->valsT,
-                                                     reinterpret_cast<double2*>(h->sl_valsT), h->nnz);
+  k_slice_vals<false><<<grid_for(h, nq4), kThreads, 0, s>>>(nq4, reinterpret_cast<const int4*>(h->sl_pos), h->valsT,
+                                                            reinterpret_cast<double2*>(h->sl_valsT), nullptr, h->nnz);
   RP_TRY_CUDA(cudaGetLastError());
   return RP_OK;
 }

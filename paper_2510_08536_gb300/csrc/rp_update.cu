@@ -88,13 +88,14 @@ __global__ void __launch_bounds__(kThreads)
 }
 
 static rp_status permute_all(rp_handle* h, const double* buf, cudaStream_t s) {
+  const bool one_pass = fill_one_pass(h);
   const int gd = grid_for(h, h->n);
   if (h->n > 0 && h->sl_vals32s)
     k_diagonal<false><<<gd, kThreads, 0, s>>>(buf, h->d_row_off, h->d_slot_off, h->k, h->n, walk_trips(h, h->n), nullptr, nullptr, h->s64, h->s2);
-  if (h->n > 0 && h->sl_slices == 0)
+  if (h->n > 0 && !one_pass)
     k_diagonal<true><<<gd, kThreads, 0, s>>>(buf, h->d_row_off, h->d_slot_off, h->k, h->n, walk_trips(h, h->n), h->dinv,
                                              h->want_fp32 ? h->dinv32 : nullptr, nullptr, nullptr);
-  if (h->sl_slices > 0) {
+  if (one_pass) {
     RP_TRY(fill_sliced(h, buf, s));
   } else {
     for (int p = 0; p < h->n_parts; ++p) {
@@ -108,6 +109,7 @@ static rp_status permute_all(rp_handle* h, const double* buf, cudaStream_t s) {
       else
         k_permute<false><<<g, kThreads, 0, s>>>(base, h->src_of + o, h->vals + o, nullptr, cnt, blen);
     }
+    if (h->sl_slices > 0) RP_TRY(gather_sliced(h, s));
   }
   if (h->nl_nnz > 0) {
     const int g = grid_for(h, h->nl_nnz), alpha = h->k / h->n_parts;
