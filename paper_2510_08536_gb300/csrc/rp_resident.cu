@@ -299,11 +299,12 @@ ResidentPlan resident_plan(const rp_handle* h, const IterArgs<T>& a, bool scaled
     if (f.id == kKept) return kept_fn<T, false>(lay, scaled);
     return f.id == kKeptFold ? kept_fn<T, true>(lay, scaled) : streamed_fn<T, true>(lay, scaled);
   };
+  constexpr int64_t kL2 = 80'000'000;
   constexpr ResidentForm kFold{4, true, kFoldRows<T>, kKeptFold, RP_FORM_RESIDENT_FOLDED};
   constexpr ResidentForm kMat{4, true, INT32_MAX, kKept, RP_FORM_RESIDENT_MATRIX};
   constexpr ResidentForm kFour{4, false, INT32_MAX, kStream4}, kTwo{2, false, INT32_MAX, kStream2};
-  if constexpr (sizeof(T) == 8) return plan_resident<T>(h, a.sl, a.n, {kFold, kMat, kFour, kTwo}, fn);
-  else return plan_resident<T>(h, a.sl, a.n, {kFold, kMat, kFour}, fn);
+  if constexpr (sizeof(T) == 8) return plan_resident<T>(h, a.sl, a.n, kL2, {kFold, kMat, kFour, kTwo}, fn);
+  else return plan_resident<T>(h, a.sl, a.n, kL2, {kFold, kMat, kFour}, fn);
 }
 template ResidentPlan resident_plan<double>(const rp_handle*, const IterArgs<double>&, bool);
 template ResidentPlan resident_plan<float>(const rp_handle*, const IterArgs<float>&, bool);

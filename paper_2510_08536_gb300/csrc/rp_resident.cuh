@@ -559,10 +559,35 @@ inline cudaError_t launch_resident(const rp_handle* h, const ResidentPlan& p, vo
   void* args[1] = {argp};
   return cudaLaunchCooperativeKernel(p.fn, dim3((unsigned)p.grid), dim3((unsigned)p.threads), args, (size_t)p.smem, s);
 }
+// How large a system in another layout than the uniform one may be. The streaming
+// products hide the latency of its loads behind twice the warps, so the resident
+// form loses where those loads miss. (us an iteration there, then here; 5 to 20
+// entries a row.)
+//
+// Sliced, FP32: at most `l2` bytes of values, indices and tables; beyond, they miss L2
+// (PCG: 76 MB 72.0, 53.8 and 69.2, 56.2; 81 MB 75.3, 75.0; 100 MB 95.5, 122.2; 131 MB
+// 114, 141; BiCGStab: 74 MB 162, 98; 76 MB 147, 161 and 159, 152; 81 MB 167, 172). FP64
+// stays ahead (480 MB: 479, 459), save with r and q alone on chip and tables that slices
+// do not share (a mesh numbered at random, 33 MB of them: 131, 140).
+//
+// CSR: threads read their rows piece by piece, and shared memory has to leave L1 a part
+// of what the rows of all threads take, here per form and for several parts.
+//   FP64, four vectors: 0.22 152, 341; 0.48 79, 83; 0.72 100, 77; 0.80 57, 48; parts 0.81
+//     64, 69; 1.19 55, 44 (BiCGStab 0.48 155, 171; 0.80 115, 104; parts 0.81 126, 147)
+//   FP64, two: 0.50 218, 260; 0.96 88, 102; 1.09 108, 93; parts 1.25 90, 97; 1.53 81, 80
+//   FP32: 0.28 178, 426; 0.72 56.6, 59.8; 0.85 122, 109; 1.03 54.6, 55.5 (BiCGStab 119,
+//     108); parts 1.24 60, 81; 1.61 57.0, 57.7; 1.97 52, 47
+constexpr int64_t kOwnTables = 16 * 1024 * 1024;  // more bytes of tables: slices do not share them
+constexpr int64_t kL1Bytes = 256 * 1024;          // L1 and shared memory of an SM
+constexpr double csr_share(bool fp64, int vecs, bool parts) {
+  if (parts) return fp64 && vecs == 4 ? 0.9 : 1.5;
+  return !fp64 ? 0.8 : vecs == 4 ? 0.6 : 1.0;
+}
+
 // fn_of(layout, form): the instance, or nullptr where there is none
 template <typename T, typename Fn>
-ResidentPlan plan_resident(const rp_handle* h, const Sliced<T>& sl, int64_t n, std::initializer_list<ResidentForm> forms,
-                           Fn&& fn_of) {
+ResidentPlan plan_resident(const rp_handle* h, const Sliced<T>& sl, int64_t n, int64_t l2,
+                           std::initializer_list<ResidentForm> forms, Fn&& fn_of) {
   ResidentPlan p;
   int coop = 0, smem_max = 0;
   if (n == 0 || h->opts.spin_limit < kResidentSpin) return p;
@@ -580,13 +605,20 @@ ResidentPlan plan_resident(const rp_handle* h, const Sliced<T>& sl, int64_t n, s
   const int64_t S = lay == kRsCsr ? (n + 31) / 32 : sl.n_slices;
   const int grid = (int)std::min<int64_t>(h->num_sms, S);
   const int64_t per = (S + grid - 1) / grid;  // slices a block at most
+  const bool general = lay == kRsSliced || lay == kRsParts;
+  const int64_t tables = 4 * sl.tabs_len;
+  if (general && sizeof(T) == 4 && 4 * sl.n_entries + 4 * sl.ibuf_len + tables > l2) return p;
+  const double row_bytes = (double)(h->nnz + h->nl_nnz) * (sizeof(T) + 4.0) / (double)n;
   for (const ResidentForm& f : forms) {
-    if ((f.mat && !u4) || per * 32 > f.max_rows) continue;
+    if ((f.mat && !u4) || per * 32 > f.max_rows || (general && f.vecs < 4 && tables > kOwnTables)) continue;
     void* fn = fn_of(lay, f);
     if (!fn) continue;
     const int64_t need =
         per * 32 * f.vecs * (int64_t)sizeof(T) + RsMatrix<T, kRsCsr>::tail_bytes(lay, per, f.mat, h->sl_width);
     const int threads = 32 * (int)std::min<int64_t>(std::max<int64_t>(per, 4), (f.mat ? kRsThreads<T, true> : kRsThreads<T, false>) / 32);
+    if (lay == kRsCsr &&
+        (double)(kL1Bytes - need) < csr_share(sizeof(T) == 8, f.vecs, h->n_parts > 1) * threads * row_bytes)
+      continue;
     cudaFuncAttributes at;
     int nb = 0;
     // the kernel's own (static) shared memory comes off the block's limit

@@ -282,7 +282,7 @@ RP_CHECK_TU(resident_bs)
 
 template <typename T>
 ResidentPlan resident_bs_plan(const rp_handle* h, const BsVecs<T>& v) {
-  return plan_resident<T>(h, v.sl, h->n, {{4, false, INT32_MAX, 0}}, [](int lay, const ResidentForm&) -> void* {
+  return plan_resident<T>(h, v.sl, h->n, 75'000'000, {{4, false, INT32_MAX, 0}}, [](int lay, const ResidentForm&) -> void* {
     switch (lay) {
       case kRsU4: return (void*)k_resident_bs<T, kRsU4>;
       case kRsSliced: return (void*)k_resident_bs<T, kRsSliced>;
