@@ -424,8 +424,9 @@ rp_status rp_batch_update_solve(rp_handle* h, const double* buffer, int32_t wher
 rp_status rp_batch_set_config(rp_handle* h, int32_t cluster, int32_t threads);
 
 /* Autotuner: times rp_batch_update_solve (device buffer, precision) for every
- * cluster size in {2, 3, 4, 5, 6, 8, 16} and CTA size in {256, 512}, keeps
- * the fastest shape in the handle and reports it. Overwrites x. Blocks. */
+ * cluster size in {2, 3, 4, 5, 6, 8, 16} and CTA size in {256, 512} and for
+ * the shape that the handle has, keeps the fastest one in the handle and
+ * reports it. Overwrites x. Blocks. */
 rp_status rp_batch_autotune(rp_handle* h, const double* buffer, const double* b, double* x, double tol,
                             int32_t precision, int32_t* best_cluster, int32_t* best_threads, float* best_ms,
                             void* stream);

@@ -1043,30 +1043,31 @@ extern "C" rp_status rp_batch_autotune(rp_handle* h, const double* buffer, const
   // team counts between these shapes matter: with the largest systems first,
   // too many small teams leave the largest system's team running alone at
   // the end, too few large teams pay more barrier latency per iteration
-  const int clusters[] = {2, 3, 4, 5, 6, 8, 16};
-  const int threads[] = {256, 512};
+  std::vector<std::pair<int, int>> shapes{{h->batch_cluster, h->batch_threads}};  // never to leave a slower one
+  for (int c : {2, 3, 4, 5, 6, 8, 16})
+    for (int t : {256, 512})
+      if (std::make_pair(c, t) != shapes[0]) shapes.emplace_back(c, t);
   cudaEvent_t e0, e1;
   RP_TRY_CUDA(cudaEventCreate(&e0));
   RP_TRY_CUDA(cudaEventCreate(&e1));
   float best = 1e30f;
   int bc = h->batch_cluster, bt = h->batch_threads;
-  for (int c : clusters)
-    for (int t : threads) {
-      if (rp_batch_set_config(h, c, t) != RP_OK) continue;
-      // one untimed run (graph build, warm caches), then one timed run
-      if (batch_run(h, buffer, RP_MEM_DEVICE, b, x, tol, precision, nullptr, s) != RP_OK) continue;
-      cudaEventRecord(e0, s);
-      if (batch_run(h, buffer, RP_MEM_DEVICE, b, x, tol, precision, nullptr, s) != RP_OK) continue;
-      cudaEventRecord(e1, s);
-      if (cudaEventSynchronize(e1) != cudaSuccess) continue;
-      float ms = 0.f;
-      cudaEventElapsedTime(&ms, e0, e1);
-      if (ms < best) {
-        best = ms;
-        bc = c;
-        bt = t;
-      }
+  for (const auto& [c, t] : shapes) {
+    if (rp_batch_set_config(h, c, t) != RP_OK) continue;
+    // one untimed run (graph build, warm caches), then one timed run
+    if (batch_run(h, buffer, RP_MEM_DEVICE, b, x, tol, precision, nullptr, s) != RP_OK) continue;
+    cudaEventRecord(e0, s);
+    if (batch_run(h, buffer, RP_MEM_DEVICE, b, x, tol, precision, nullptr, s) != RP_OK) continue;
+    cudaEventRecord(e1, s);
+    if (cudaEventSynchronize(e1) != cudaSuccess) continue;
+    float ms = 0.f;
+    cudaEventElapsedTime(&ms, e0, e1);
+    if (ms < best) {
+      best = ms;
+      bc = c;
+      bt = t;
     }
+  }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   RP_TRY(rp_batch_set_config(h, bc, bt));
