@@ -826,13 +826,31 @@ rp_status build_batch_graph(rp_handle* h, int mode, int cluster, int threads, cu
   return RP_OK;
 }
 
+// Teams of c CTAs that run at once whatever precision is asked for (0: one of the
+// kernels cannot be scheduled so).
+int teams_of(rp_handle* h, int c) {
+  int least = 0;
+  for (int mode = 0; mode < (h->want_fp32 ? 3 : 1); ++mode) {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr;
+    int nc = 0;
+    if (launch_config(h, mode, c, h->batch_threads, &cfg, &attr, &nc) != RP_OK) {
+      cudaGetLastError();
+      return 0;
+    }
+    least = mode == 0 ? nc : std::min(least, nc);
+  }
+  return least;
+}
+
 // The team size of a batch whose caller sets none. A system of n rows takes about
 // n^(1/3) iterations of 5000 + n / c rows' time on a team of c CTAs (the constant:
-// the barriers and sums of an iteration; fitted, within 10% of all the times below),
-// and the queue hands the largest systems out first, so the step ends with the last
-// team of that schedule. Few systems leave most SMs idle behind the largest one on
-// small teams; many, on large teams, pay the constant too often. ms a step
-// (continued refinement) with teams of 5, 8, 10, 12, 16 -- all batches took 5:
+// the barriers and sums of an iteration; fitted to continued refinement, within 10% of
+// all the times below; FP64 and restarted refinement with the size it gives take 0.4 to
+// 0.98 of their times with 5 on these batches and smaller ones), and the queue hands
+// the largest systems out first, so the step ends with the last team of that schedule.
+// Few systems leave most SMs idle behind the largest one on small teams; many, on large
+// teams, pay the constant too often. ms a step (continued refinement) with teams of 5, 8, 10, 12, 16 -- all batches took 5:
 //   48 systems of 8k-300k rows  125.5  84.6  67.4  59.1  66.9  (12 taken)
 //   48 of 1k-40k                 12.6  10.6   9.1  10.4  15.9  (10)
 //   32 of 4k-300k               114.7  79.2  64.1  52.5  43.9  (16)
@@ -845,13 +863,8 @@ int team_size(rp_handle* h) {
   int best = h->batch_cluster;
   double least = 0.0;
   for (int c : {4, 5, 6, 8, 10, 12, 16}) {
-    cudaLaunchConfig_t cfg;
-    cudaLaunchAttribute attr;
-    int nc = 0;
-    if (launch_config(h, 0, c, h->batch_threads, &cfg, &attr, &nc) != RP_OK) {
-      cudaGetLastError();
-      continue;
-    }
+    const int nc = teams_of(h, c);
+    if (nc == 0) continue;
     std::priority_queue<double, std::vector<double>, std::greater<double>> team(std::greater<double>(),
                                                                                 std::vector<double>(nc, 0.0));
     double end = 0.0;
