@@ -1,5 +1,5 @@
 // Building blocks of the resident solver kernels (rp_resident.cu: PCG,
-// rp_bicgstab.cu: BiCGStab): one block an SM owns a contiguous run of 32-row
+// rp_resident_bs.cu: BiCGStab): one block an SM owns a contiguous run of 32-row
 // slices, a warp takes every nw-th of them in the products and 16-byte groups of
 // rows in the passes over vectors, and the grid meets at an arrival counter.
 #pragma once
@@ -263,16 +263,21 @@ struct RsFold {
 };
 
 // The products of a row of the uniform layout in entry order: x seen from the row, L
-// entries, their values val(e), index word wd, table entry tv.
+// entries, their values val(e), index word wd, table entry tv of D (D and ck: what the
+// checked build tests).
 // (Taking the block's own rows from shared memory instead, under a predicate a lane,
 // lost 4 to 20%: the products are bound by their instructions, and rank boundaries
 // leave a far column in nearly every slice.)
 template <typename T, class G, class Val>
-__device__ __forceinline__ T rs_products(const G& x, bool valid, uint32_t wd, int32_t tv, int L, Val&& val) {
+__device__ __forceinline__ T rs_products(const G& x, bool valid, uint32_t wd, int32_t tv, int L, int D, const SliceCk& ck,
+                                         Val&& val) {
   T g[8], s = T(0);
   if (L == 7 && __all_sync(0xffffffffu, valid)) {  // most slices: without a test an entry
 #pragma unroll
-    for (int e = 0; e < 7; ++e) g[e] = x(slice_offset<kIdx4>(wd, e, tv, nullptr, 0));
+    for (int e = 0; e < 7; ++e) {
+      const int off = slice_offset<kIdx4>(wd, e, tv, nullptr, 0);
+      g[e] = slice_ok<kIdx4>(wd, e, off, D, ck) ? x(off) : T(0);
+    }
 #pragma unroll
     for (int e = 0; e < 7; ++e) s = fma(val(e), g[e], s);
     return s;
@@ -281,7 +286,7 @@ __device__ __forceinline__ T rs_products(const G& x, bool valid, uint32_t wd, in
   for (int e = 0; e < 8; ++e)
     if (e < L) {
       const int off = slice_offset<kIdx4>(wd, e, tv, nullptr, 0);
-      g[e] = valid ? x(off) : T(0);
+      g[e] = valid && slice_ok<kIdx4>(wd, e, off, D, ck) ? x(off) : T(0);
     }
 #pragma unroll
   for (int e = 0; e < 8; ++e)
@@ -298,8 +303,8 @@ struct RsSlice {
   uint32_t wd;
   int32_t tv;
   int L;
-  __device__ __forceinline__ void load(const Sliced<T>& sl, uint32_t x0, uint32_t x1, uint32_t y0, uint32_t tab, int lane) {
-    L = (int)((x1 - x0) >> 5);
+  __device__ __forceinline__ void load(const Sliced<T>& sl, uint32_t x0, int len, uint32_t y0, uint32_t tab, int lane) {
+    L = len;
     const T* p = sl.vals + x0 + lane;
     wd = ldg_stream(reinterpret_cast<const uint32_t*>(sl.ibuf) + y0 + lane);
     tv = __ldg(sl.tabs + tab + (lane & 15));
@@ -422,10 +427,13 @@ struct RsMatrix {
     if constexpr (MAT) {
       const uint32_t x0 = sx[0], m = sx[cnt] - x0;
       T* q = const_cast<T*>(mv);
-      for (uint32_t e = threadIdx.x; e < m; e += blockDim.x) q[e] = ldg_stream(sl.vals + x0 + e);
+      for (uint32_t e = threadIdx.x; e < m; e += blockDim.x)
+        if (RP_IN(x0 + e, 0, sl.n_entries, kChkSliceCopy) && RP_IN(e, 0, per * kSliceRows * width, kChkSliceCopy))
+          q[e] = ldg_stream(sl.vals + x0 + e);
       uint32_t* iw = const_cast<uint32_t*>(mw);
       for (int e = threadIdx.x; e < cnt * kSliceRows; e += blockDim.x)
-        iw[e] = ldg_stream(reinterpret_cast<const uint32_t*>(sl.ibuf) + (size_t)kSliceRows * s0 + e);
+        if (RP_IN(kSliceRows * s0 + e, 0, sl.ibuf_len, kChkSliceCopy))
+          iw[e] = ldg_stream(reinterpret_cast<const uint32_t*>(sl.ibuf) + (size_t)kSliceRows * s0 + e);
       __syncthreads();
     } else if (U4 && w < cnt) {
       fetch(w);
@@ -459,12 +467,33 @@ struct RsMatrix {
       if (m > 0) f(k, i, m, W == 1 || (!MP && m == W));
     }
   }
+  // entries a row of slice j of the uniform layout (checked build: 0 where its
+  // descriptor, index words or table reference leave their arrays)
+  __device__ __forceinline__ int slice_len(int j) const {
+    const uint32_t x0 = sx[j], x1 = sx[j + 1];
+#ifdef RP_CHECK
+    if (!RP_IN(x1, x0, sl.n_entries + 1, kChkSliceDesc) || !RP_IN(x1 - x0, kSliceRows, 8 * kSliceRows + 1, kChkSliceDesc) ||
+        !RP_IN((int64_t)kSliceRows * (s0 + j + 1), 0, sl.ibuf_len + 1, kChkSliceDesc) ||
+        !RP_IN(sinfo[j], 1, sl.tabs_len - 32 + 1, kChkSliceDesc))
+      return 0;
+#endif
+    return (int)((x1 - x0) >> 5);
+  }
+  // length of its table (checked build)
+  __device__ __forceinline__ int table_len(int j, int L) const {
+#ifdef RP_CHECK
+    return L > 0 ? __ldg(sl.tabs + sinfo[j] - 1) : 0;
+#else
+    (void)j, (void)L;
+    return 0;
+#endif
+  }
   __device__ __forceinline__ NlRange nl_range(int j) const {
     const int i = row_of(j);
     return i >= 0 ? nonlocal_range<T>(parts, srow[j].y >> 6, i) : NlRange{0, 0};
   }
   __device__ __forceinline__ void fetch(int j) {
-    f.load(sl, sx[j], sx[j + 1], (uint32_t)(kSliceRows * (s0 + j)), sinfo[j], lane);
+    f.load(sl, sx[j], slice_len(j), (uint32_t)(kSliceRows * (s0 + j)), sinfo[j], lane);
     if (MP) fnl = nl_range(j);
   }
   // slice j's product with x; i: row_of(j)
@@ -474,24 +503,28 @@ struct RsMatrix {
     T sum = T(0);
     if constexpr (U4) {
       const G xr = x.at(valid ? i : 0);
+      const int part_id = MP ? srow[j].y >> 6 : 0;
+      const SliceCk ck = slice_ck<T, MP>(sl, parts, part_id, valid ? i : 0, n);
       NlRange nl{0, 0};
       if (MP) nl = MAT ? nl_range(j) : fnl;
-      // the first non-local entry (most rows that have any have one) under way with the gathers
       if constexpr (MAT) {
-        const uint32_t x0 = sx[j];
-        const T* v = mv + (x0 - sx[0]) + lane;
+        const int L = slice_len(j);
+        const T* v = mv + (sx[j] - sx[0]) + lane;
         const int32_t tv = __ldg(sl.tabs + sinfo[j] + (lane & 15));
-        sum = rs_products<T>(xr, valid, mw[j * kSliceRows + lane], tv, (int)((sx[j + 1] - x0) >> 5),
+        sum = rs_products<T>(xr, valid, mw[j * kSliceRows + lane], tv, L, table_len(j, L), ck,
                              [&](int e) { return v[kSliceRows * e]; });
       } else {
         const RsSlice<T> cur = f;
         fetch(j + nw < cnt ? j + nw : w);  // the last one fetches the first of the next product
-        sum = rs_products<T>(xr, valid, cur.wd, cur.tv, cur.L, [&](int e) { return cur.v[e]; });
+        sum = rs_products<T>(xr, valid, cur.wd, cur.tv, cur.L, table_len(j, cur.L), ck, [&](int e) { return cur.v[e]; });
       }
       if (MP && nl.j0 < nl.j1) {
         const int nlo = snl[j];
-        for (int e = nl.j0; e < nl.j1; ++e)
-          sum = fma(__ldg(parts.nl_vals + nlo + e), x(__ldg(parts.nl_gcol + nlo + e)), sum);
+        const int64_t nco = __ldg(parts.nlcol_off + part_id);
+        for (int e = nl.j0; e < nl.j1; ++e) {
+          const int g = nl_row_of<T>(parts, part_id, nlo, nco, e);
+          if (RP_IDX_OK(g)) sum = fma(__ldg(parts.nl_vals + nlo + e), x(g), sum);
+        }
       }
     } else if constexpr (LAY == kRsCsr) {
       if (valid) sum = row_dot_any<T, true>(parts, row_ptr, col, vals, x.x, i, n);
@@ -596,11 +629,7 @@ ResidentPlan plan_resident(const rp_handle* h, const Sliced<T>& sl, int64_t n, i
     cudaGetLastError();
     return p;
   }
-#ifdef RP_CHECK
-  const bool u4 = false;  // the checked build tests every slice
-#else
   const bool u4 = sl.u4 != 0;
-#endif
   const int lay = sl.n_slices == 0 ? kRsCsr : sl.srow ? (u4 ? kRsPartsU4 : kRsParts) : u4 ? kRsU4 : kRsSliced;
   const int64_t S = lay == kRsCsr ? (n + 31) / 32 : sl.n_slices;
   const int grid = (int)std::min<int64_t>(h->num_sms, S);

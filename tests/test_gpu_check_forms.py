@@ -3,7 +3,8 @@ launches refused (as a driver under MPS refuses them) from the solve graph and
 from the host loop, which then run the streaming kernels to the same residual;
 and grid meetings that run out (their limit set to 0: every block gives up at its
 first one), which end each solve with RP_DEVICE_TIMEOUT and leave the handle as good
-as a fresh one.
+as a fresh one; and solves of every resident form of the uniform layout, the forms
+that the normal build runs on the same systems, with no access out of range.
 
 A child process loads that library (the binding holds one library per process).
 True residuals are recomputed with the oracle's matrix; 1e-9 is what the solves
@@ -88,6 +89,31 @@ def _timeouts():
     return out
 
 
+# rows where the forms change: one slice a warp, the matrix on chip, the matrix streamed (FP64)
+FORMS = [
+    ((19, 17, 23), {}, {"fp64": "resident_folded", "mixed": "resident_folded", "mixed_ru": "resident_folded"}),
+    ((19, 17, 23), {"n_parts": 4}, {"fp64": "resident_folded", "mixed_ru": "resident_folded"}),
+    ((61, 53, 67), {}, {"fp64": "resident_matrix", "mixed": "resident_matrix"}),
+    ((61, 53, 67), {"n_parts": 2}, {"fp64": "resident_matrix", "mixed_ru": "resident_matrix"}),
+    ((83, 79, 71), {}, {"fp64": "resident", "mixed_ru": "resident_matrix"}),
+    ((83, 79, 71), {"n_parts": 2}, {"fp64": "resident", "mixed": "resident_matrix"}),
+]
+
+
+def _uniform():
+    from paper_2510_08536_gb300 import repart
+    out = {}
+    for k, (dims, kw, forms) in enumerate(FORMS):
+        s = _Systems(dims)
+        h = repart.build_repartition(s.ranks, **kw)
+        for precision in forms:
+            out[k, "pcg", precision] = s.solve(h, "pcg", precision)
+        for precision in ("fp64", "mixed"):
+            out[k, "bicgstab", precision] = s.solve(h, "bicgstab", precision)
+        h.close()
+    return out
+
+
 def _child(q, name):
     sys.path[:0] = [ROOT, HERE]
     try:
@@ -123,6 +149,12 @@ def test_grid_meetings_run_out():
             assert got is True, case
         else:
             assert got[0] == repart.RP_DEVICE_TIMEOUT and got[1] != "streaming", case
+
+
+def test_uniform_forms():
+    for (k, kind, precision), (status, residual, form) in _run("_uniform").items():
+        want = FORMS[k][2][precision] if kind == "pcg" else "resident"
+        assert status == 0 and residual <= 1e-9 and form == want, (FORMS[k][:2], kind, precision, status, residual, form)
 
 
 def test_refused_cooperative_launches():
