@@ -112,14 +112,15 @@ __device__ __forceinline__ void warp_sums(const T (&v)[NV], RsFlags& sh, int lan
 // Grid sum of NV values a thread. Warp 0 of every block receives the totals in
 // tot[] (all lanes) and calls fin(tot); then the block goes on together.
 // For sums that change little from one iteration to the next: unit[i],
-// kept over the iterations, is 2^-80 of the last total. The threads' values
+// kept over the iterations, is 2^-79 to 2^-80 of the last total. The threads' values
 // become integers in that unit (fix_digits), the warps and the block add
-// integers, and the block adds its sum, rounded to 2^-66 of the last total, to two
+// integers, and the block adds its sum, rounded to 2^-65 of the last total, to two
 // 64-bit words in L2: 40 low bits with the count of values out of range above
 // them, 48 high bits, and the count of arrivals in the top byte of both. A word
 // whose count is complete needs no fence and no second read: one exchange instead
 // of a release, an arrival, its poll, and 152 loads and their sum. Rounding: at most
-// 2^17 halves of 2^-80 and 152 halves of 2^-66 of the last total; the sum is taken
+// 155,648 halves (152 blocks of 1024 threads) of 2^-79 and 152 halves of 2^-65 of the
+// last total, together below 2^-58; the sum is taken
 // again the long way where a value reaches 2^9 of the last total, a block 2^20, or
 // the total falls below 2^-7 of it (and the first time): all blocks see the same
 // words and decide alike.
