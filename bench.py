@@ -726,8 +726,8 @@ def run_ours(args):
 
     def launches(prec, info):
         per_pass = {"fp64": 1, "mixed": 2, "mixed_ru": 3}[prec]  # residual (+ correction, + p continuation)
-        # three kernels an iteration, or the resident kernel once a pass (vectors that fit the chip)
-        inner = info["passes"] if mesh.n_cells <= 2_100_000 else 3 * info["iterations"]
+        # three kernels an iteration, or the resident kernel once a pass, as the latest solve ran
+        inner = 3 * info["iterations"] if repart.solve_form(h) == "streaming" else info["passes"]
         update = (1 if prec == "fp64" else 2) if sliced else 2  # all values (+ scaling); permutation + diagonal
         return update + 1 + inner + per_pass * info["passes"]
 
@@ -805,7 +805,7 @@ def run_ours(args):
         repart.set_solver_options(h, precond=repart.RP_PRECOND_JACOBI)
         repart.update_values_packed(h, stg_dev[0])
 
-    # kernel durations (CUDA events on the launching stream, same kernels as the graph runs)
+    # kernel durations (CUDA events on the launching stream): the streaming iteration's kernels
     kern = {}
     for prec in precs:
         if prec == "mixed_ru" and "mixed" in kern:  # the same FP32 iteration kernels

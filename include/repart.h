@@ -436,8 +436,10 @@ rp_status rp_batch_autotune(rp_handle* h, const double* buffer, const double* b,
  * iteration kernels of `precision` on the stream (outside any graph, with no
  * stopping test), each bracketed by CUDA events. ms_out[0..2] receives the
  * average duration of the SpMV kernel, the residual-update kernel and the
- * x/p-update kernel. The kernels are the ones rp_solve's graph runs. Uses the
- * handle's work vectors; blocks the host. */
+ * x/p-update kernel. They are the kernels of the streaming iteration
+ * (RP_FORM_STREAMING); a system whose vectors fit the chip is solved with the
+ * resident kernel instead (rp_get_solve_form), which has no such parts. Uses
+ * the handle's work vectors; blocks the host. */
 rp_status rp_profile_iteration(rp_handle* h, const double* b, int32_t precision, int32_t iters,
                                float* ms_out, void* stream);
 

@@ -446,7 +446,7 @@ def solve_form(h: Handle) -> str:
 
 
 def profile_iteration(h: Handle, b, precision: str = "fp64", iters: int = 20, stream=None):
-    """rp_profile_iteration: average ms of the SpMV, residual and x/p kernels."""
+    """rp_profile_iteration: average ms of the streaming iteration's SpMV, residual and x/p kernels."""
     ms = (ctypes.c_float * 3)()
     prec = PRECISIONS[precision]
     _check(load().rp_profile_iteration(h.ptr, _ptr(b), prec, int(iters), ms, _stream(stream)), "rp_profile_iteration")
