@@ -379,8 +379,9 @@ __device__ __forceinline__ void st_ef(float4* p, float4 v, uint64_t pol) {
                : "memory");
 }
 
-template <typename T, bool LINE, bool SCALED = false>
-__global__ void __launch_bounds__(kThreads) k_it_resid(IterArgs<T> a) {
+// BLOCKS: blocks an SM that the registers have to allow (0: as they come)
+template <typename T, bool LINE, bool SCALED = false, int BLOCKS = 0>
+__global__ void __launch_bounds__(kThreads, BLOCKS) k_it_resid(IterArgs<T> a) {
   Ctl* c = a.ctl;
   if (c->stop) {
     if (blockIdx.x == 0 && threadIdx.x == 0 && a.in_graph) cudaGraphSetConditional(a.inner, 0);
@@ -513,6 +514,17 @@ __global__ void __launch_bounds__(kThreads) k_it_resid(IterArgs<T> a) {
     }
     if (a.in_graph) cudaGraphSetConditional(a.inner, c->stop ? 0u : 1u);
   }
+}
+
+// K2 with the line preconditioner. FP32 takes 36 registers, seven blocks an SM; held to
+// 32 it spills one and runs eight, which pays where HBM bounds it (us, seven then eight
+// blocks: 100^3 16.9, 18.3; 128^3 22.6, 23.1; 150^3 30.7, 30.7; 170^3 41.3, 39.1; 200^3
+// 57.8, 54.5; 256^3 103.9, 96.5).
+template <typename T>
+void* line_resid(int64_t n) {
+  if constexpr (sizeof(T) == 4)
+    if (n > 4'000'000) return (void*)k_it_resid<T, true, false, kBlocksPerSm>;
+  return (void*)k_it_resid<T, true>;
 }
 
 // K3: x += alpha p; p = z + beta p (the latter only while iterating; z = D^-1 r,
@@ -932,7 +944,7 @@ SolveSet solve_set(rp_handle* h, int mode, const double* vals, const double* din
     k.rup = (void*)k_ru_p<true>;
     k.k2_64 = (void*)k_it_resid<double, true>;
     k.k3_64 = (void*)k_it_xp<double, true>;
-    k.k2_32 = (void*)k_it_resid<float, true>;
+    k.k2_32 = line_resid<float>(h->n);
     k.k3_32 = (void*)k_it_xp<float, true>;
     k.g2_64 = h->igrid64.k2l;
     k.g3_64 = h->igrid64.k3l;
@@ -1060,7 +1072,7 @@ IterGrid iter_grid(const rp_handle* h) {
   gr.k1sm = g(resident((const void*)k_it_spmv_sl_mp<T>, SlStage<T>::kSmem, kSlThreads));
   gr.k2 = g(resident((const void*)k_it_resid<T, false>));
   gr.k3 = g(resident((const void*)k_it_xp<T, false>));
-  gr.k2l = g(resident((const void*)k_it_resid<T, true>));
+  gr.k2l = g(resident(line_resid<T>(h->n)));
   gr.k3l = g(resident((const void*)k_it_xp<T, true>));
   gr.k2s = g(resident((const void*)k_it_resid<T, false, true>));
   gr.k3s = g(resident((const void*)k_it_xp<T, false, true>));

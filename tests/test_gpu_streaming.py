@@ -132,3 +132,19 @@ def test_no_probe_at_all(layout, host_loop):
                 assert e.value.status == repart.RP_DEVICE_TIMEOUT, precision
             assert repart.solve_form(h) == "streaming"
     h.close()
+
+
+def test_line_preconditioner_on_many_rows():
+    """4.1M rows: the FP32 residual kernel held to the registers of eight blocks an SM.
+    Iterations as in the line preconditioner's own tests: 1.25 of FP64's and 10."""
+    c = Case((161, 163, 157), (2, 2, 2))
+    h = repart.build_repartition(c.mesh.ranks, precond=repart.RP_PRECOND_LINE)
+    repart.update_values_packed(h, _t(c.staging))
+    its = {}
+    for precision in ("fp64", "mixed_ru"):
+        x = _zeros(c.mesh.n_cells)
+        info = repart.solve(h, _t(c.b), x, tol=1e-9, precision=precision)
+        assert info["status"] == 0 and c.true_rel_residual(x.cpu().numpy()) <= 1e-9, (precision, info)
+        its[precision] = info["iterations"]
+    assert its["mixed_ru"] <= 1.25 * its["fp64"] + 10, its
+    h.close()
