@@ -832,13 +832,15 @@ def run_ours(args):
     def gbs(bytes_, ms):
         return bytes_ / (ms * 1e-3) / 1e9
 
-    upd_bytes = 20 * nnz + 4 * nnz + 20 * n  # idx + gather + FP64 write + FP32 write; diag read + 2 writes
-    if sliced:  # sliced values: position + CSR value read, FP64 + FP32 write per padded entry
-        upd_bytes += 24 * sliced[1]
+    # CSR handles: slot, buffer value, FP64 and FP32 written per entry; diagonal read, both
+    # reciprocals written per row
+    upd_bytes = 24 * nnz + 20 * n
+    if sliced:  # one pass: the diagonal is among the entries; FP64 and FP32 written per padded entry
+        upd_bytes += 12 * sliced[1] - 8 * n
     if sliced and repart.inner_scaled(h):
-        # S A S values: FP64 sliced value read, s (FP64) at the column, FP32 write per
-        # padded entry, index words; s itself: diagonal position + value read, FP64 write per row
-        upd_bytes += (8 + 8 + 4) * sliced[1] + 4 * sliced[2] + 20 * n
+        # S A S: FP32 written per padded entry, index words; s: diagonal read, FP64 and the FP32
+        # pair written, the pair read again per row
+        upd_bytes += 4 * sliced[1] + 4 * sliced[2] + 32 * n
     k1_name = "k_it_spmv_sl" if sliced else "k_it_spmv"
     u4 = ", true" if sliced and uniform4 else ""  # the uniform-slice instance
     roof = {"bound": "hbm", "kernel": f"{k1_name}<{'double' if head == 'fp64' else 'float'}{u4}>",
