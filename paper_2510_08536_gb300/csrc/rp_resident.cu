@@ -15,7 +15,8 @@
 // are the same integers in every block (grid_sum_unit), so all blocks hold the same
 // scalars and take the same branches.
 //
-// Forms (resident_plan takes the first that fits):
+// Forms (resident_plan takes the first that fits; on layouts other than the uniform one
+// within the lines at plan_resident):
 //   matrix kept too, C folded into the next A: at most one slice a warp (117k rows
 //     in FP64, 156k in FP32); the product gathers z + beta p
 //   matrix kept: to 380k rows in FP64, 725k in FP32; its values stay off L2
@@ -30,7 +31,7 @@
 // 5400 to 6700 cycles a sum with any number of replicas polled: the polls delay the
 // writes they wait for.) The launch is cooperative, so all blocks are resident; every
 // wait is bounded by spin probes all the same and ends the solve with
-// RP_DEVICE_TIMEOUT.
+// RP_DEVICE_TIMEOUT (limits too small for a meeting never get here: kResidentSpin).
 //
 // Bound: small systems by the meetings (4000 cycles a sum, 2600 the barrier) and the
 // latency of the gathers; FP32 at 2M rows by the products' instructions; FP64 at 128^3

@@ -3,7 +3,8 @@
 // permutation P (src_of). The sparsity is never rebuilt. Where the iteration
 // runs on the sliced layout, the same pass over the buffer writes the CSR
 // values, their FP32 copies, the sliced values in both precisions and, once a
-// mixed solve has asked for them, the FP32 values of S A S.
+// mixed solve has asked for them, the FP32 values of S A S (where slices are
+// long, the sliced values are gathered from the CSR values: fill_one_pass).
 //
 // Bound: HBM, with the FP64 pipe (two lanes a clock and SM, conversions
 // included) close behind: 4 + 8 bytes read and 8 + 4 + 8 + 4 [+ 4] written an
